@@ -687,17 +687,15 @@ int tpfa_create_grid(tpfa_handle* out, int nx, int ny, int nz, const tpfa_params
     if (e == cudaSuccess) {
         if (prec == TPFA_MIXED)
             e = launch_transmissibility_f32(h->geom, h->sp, perm_dev, (float*)h->T[0], (float*)h->T[1], (float*)h->T[2],
-                                            (float*)h->T[3], (float*)h->T[4], st);
+                                            (float*)h->T[3], (float*)h->T[4], (float*)h->kperm, st);
         else
             e = launch_transmissibility_f64(h->geom, h->sp, perm_dev, (double*)h->T[0], (double*)h->T[1],
-                                            (double*)h->T[2], (double*)h->T[3], (double*)h->T[4], st);
+                                            (double*)h->T[2], (double*)h->T[3], (double*)h->T[4], (double*)h->kperm,
+                                            st);
     }
     if (e == cudaSuccess)
         e = prec == TPFA_MIXED ? launch_convert_f32(depth_dev, (float*)h->z, N, st)
                                : launch_copy_f64(depth_dev, (double*)h->z, N, st);
-    if (e == cudaSuccess)
-        e = prec == TPFA_MIXED ? launch_store_perm_f32(perm_dev, (float*)h->kperm, N, st)
-                               : launch_store_perm_f64(perm_dev, (double*)h->kperm, N, st);
     if (e == cudaSuccess) e = launch_copy_f64(poro_dev, h->phi0_d, N, st);
     if (e == cudaSuccess && h->crk)
         e = prec == TPFA_MIXED ? launch_convert_f32(poro_dev, (float*)h->phi0_r, N, st)
@@ -896,15 +894,13 @@ int set_perm(tpfa_handle h, const double* perm_dev, void* stream, bool log_k) {
     DeviceGuard dg(h->device);
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     cudaError_t e;
-    if (h->prec == TPFA_MIXED) {
+    if (h->prec == TPFA_MIXED)
         e = launch_transmissibility_f32(h->geom, h->sp, perm_dev, (float*)h->T[0], (float*)h->T[1], (float*)h->T[2],
-                                        (float*)h->T[3], (float*)h->T[4], st, log_k);
-        if (e == cudaSuccess) e = launch_store_perm_f32(perm_dev, (float*)h->kperm, h->N, st, log_k);
-    } else {
+                                        (float*)h->T[3], (float*)h->T[4], (float*)h->kperm, st, log_k);
+    else
         e = launch_transmissibility_f64(h->geom, h->sp, perm_dev, (double*)h->T[0], (double*)h->T[1],
-                                        (double*)h->T[2], (double*)h->T[3], (double*)h->T[4], st, log_k);
-        if (e == cudaSuccess) e = launch_store_perm_f64(perm_dev, (double*)h->kperm, h->N, st, log_k);
-    }
+                                        (double*)h->T[2], (double*)h->T[3], (double*)h->T[4], (double*)h->kperm, st,
+                                        log_k);
     if (e != cudaSuccess) return cuda_fail(e, "set_permeability launch");
     return TPFA_OK;
 }

@@ -83,6 +83,25 @@ __device__ __forceinline__ float narrow_rz(double x) {
     return (float)x;
 }
 
+// The two conversions above without their general branch: its conversion
+// instruction is predicated, not jumped over, and takes its time on the FP64
+// pipe even when no lane needs it.  narrow_flush: |x| < 2^128, values below
+// 2^-126 give zero.  widen_flush: finite x, subnormals give zero.
+__device__ __forceinline__ float narrow_flush(double x) {
+    const uint32_t hi = (uint32_t)__double2hiint(x);
+    const uint32_t lo = (uint32_t)__double2loint(x);
+    const uint32_t a = hi & 0x7fffffffu;
+    const uint32_t f = ((a - 0x38000000u) << 3) | (lo >> 29);
+    return __uint_as_float((hi & 0x80000000u) | (a >= 0x38100000u ? f : 0u));
+}
+__device__ __forceinline__ double widen_flush(float x) {
+    const uint32_t u = __float_as_uint(x);
+    const uint32_t a = u & 0x7fffffffu;
+    const bool n = a >= 0x00800000u;
+    const uint32_t hi = (n ? (a >> 3) + 0x38000000u : 0u) | (u & 0x80000000u);
+    return __hiloint2double((int)hi, n ? (int)(u << 29) : 0);
+}
+
 // A double as an unevaluated FP32 pair v = hi + lo (hi the truncation of v,
 // lo the exact remainder narrowed; |lo| < ulp(hi)), so differences of nearby
 // values can be formed in FP32: (hi_a - hi_b) + (lo_a - lo_b) is accurate to

@@ -28,6 +28,7 @@ __device__ __forceinline__ double two_point(double kK, double kL, double area_ov
 
 struct Geo {
     double ax, ay, az, ad;  // area / distance of x, y, z faces and of an in-plane diagonal
+    float2 px, py, pz, pd;  // twice that as FP32 pairs
 };
 
 // Permeability of cell c: the stored value, or exp of the stored natural
@@ -37,35 +38,260 @@ __device__ __forceinline__ double perm_at(const double* __restrict__ perm, long 
     return LOG ? exp(perm[c]) : perm[c];
 }
 
-template <typename Real, bool LOG>
-__global__ void k_trans(GridGeom g, Geo geo, const double* __restrict__ perm, Real* Tx, Real* Ty, Real* Tz,
-                        Real* Tpp, Real* Tmp) {
-    const long long nx = g.nx, nxy = nx * g.ny, N = nxy * g.nz;
-    for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < N;
-         c += (long long)gridDim.x * blockDim.x) {
-        const int k = (int)(c / nxy);
-        const int j = (int)((c - k * nxy) / nx);
-        const int i = (int)(c - k * nxy - j * nx);
-        // neighbour indices fall back to c itself where the link does not
-        // exist, so every address formed is inside perm
-        const double kc = perm_at<LOG>(perm, c);
-        const bool xp = i + 1 < g.nx, yp = j + 1 < g.ny, zp = k + 1 < g.nz;
-        Tx[c] = (Real)(xp ? two_point(kc, perm_at<LOG>(perm, xp ? c + 1 : c), geo.ax) : 0.0);
-        Ty[c] = (Real)(yp ? two_point(kc, perm_at<LOG>(perm, yp ? c + nx : c), geo.ay) : 0.0);
-        Tz[c] = (Real)(zp ? two_point(kc, perm_at<LOG>(perm, zp ? c + nxy : c), geo.az) : 0.0);
-        if (g.diag) {
-            const bool pp = yp && xp, mp = yp && i > 0;
-            Tpp[c] = (Real)(pp ? two_point(kc, perm_at<LOG>(perm, pp ? c + nx + 1 : c), geo.ad) : 0.0);
-            Tmp[c] = (Real)(mp ? two_point(kc, perm_at<LOG>(perm, mp ? c + nx - 1 : c), geo.ad) : 0.0);
-        }
-    }
+// ---- reciprocal permeabilities and links without the FP64 pipe
+//
+// With r = 1/k the harmonic two-point value is 2 (area/d) / (r_K + r_L), and
+// from ln k the reciprocal is one exponential, r = exp(-ln k).  The FP64
+// pipe does two operations per clock per multiprocessor, so the first form
+// of this kernel (six exponentials and five divisions per cell, all FP64)
+// took 638 us from ln k on a 128^3 grid, 33 times its memory traffic.  Here
+// a block computes r once per cell of its tile (and its one-cell halo) in
+// shared memory; on the mixed path r, the sum and the quotient are FP32
+// pairs (value = h + l, about 45 bits), which the FP32 pipe does 64 times
+// faster.  The stored FP32 value is accepted only if every number within
+// 2^-40 of the pair's value rounds to it (Ziv's rounding test); FP64 rounding
+// errors and the pair's own are far below that, so the accepted values are
+// those of the FP64 evaluation bit for bit, and the rest (about one link in
+// 10^5, and every input outside the pairs' range, zero and NaN included) are
+// evaluated by the FP64 formula.
+
+struct Pair32 {
+    float h, l;
+};
+__device__ __forceinline__ Pair32 fast_two_sum(float a, float b) {  // |a| >= |b|
+    const float h = __fadd_rn(a, b);
+    return {h, __fsub_rn(b, __fsub_rn(h, a))};
+}
+__device__ __forceinline__ Pair32 pair_mul(Pair32 a, Pair32 b) {
+    const float p = __fmul_rn(a.h, b.h);
+    float e = __fmaf_rn(a.h, b.h, -p);
+    e = __fmaf_rn(a.h, b.l, e);
+    e = __fmaf_rn(a.l, b.h, e);
+    return fast_two_sum(p, e);
+}
+__device__ __forceinline__ Pair32 pair_add(Pair32 a, Pair32 b) {
+    const float h = __fadd_rn(a.h, b.h);
+    const float t = __fsub_rn(h, a.h);
+    const float e = __fadd_rn(__fsub_rn(a.h, __fsub_rn(h, t)), __fsub_rn(b.h, t));
+    return {h, __fadd_rn(e, __fadd_rn(a.l, b.l))};
+}
+// c + t s for a constant c with |c| >= |t s|
+__device__ __forceinline__ Pair32 pair_step(float c, Pair32 t, Pair32 s) {
+    const float p = __fmul_rn(t.h, s.h);
+    float e = __fmaf_rn(t.h, s.h, -p);
+    e = __fmaf_rn(t.h, s.l, e);
+    e = __fmaf_rn(t.l, s.h, e);
+    const float h = __fadd_rn(c, p);
+    return {h, __fadd_rn(__fsub_rn(p, __fsub_rn(h, c)), e)};
+}
+__device__ __forceinline__ float rcp_approx(float x) {  // 1/x within 2^-23
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+// num / d: the quotient h of the leading parts and the remainder over d
+__device__ __forceinline__ Pair32 pair_div(Pair32 num, Pair32 d) {
+    const float q = rcp_approx(d.h);
+    const float h = __fmul_rn(num.h, q);
+    const float rem = __fmaf_rn(-h, d.l, __fadd_rn(__fmaf_rn(-h, d.h, num.h), num.l));
+    return {h, __fmul_rn(rem, q)};
+}
+// Pairs are used for magnitudes in [2^-90, 2^90]; NaN fails the test.
+__device__ __forceinline__ bool pair_range(float h) { return h >= 0x1p-90f && h <= 0x1p90f; }
+
+// The FP32 value every number within 2^-40 of v (relative) rounds to, or
+// false if there is none.
+__device__ __forceinline__ bool round_pair(Pair32 v, float& out) {
+    const float d = __fmul_rn(v.h, 0x1p-40f);
+    const float a = __fadd_rn(v.h, __fadd_rn(v.l, d)), b = __fadd_rn(v.h, __fsub_rn(v.l, d));
+    out = a;
+    return a == b && pair_range(v.h);
 }
 
-// k in the path's precision for the adjoint, from k or from ln k.
+constexpr float kNoPair = -1.f;  // h of a cell whose reciprocal has no pair
+
+// 2^(j/8), j = 0..7
+__constant__ const double kEighth[8] = {1.0,
+                                        1.0905077326652577,
+                                        1.1892071150027210,
+                                        1.2968395546510096,
+                                        1.4142135623730951,
+                                        1.5422108254079407,
+                                        1.6817928305074290,
+                                        1.8340080864093424};
+
+// exp(-x) for |x| < 60: -x = n ln2 / 8 + t, |t| < 0.0434; exp(t) by its Taylor
+// series up to t^7 / 7! (the next term is below 2^-51), the terms from t^4 on in
+// FP32 (they are below 2^-22 of the sum), the others in pairs; times 2^(n/8).
+// `eighth` holds 2^(j/8) as pairs (shared memory).
+__device__ __forceinline__ Pair32 split_pair(double v) {
+    const float h = narrow_flush(v);
+    return {h, narrow_flush(__dadd_rn(v, -widen_flush(h)))};
+}
+__device__ __forceinline__ Pair32 exp_neg_pair(double x, const float2* eighth) {
+    const float nf = rintf(__fmul_rn(narrow_flush(x), -11.541560327111708f));  // -8 / ln 2
+    const int n = (int)nf;
+    const Pair32 t = split_pair(__fma_rn(widen_flush(-nf), 0.086643397569993164, -x));  // ln 2 / 8
+    float u = __fmaf_rn(t.h, 1.f / 5040.f, 1.f / 720.f);
+    u = __fmaf_rn(t.h, u, 1.f / 120.f);
+    u = __fmaf_rn(t.h, u, 1.f / 24.f);
+    constexpr float s6 = (float)(1.0 / 6.0), s6l = (float)(1.0 / 6.0 - (double)s6);
+    Pair32 s = fast_two_sum(s6, __fmul_rn(t.h, u));
+    s.l = __fadd_rn(s.l, s6l);
+    s = pair_step(0.5f, t, s);
+    s = pair_step(1.f, t, s);
+    s = pair_step(1.f, t, s);
+    const float2 e = eighth[n & 7];
+    const Pair32 r = pair_mul(s, Pair32{e.x, e.y});
+    const float scale = __int_as_float(((n >> 3) + 127) << 23);
+    return {__fmul_rn(r.h, scale), __fmul_rn(r.l, scale)};
+}
+
+// r = 1/k of cell c as a pair, h = kNoPair where k lies outside the pairs' range.
+template <bool LOG>
+__device__ __forceinline__ Pair32 recip_pair(double v, const float2* eighth) {
+    if (LOG) {
+        if (((uint32_t)__double2hiint(v) & 0x7fffffffu) >= 0x404e0000u) return {kNoPair, 0.f};  // |v| >= 60, NaN
+        return exp_neg_pair(v, eighth);
+    }
+    const uint32_t ex = (uint32_t)__double2hiint(v) >> 20;  // sign and exponent
+    if (!(ex > 1023u - 90u && ex < 1023u + 90u)) return {kNoPair, 0.f};
+    return pair_div(Pair32{1.f, 0.f}, split_pair(v));
+}
+
+// num / s in FP64 for s inside the pairs' range: the FP32 reciprocal refined to
+// y = 1/s by y (1 + e + e^2), e = 1 - s y (the third-order iteration for the
+// reciprocal; e is below 2^-22), then the quotient with its remainder folded
+// in once, which rounds it correctly (Markstein's final step).
+__device__ __forceinline__ double quotient(double num, double s) {
+    const double y0 = widen_flush(rcp_approx(narrow_flush(s)));
+    const double e = __fma_rn(-s, y0, 1.0);
+    const double y = __fma_rn(y0, __fma_rn(e, e, e), y0);
+    const double q = __dmul_rn(num, y);
+    return __fma_rn(__fma_rn(-s, q, num), y, q);
+}
+
+// What a tile holds per cell: 1/k as a pair (mixed path) or k (FP64 path).
+template <typename Real>
+struct Tile;
+template <>
+struct Tile<float> {
+    using type = float2;
+    template <bool LOG>
+    static __device__ __forceinline__ double pre(double v) { return v; }
+    template <bool LOG>
+    static __device__ __forceinline__ float2 of(double v, const float2* eighth) {
+        const Pair32 r = recip_pair<LOG>(v, eighth);
+        return make_float2(r.h, r.l);
+    }
+    // 2 (area/d) / (r_K + r_L); false if the FP64 formula has to decide
+    static __device__ __forceinline__ bool link(float2 a, float2 b, float2 ap, double, float& T) {
+        if (a.x == kNoPair || b.x == kNoPair) return false;
+        return round_pair(pair_div(Pair32{ap.x, ap.y}, pair_add(Pair32{a.x, a.y}, Pair32{b.x, b.y})), T);
+    }
+};
+template <>
+struct Tile<double> {
+    using type = double;
+    template <bool LOG>
+    static __device__ __forceinline__ double pre(double v) { return LOG ? exp(v) : v; }
+    template <bool LOG>
+    static __device__ __forceinline__ double of(double k, const float2*) { return k; }
+    // two_point() with the quotient above
+    static __device__ __forceinline__ bool link(double a, double b, float2, double area, double& T) {
+        const uint32_t ea = (uint32_t)__double2hiint(a) >> 20, eb = (uint32_t)__double2hiint(b) >> 20;
+        if (!(min(ea, eb) > 1023u - 90u && max(ea, eb) < 1023u + 90u)) return false;
+        T = __dmul_rn(quotient(__dmul_rn(__dadd_rn(a, a), b), __dadd_rn(a, b)), area);
+        return true;
+    }
+};
+
+constexpr int kTx = 32, kTy = 8;  // cells of a tile (one thread each)
+constexpr int kTransRun = 4;      // planes a block walks (its next plane's own cells are already there)
+
+// Owned transmissibilities of a tile of 32 x 8 cells over kTransRun planes,
+// and (kperm != null) the adjoint's copy of k.  Per plane the tile's
+// reciprocals with the cells its links reach (x - 1 .. x + 32, y .. y + 8) sit
+// in shared memory: 1.2 per cell instead of six.  Measured from ln k with the
+// copy of k (a kernel of its own before): mixed 128^3 704 -> 42 us, FP64
+// 97 x 83 x 50 144 -> 87 us (bound by the FP64 pipe: 1.5 exponentials and five
+// quotients per cell).  Runs of 8 planes instead of 4 measured the same on the
+// mixed path and 7 % slower in FP64 (fewer blocks).
 template <typename Real, bool LOG>
-__global__ void k_store_perm(const double* __restrict__ perm, Real* out, long long n) {
-    for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < n; c += (long long)gridDim.x * blockDim.x)
-        out[c] = (Real)perm_at<LOG>(perm, c);
+__global__ void __launch_bounds__(kTx* kTy) k_trans(GridGeom g, Geo geo, const double* __restrict__ perm, Real* Tx,
+                                                    Real* Ty, Real* Tz, Real* Tpp, Real* Tmp, Real* kperm) {
+    using R = Tile<Real>;
+    using RT = typename R::type;
+    constexpr int PX = kTx + 2, PY = kTy + 1;
+    __shared__ RT tile[2][PY][PX];
+    __shared__ float2 eighth[8];
+    const int tx = threadIdx.x, ty = threadIdx.y, t = tx + kTx * ty;
+    if (sizeof(Real) == 4 && LOG && t < 8) {
+        const float h = (float)kEighth[t];
+        eighth[t] = make_float2(h, (float)(kEighth[t] - (double)h));
+    }
+    if (sizeof(Real) == 4 && LOG) __syncthreads();
+    const int nx = g.nx, ny = g.ny;
+    const long long nxy = (long long)nx * ny;
+    const unsigned bx = (unsigned)(nx + kTx - 1) / kTx, by = (unsigned)(ny + kTy - 1) / kTy;
+    const unsigned bt = blockIdx.x / bx;
+    const int i0 = (int)(blockIdx.x - bt * bx) * kTx, j0 = (int)(bt % by) * kTy;
+    const int i = i0 + tx, j = j0 + ty;
+    const bool act = i < nx && j < ny;
+    // in-range cell of tile position (x, y), x = 0 the cell left of the tile
+    auto cell = [&](int x, int y) {
+        const int ci = min(max(i0 + x - 1, 0), nx - 1), cj = min(j0 + y, ny - 1);
+        return ci + (long long)nx * cj;
+    };
+    const long long own = cell(tx + 1, ty);
+    // the tile's other cells: the row above (34) and the columns left and right (8 each)
+    const bool edge = t < PX + 2 * kTy;
+    const int ex = t < PX ? t : (t - PX < kTy ? 0 : PX - 1);
+    const int ey = t < PX ? kTy : (t - PX) % kTy;
+    const long long ecell = cell(ex, ey);
+    const int k0 = (int)(bt / by) * kTransRun, k1 = min(k0 + kTransRun, g.nz);
+    double vc = R::template pre<LOG>(perm[own + nxy * k0]);  // own k (FP64 path) or the stored value
+    RT rc = R::template of<LOG>(vc, eighth);
+    for (int k = k0; k < k1; ++k) {
+        auto& P = tile[(k - k0) & 1];
+        const long long base = nxy * k;
+        P[ty][tx + 1] = rc;
+        if (edge) P[ey][ex] = R::template of<LOG>(R::template pre<LOG>(perm[base + ecell]), eighth);
+        const bool zp = k + 1 < g.nz;
+        const double vn = zp ? R::template pre<LOG>(perm[base + nxy + own]) : vc;
+        const RT rn = zp ? R::template of<LOG>(vn, eighth) : rc;
+        __syncthreads();
+        const long long c = base + own;
+        auto put = [&](Real* T, bool there, RT rb, float2 ap, double a, long long d) {
+            Real v = Real(0);
+            if (there && !R::link(rc, rb, ap, a, v))
+                v = (Real)two_point(perm_at<LOG>(perm, c), perm_at<LOG>(perm, d), a);
+            T[c] = v;
+        };
+        if (act) {
+            const bool xp = i + 1 < nx, yp = j + 1 < ny;
+            put(Tx, xp, P[ty][tx + 2], geo.px, geo.ax, xp ? c + 1 : c);
+            put(Ty, yp, P[ty + 1][tx + 1], geo.py, geo.ay, yp ? c + nx : c);
+            put(Tz, zp, rn, geo.pz, geo.az, zp ? c + nxy : c);
+            if (g.diag) {
+                const bool pp = yp && xp, mp = yp && i > 0;
+                put(Tpp, pp, P[ty + 1][tx + 2], geo.pd, geo.ad, pp ? c + nx + 1 : c);
+                put(Tmp, mp, P[ty + 1][tx], geo.pd, geo.ad, mp ? c + nx - 1 : c);
+            }
+            if (kperm) {
+                Real kv;
+                if constexpr (sizeof(Real) == 4 && LOG) {
+                    if (rc.x == kNoPair || !round_pair(pair_div(Pair32{1.f, 0.f}, Pair32{rc.x, rc.y}), kv))
+                        kv = (Real)exp(vc);
+                } else {
+                    kv = (Real)vc;
+                }
+                kperm[c] = kv;
+            }
+        }
+        vc = vn;
+        rc = rn;
+    }
 }
 
 // The library's own exponentials, one argument per element: exp_fp64,
@@ -89,6 +315,11 @@ Geo make_geo(const SetupPhys& s) {
     q.az = s.dx * s.dy / s.dz;
     // diagonal: distance sqrt(dx^2 + dy^2), area dz dx dy / distance
     q.ad = s.dz * s.dx * s.dy / (s.dx * s.dx + s.dy * s.dy);
+    auto pair = [](double v) {
+        const float h = (float)v;
+        return make_float2(h, (float)(v - (double)h));
+    };
+    q.px = pair(2.0 * q.ax), q.py = pair(2.0 * q.ay), q.pz = pair(2.0 * q.az), q.pd = pair(2.0 * q.ad);
     return q;
 }
 
@@ -147,33 +378,28 @@ __global__ void k_pattern(GridGeom g, long long* row_ptr, int* col_idx) {
 
 }  // namespace
 
-cudaError_t launch_transmissibility_f32(const GridGeom& g, const SetupPhys& s, const double* perm, float* Tx,
-                                        float* Ty, float* Tz, float* Tpp, float* Tmp, cudaStream_t st, bool log_k) {
-    const long long N = (long long)g.nx * g.ny * g.nz;
-    if (log_k) k_trans<float, true><<<blocks_for(N), kThreads, 0, st>>>(g, make_geo(s), perm, Tx, Ty, Tz, Tpp, Tmp);
-    else k_trans<float, false><<<blocks_for(N), kThreads, 0, st>>>(g, make_geo(s), perm, Tx, Ty, Tz, Tpp, Tmp);
+template <typename Real>
+static cudaError_t launch_trans_t(const GridGeom& g, const SetupPhys& s, const double* perm, Real* Tx, Real* Ty,
+                                  Real* Tz, Real* Tpp, Real* Tmp, Real* kperm, cudaStream_t st, bool log_k) {
+    // one block index for tiles and z-runs: any grid shape of fewer than 2^31 cells fits
+    const long long nb = (long long)((g.nx + kTx - 1) / kTx) * ((g.ny + kTy - 1) / kTy) *
+                         ((g.nz + kTransRun - 1) / kTransRun);
+    const dim3 block(kTx, kTy, 1);
+    if (log_k) k_trans<Real, true><<<(unsigned)nb, block, 0, st>>>(g, make_geo(s), perm, Tx, Ty, Tz, Tpp, Tmp, kperm);
+    else k_trans<Real, false><<<(unsigned)nb, block, 0, st>>>(g, make_geo(s), perm, Tx, Ty, Tz, Tpp, Tmp, kperm);
     return cudaGetLastError();
+}
+
+cudaError_t launch_transmissibility_f32(const GridGeom& g, const SetupPhys& s, const double* perm, float* Tx,
+                                        float* Ty, float* Tz, float* Tpp, float* Tmp, float* kperm, cudaStream_t st,
+                                        bool log_k) {
+    return launch_trans_t<float>(g, s, perm, Tx, Ty, Tz, Tpp, Tmp, kperm, st, log_k);
 }
 
 cudaError_t launch_transmissibility_f64(const GridGeom& g, const SetupPhys& s, const double* perm, double* Tx,
-                                        double* Ty, double* Tz, double* Tpp, double* Tmp, cudaStream_t st,
-                                        bool log_k) {
-    const long long N = (long long)g.nx * g.ny * g.nz;
-    if (log_k) k_trans<double, true><<<blocks_for(N), kThreads, 0, st>>>(g, make_geo(s), perm, Tx, Ty, Tz, Tpp, Tmp);
-    else k_trans<double, false><<<blocks_for(N), kThreads, 0, st>>>(g, make_geo(s), perm, Tx, Ty, Tz, Tpp, Tmp);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_store_perm_f32(const double* perm, float* out, long long n, cudaStream_t st, bool log_k) {
-    if (log_k) k_store_perm<float, true><<<blocks_for(n), kThreads, 0, st>>>(perm, out, n);
-    else k_store_perm<float, false><<<blocks_for(n), kThreads, 0, st>>>(perm, out, n);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_store_perm_f64(const double* perm, double* out, long long n, cudaStream_t st, bool log_k) {
-    if (log_k) k_store_perm<double, true><<<blocks_for(n), kThreads, 0, st>>>(perm, out, n);
-    else k_store_perm<double, false><<<blocks_for(n), kThreads, 0, st>>>(perm, out, n);
-    return cudaGetLastError();
+                                        double* Ty, double* Tz, double* Tpp, double* Tmp, double* kperm,
+                                        cudaStream_t st, bool log_k) {
+    return launch_trans_t<double>(g, s, perm, Tx, Ty, Tz, Tpp, Tmp, kperm, st, log_k);
 }
 
 cudaError_t launch_convert_f32(const double* in, float* out, long long n, cudaStream_t st) {

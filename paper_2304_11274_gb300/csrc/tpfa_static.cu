@@ -148,7 +148,7 @@ extern "C" int tpfa_assemble_jacobian_static(int nx, int ny, int nz, const tpfa_
         float* phi = crk ? reinterpret_cast<float*>(ws + offPhi) : z;  // read only when c_r != 0; never NULL
         if (e == cudaSuccess)
             e = launch_transmissibility_f32(g, sp, perm_dev, (float*)T[0], (float*)T[1], (float*)T[2], (float*)T[3],
-                                            (float*)T[4], st);
+                                            (float*)T[4], nullptr, st);
         if (e == cudaSuccess) e = launch_convert_f32(depth_dev, z, N, st);
         if (e == cudaSuccess && crk) e = launch_convert_f32(poro_dev, phi, N, st);
         if (e == cudaSuccess) e = launch_prev_mass_f32(sp, (const float*)p_prev_dev, poro_dev, mn, N, st);
@@ -164,7 +164,7 @@ extern "C" int tpfa_assemble_jacobian_static(int nx, int ny, int nz, const tpfa_
     } else {
         if (e == cudaSuccess)
             e = launch_transmissibility_f64(g, sp, perm_dev, (double*)T[0], (double*)T[1], (double*)T[2],
-                                            (double*)T[3], (double*)T[4], st);
+                                            (double*)T[3], (double*)T[4], nullptr, st);
         if (e == cudaSuccess) e = launch_prev_mass_f64(sp, (const double*)p_prev_dev, poro_dev, mn, N, st);
         if (e == cudaSuccess) {
             const PhysD q{prm->rho_ref, prm->p_ref, prm->c_f, 1.0 / prm->mu, prm->g, 0.5 * prm->g, V_dt, prm->c_r};
