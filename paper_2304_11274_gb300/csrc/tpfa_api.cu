@@ -108,6 +108,7 @@ struct tpfa_grid {
     void* kperm = nullptr;  // permeability in the field type (adjoint)
     float2* vsplit = nullptr;  // the mixed adjoint's cotangent as FP32 pairs (allocated on first use)
     LinkGeo lg{};           // distance / area per link direction (adjoint)
+    LinkGeoD lgd{};         // the same for the FP64 path
     double* phi0_d = nullptr;
     void* phi0_r = nullptr;  // phi0 in the field type (mixed path with c_r != 0)
     double* mn = nullptr;
@@ -297,7 +298,7 @@ int launch(tpfa_grid* h, AsmKernel kern, double* R, void* vals, double* diag64, 
             e = launch_assemble_mixed(kern, h->geom, h->qf, h->crk, fields_of<float>(h), o, h->JY, h->W, st, k0, k1);
     } else {
         AsmOut<double> o{R, static_cast<double*>(vals), nullptr, h->status};
-        e = launch_assemble_fp64(kern, h->geom, h->qd, h->crk, fields_of<double>(h), o, h->JY, h->W, st, k0, k1);
+        e = launch_assemble_fp64(kern, h->geom, h->qd, h->crk, fields_of<double>(h), o, st, k0, k1);
     }
     if (e != cudaSuccess) return cuda_fail(e, "assembly launch");
     return TPFA_OK;
@@ -658,13 +659,13 @@ int tpfa_create_grid(tpfa_handle* out, int nx, int ny, int nz, const tpfa_params
     h->crk = prm->c_r != 0.0;
     h->real_size = prec == TPFA_MIXED ? sizeof(float) : sizeof(double);
     const double V_dt = prm->dx * prm->dy * prm->dz / prm->dt;
-    h->qd = PhysD{prm->rho_ref, prm->p_ref, prm->c_f, 1.0 / prm->mu, prm->g, 0.5 * prm->g, V_dt, prm->c_r};
+    h->qd = make_phys_d(prm->rho_ref, prm->p_ref, prm->c_f, prm->mu, prm->g, V_dt, prm->c_r);
     h->qf = PhysF{(float)prm->rho_ref, (float)prm->p_ref, (float)prm->c_f, (float)(1.0 / prm->mu),
                   (float)prm->g, (float)(0.5 * prm->g), (float)V_dt, (float)prm->c_r};
     h->sp = SetupPhys{prm->dx, prm->dy, prm->dz, prm->rho_ref, prm->p_ref, prm->c_f, prm->c_r, V_dt};
-    h->lg = LinkGeo{(float)(prm->dx / (prm->dy * prm->dz)), (float)(prm->dy / (prm->dx * prm->dz)),
-                    (float)(prm->dz / (prm->dx * prm->dy)),
-                    (float)((prm->dx * prm->dx + prm->dy * prm->dy) / (prm->dz * prm->dx * prm->dy))};
+    h->lgd = LinkGeoD{prm->dx / (prm->dy * prm->dz), prm->dy / (prm->dx * prm->dz), prm->dz / (prm->dx * prm->dy),
+                      (prm->dx * prm->dx + prm->dy * prm->dy) / (prm->dz * prm->dx * prm->dy)};
+    h->lg = LinkGeo{(float)h->lgd.cx, (float)h->lgd.cy, (float)h->lgd.cz, (float)h->lgd.cd};
     h->nnz = total_nnz(h->geom);
 
     const size_t rb = h->real_size * (size_t)N;
@@ -944,8 +945,8 @@ int tpfa_vjp_kernel(tpfa_handle h, tpfa_kernel kern, const double* v_dev, double
                              h->vsplit, g_p_dev, g_lnk_dev, h->status,
                              k == AsmKernel::XMarch ? march_rows2(h) : march_rows(h), h->W, st);
     else
-        e = launch_vjp_fp64(h->geom, h->qd, h->crk, fields_of<double>(h), (const double*)h->kperm, v_dev, g_p_dev,
-                            g_lnk_dev, h->status, st);
+        e = launch_vjp_fp64(h->geom, h->qd, h->crk, fields_of<double>(h), (const double*)h->kperm, h->lgd, v_dev,
+                            g_p_dev, g_lnk_dev, h->status, st);
     if (e != cudaSuccess) return cuda_fail(e, "vjp launch");
     return TPFA_OK;
 }
@@ -1252,7 +1253,7 @@ int tpfa_create_mesh(tpfa_mesh* out, long long n_cells, long long n_conn, const 
     m->crk = prm->c_r != 0.0;
     m->real_size = prec == TPFA_MIXED ? sizeof(float) : sizeof(double);
     // the cell volume is folded into m^n and into (V/dt) phi0, so V_dt = 1
-    m->qd = PhysD{prm->rho_ref, prm->p_ref, prm->c_f, 1.0 / prm->mu, prm->g, 0.5 * prm->g, 1.0, prm->c_r};
+    m->qd = make_phys_d(prm->rho_ref, prm->p_ref, prm->c_f, prm->mu, prm->g, 1.0, prm->c_r);
     m->qf = PhysF{(float)prm->rho_ref, (float)prm->p_ref, (float)prm->c_f, (float)(1.0 / prm->mu), (float)prm->g,
                   (float)(0.5 * prm->g), 1.0f, (float)prm->c_r};
     m->sp = SetupPhys{1.0, 1.0, 1.0, prm->rho_ref, prm->p_ref, prm->c_f, prm->c_r, 1.0};

@@ -1,6 +1,7 @@
 // tpfa_assemble.cu -- residual + Jacobian assembly kernels (sm_103a).
 //
-// Two kernels compute the same rows (see tpfa_row.cuh for the row layout and
+// The mixed path's kernels and the naive kernel of both paths (the FP64 path's
+// own kernel is in tpfa_fp64.cu).  They compute the same rows (see tpfa_row.cuh for the row layout and
 // summation order), so their outputs are bit-identical:
 //
 //   k_assemble_naive  -- one thread per cell; the cell and its 10 neighbours
@@ -49,25 +50,23 @@ static cudaError_t launch_naive_t(const GridGeom& g, const typename PhysOf<Real>
 }
 
 // Planes [k0, k1) of the grid; the whole grid by default.
-template <typename Real, bool DIAG, bool CRK, bool JAC, int W>
-static cudaError_t launch_ymarch_w(const GridGeom& g, const typename PhysOf<Real>::type& q,
-                                   const AsmFields<Real>& f, const AsmOut<Real>& o, int JY, int k0, int k1,
-                                   cudaStream_t st) {
-    constexpr int smem = ymarch_smem_bytes<Real, W>();
-    const cudaError_t e = ensure_smem_limit(reinterpret_cast<const void*>(&k_assemble_ymarch<Real, DIAG, CRK, JAC, W>), smem);
+template <bool DIAG, bool CRK, bool JAC, int W>
+static cudaError_t launch_ymarch_w(const GridGeom& g, const PhysF& q, const AsmFields<float>& f,
+                                   const AsmOut<float>& o, int JY, int k0, int k1, cudaStream_t st) {
+    constexpr int smem = ymarch_smem_bytes<W>();
+    const cudaError_t e = ensure_smem_limit(reinterpret_cast<const void*>(&k_assemble_ymarch<DIAG, CRK, JAC, W>), smem);
     if (e != cudaSuccess) return e;
     dim3 block(32, W, 1);
     dim3 grid((g.nx + 31) / 32, (g.ny + JY - 1) / JY, (k1 - k0 + W - 1) / W);
-    k_assemble_ymarch<Real, DIAG, CRK, JAC, W><<<grid, block, smem, st>>>(g, q, f, o, JY, k0, k1);
+    k_assemble_ymarch<DIAG, CRK, JAC, W><<<grid, block, smem, st>>>(g, q, f, o, JY, k0, k1);
     return cudaGetLastError();
 }
 
-template <typename Real, bool DIAG, bool CRK, bool JAC>
-static cudaError_t launch_ymarch_t(const GridGeom& g, const typename PhysOf<Real>::type& q,
-                                   const AsmFields<Real>& f, const AsmOut<Real>& o, int JY, int W, int k0,
-                                   int k1, cudaStream_t st) {
-    if (W == 8) return launch_ymarch_w<Real, DIAG, CRK, JAC, 8>(g, q, f, o, JY, k0, k1, st);
-    return launch_ymarch_w<Real, DIAG, CRK, JAC, 4>(g, q, f, o, JY, k0, k1, st);
+template <bool DIAG, bool CRK, bool JAC>
+static cudaError_t launch_ymarch_t(const GridGeom& g, const PhysF& q, const AsmFields<float>& f,
+                                   const AsmOut<float>& o, int JY, int W, int k0, int k1, cudaStream_t st) {
+    if (W == 8) return launch_ymarch_w<DIAG, CRK, JAC, 8>(g, q, f, o, JY, k0, k1, st);
+    return launch_ymarch_w<DIAG, CRK, JAC, 4>(g, q, f, o, JY, k0, k1, st);
 }
 
 // ------------------------------------------------------------------ two cells per lane
@@ -113,37 +112,17 @@ bool xmarch_ok(const GridGeom& g, const AsmFields<float>& f) {
 }
 
 template <typename Real>
-static cudaError_t dispatch(AsmKernel kern, const GridGeom& g, const typename PhysOf<Real>::type& q,
-                            bool crk, const AsmFields<Real>& f, const AsmOut<Real>& o, int JY, int W, int k0,
-                            int k1, cudaStream_t st) {
+static cudaError_t launch_naive(const GridGeom& g, const typename PhysOf<Real>::type& q, bool crk,
+                                const AsmFields<Real>& f, const AsmOut<Real>& o, cudaStream_t st) {
     const bool jac = o.vals != nullptr;
+    if (crk) return jac ? launch_naive_t<Real, true, true>(g, q, f, o, st) : launch_naive_t<Real, true, false>(g, q, f, o, st);
+    return jac ? launch_naive_t<Real, false, true>(g, q, f, o, st) : launch_naive_t<Real, false, false>(g, q, f, o, st);
+}
+
+// The planes of a launch: all of them by default.
+static void clamp_planes(const GridGeom& g, int& k0, int& k1) {
     if (k1 < 0 || k1 > g.nz) k1 = g.nz;
     if (k0 < 0 || k0 >= k1) k0 = 0;
-    if (kern == AsmKernel::Naive) {
-        if (crk) return jac ? launch_naive_t<Real, true, true>(g, q, f, o, st) : launch_naive_t<Real, true, false>(g, q, f, o, st);
-        return jac ? launch_naive_t<Real, false, true>(g, q, f, o, st) : launch_naive_t<Real, false, false>(g, q, f, o, st);
-    }
-    if constexpr (sizeof(Real) == 4) {
-        // two cells per lane: the mixed path's fused R + J on grids with nx even
-        // and pair-aligned fields; otherwise (and for residual-only calls) the
-        // one-cell march
-        if (kern == AsmKernel::XMarch && jac && xmarch_ok(g, f)) {
-            if (g.diag) return crk ? launch_xmarch_t<true, true>(g, q, f, o, JY, W, k0, k1, st)
-                                   : launch_xmarch_t<true, false>(g, q, f, o, JY, W, k0, k1, st);
-            return crk ? launch_xmarch_t<false, true>(g, q, f, o, JY, W, k0, k1, st)
-                       : launch_xmarch_t<false, false>(g, q, f, o, JY, W, k0, k1, st);
-        }
-    }
-    if (g.diag) {
-        if (crk) return jac ? launch_ymarch_t<Real, true, true, true>(g, q, f, o, JY, W, k0, k1, st)
-                            : launch_ymarch_t<Real, true, true, false>(g, q, f, o, JY, W, k0, k1, st);
-        return jac ? launch_ymarch_t<Real, true, false, true>(g, q, f, o, JY, W, k0, k1, st)
-                   : launch_ymarch_t<Real, true, false, false>(g, q, f, o, JY, W, k0, k1, st);
-    }
-    if (crk) return jac ? launch_ymarch_t<Real, false, true, true>(g, q, f, o, JY, W, k0, k1, st)
-                        : launch_ymarch_t<Real, false, true, false>(g, q, f, o, JY, W, k0, k1, st);
-    return jac ? launch_ymarch_t<Real, false, false, true>(g, q, f, o, JY, W, k0, k1, st)
-               : launch_ymarch_t<Real, false, false, false>(g, q, f, o, JY, W, k0, k1, st);
 }
 
 // ------------------------------------------------------------------ TMA march
@@ -157,7 +136,7 @@ template <bool DIAG, bool CRK, bool JAC>
 static cudaError_t launch_tma_t(const GridGeom& g, const PhysF& q, const AsmFields<float>& f, const AsmOut<float>& o,
                                 const TmaMaps& maps, int JY, int k0, int k1, cudaStream_t st) {
     constexpr int W = kTmaWarps;
-    constexpr int smem = ymarch_tma_smem_bytes<W, YMarch<float, DIAG, CRK, JAC, W>::TRING>();
+    constexpr int smem = ymarch_tma_smem_bytes<W, YMarch<DIAG, CRK, JAC, W>::TRING>();
     const cudaError_t e = ensure_smem_limit(reinterpret_cast<const void*>(&k_assemble_ymarch_tma<DIAG, CRK, JAC, W>), smem);
     if (e != cudaSuccess) return e;
     dim3 block(32, W, 1);
@@ -170,8 +149,7 @@ cudaError_t launch_assemble_mixed_tma(const GridGeom& g, const PhysF& q, bool cr
                                       const AsmOut<float>& o, const TmaMaps& maps, int JY, int W, cudaStream_t st,
                                       int k0, int k1) {
     const bool jac = o.vals != nullptr;
-    if (k1 < 0 || k1 > g.nz) k1 = g.nz;
-    if (k0 < 0 || k0 >= k1) k0 = 0;
+    clamp_planes(g, k0, k1);
     if (g.diag) {
         if (crk) return jac ? launch_tma_t<true, true, true>(g, q, f, o, maps, JY, k0, k1, st)
                             : launch_tma_t<true, true, false>(g, q, f, o, maps, JY, k0, k1, st);
@@ -249,13 +227,34 @@ bool tma_encode_static(TmaMaps* m, const GridGeom& g, const AsmFields<float>& f,
 cudaError_t launch_assemble_mixed(AsmKernel kern, const GridGeom& g, const PhysF& q, bool crk,
                                   const AsmFields<float>& f, const AsmOut<float>& o, int JY, int W,
                                   cudaStream_t st, int k0, int k1) {
-    return dispatch<float>(kern, g, q, crk, f, o, JY, W, k0, k1, st);
+    const bool jac = o.vals != nullptr;
+    clamp_planes(g, k0, k1);
+    if (kern == AsmKernel::Naive) return launch_naive<float>(g, q, crk, f, o, st);
+    // two cells per lane: fused R + J on grids with nx even and pair-aligned
+    // fields; otherwise (and for residual-only calls) the one-cell march
+    if (kern == AsmKernel::XMarch && jac && xmarch_ok(g, f)) {
+        if (g.diag) return crk ? launch_xmarch_t<true, true>(g, q, f, o, JY, W, k0, k1, st)
+                               : launch_xmarch_t<true, false>(g, q, f, o, JY, W, k0, k1, st);
+        return crk ? launch_xmarch_t<false, true>(g, q, f, o, JY, W, k0, k1, st)
+                   : launch_xmarch_t<false, false>(g, q, f, o, JY, W, k0, k1, st);
+    }
+    if (g.diag) {
+        if (crk) return jac ? launch_ymarch_t<true, true, true>(g, q, f, o, JY, W, k0, k1, st)
+                            : launch_ymarch_t<true, true, false>(g, q, f, o, JY, W, k0, k1, st);
+        return jac ? launch_ymarch_t<true, false, true>(g, q, f, o, JY, W, k0, k1, st)
+                   : launch_ymarch_t<true, false, false>(g, q, f, o, JY, W, k0, k1, st);
+    }
+    if (crk) return jac ? launch_ymarch_t<false, true, true>(g, q, f, o, JY, W, k0, k1, st)
+                        : launch_ymarch_t<false, true, false>(g, q, f, o, JY, W, k0, k1, st);
+    return jac ? launch_ymarch_t<false, false, true>(g, q, f, o, JY, W, k0, k1, st)
+               : launch_ymarch_t<false, false, false>(g, q, f, o, JY, W, k0, k1, st);
 }
 
 cudaError_t launch_assemble_fp64(AsmKernel kern, const GridGeom& g, const PhysD& q, bool crk,
-                                 const AsmFields<double>& f, const AsmOut<double>& o, int JY, int W,
-                                 cudaStream_t st, int k0, int k1) {
-    return dispatch<double>(kern, g, q, crk, f, o, JY, W, k0, k1, st);
+                                 const AsmFields<double>& f, const AsmOut<double>& o, cudaStream_t st, int k0, int k1) {
+    clamp_planes(g, k0, k1);
+    if (kern == AsmKernel::Naive) return launch_naive<double>(g, q, crk, f, o, st);
+    return launch_cells_fp64(g, q, crk, f, o, st, k0, k1);
 }
 
 }  // namespace tpfa

@@ -48,14 +48,14 @@ __global__ void __launch_bounds__(32 * W, 16 / W)
         }
         __syncthreads();
         if (s_tile >= total) break;
-        ymarch_tile<float, DIAG, CRK, true, W, true>(sm.g, sm.q, sm.f, sm.o, JY, s_bx, s_by, s_bz, smem);
+        ymarch_tile<DIAG, CRK, true, W, true>(sm.g, sm.q, sm.f, sm.o, JY, s_bx, s_by, s_bz, smem);
         __syncthreads();  // every warp is done with this tile's descriptor and buffers
     }
 }
 
 template <bool DIAG, bool CRK, int W>
 cudaError_t config(const void** func, int* smem_bytes) {
-    constexpr int smem = ymarch_smem_bytes<float, W>();
+    constexpr int smem = ymarch_smem_bytes<W>();
     const void* f = reinterpret_cast<const void*>(&k_assemble_batch<DIAG, CRK, W>);
     const cudaError_t e = ensure_smem_limit(f, smem);
     if (e != cudaSuccess) return e;

@@ -127,7 +127,9 @@ __device__ __forceinline__ float diff_f2(const F2Split& a, const F2Split& b) {
 struct LinkGeo {
     float cx, cy, cz, cd;
 };
-
+struct LinkGeoD {
+    double cx, cy, cz, cd;
+};
 
 // ---------------------------------------------------------------- Kahan
 
@@ -147,13 +149,35 @@ template <typename T>
 struct CellVal {
     T p, z, rho, drho;  // pressure, depth, density, d rho / dp
 };
+// The FP64 path carries the mobility rho / mu instead of the density (one
+// product per cell instead of one per link); its derivative c_f rho / mu
+// only appears inside the link.
+template <>
+struct CellVal<double> {
+    double p, z, lam;  // pressure, depth, rho / mu
+};
 
 struct PhysF {
     float rho_ref, p_ref, c_f, inv_mu, g, half_g, V_dt, c_r;
 };
+// FP64 constants, combined once on the host.
 struct PhysD {
-    double rho_ref, p_ref, c_f, inv_mu, g, half_g, V_dt, c_r;
+    double p_ref, c_f;
+    double lam_ref;  // rho_ref / mu
+    double hg, chg;  // g mu / 2 and c_f g mu / 2: (rho_a + rho_b) g / 2 = (lam_a + lam_b) hg
+    double vol;      // (V/dt) mu
+    double vol_cr;   // (V/dt) mu c_r
+    double cc, cs;   // c_f c_r and c_f + c_r
 };
+inline PhysD make_phys_d(double rho_ref, double p_ref, double c_f, double mu, double g, double V_dt, double c_r) {
+    PhysD q;
+    q.p_ref = p_ref, q.c_f = c_f;
+    q.lam_ref = rho_ref / mu;
+    q.hg = 0.5 * g * mu, q.chg = c_f * (0.5 * g * mu);
+    q.vol = V_dt * mu, q.vol_cr = V_dt * mu * c_r;
+    q.cc = c_f * c_r, q.cs = c_f + c_r;
+    return q;
+}
 
 // exp(x) and expm1(x) in FP64 for the small arguments the state equation
 // meets (|x| < 2^-5: c_f (p - p_ref) with c_f ~ 1e-9 / Pa and pressures
@@ -161,32 +185,52 @@ struct PhysD {
 // and x^9 (expm1): the remainder is below 2^-60 of the value, so the result
 // is the function's within the few roundings of the Horner steps.  Larger
 // arguments (and NaN or infinity) take exp() / expm1().  The FP64 path is
-// bound by the FP64 pipe, and these series need fewer FP64 instructions per
-// exponential call.  The range test reads the high word (integer pipe).
-__device__ __forceinline__ bool small_arg(double x) {
-    return ((uint32_t)__double2hiint(x) & 0x7fffffffu) < 0x3fa00000u;  // |x| < 2^-5
-}
+// bound by the FP64 pipe (two operations per clock per multiprocessor), and
+// these series need fewer FP64 instructions per call; smaller arguments still
+// fewer: below 2^-6 the terms of exp from x^5 / 5! on are less than 2^-36 of
+// the value, so their sum over x^5 is taken in FP32 (its error stays below
+// 2^-59 of the value) and five FP64 operations remain of eight; below 2^-10 the
+// terms of expm1 from x^4 / 4! on are less than 2^-34 of it, and four of ten
+// remain.  The range tests read the high word (integer pipe).
+__device__ __forceinline__ uint32_t abs_hi(double x) { return (uint32_t)__double2hiint(x) & 0x7fffffffu; }
 __device__ __forceinline__ double exp_fp64(double x) {
-    if (!small_arg(x)) return exp(x);
-    double r = 1.0 / 40320.0;  // 1/8!
-    r = __fma_rn(r, x, 1.0 / 5040.0);
-    r = __fma_rn(r, x, 1.0 / 720.0);
-    r = __fma_rn(r, x, 1.0 / 120.0);
-    r = __fma_rn(r, x, 1.0 / 24.0);
+    const uint32_t a = abs_hi(x);
+    double r;
+    if (a < 0x3f900000u) {  // |x| < 2^-6
+        const float xf = narrow_flush(x);
+        const float t = __fmaf_rn(__fmaf_rn(xf, 1.f / 5040.f, 1.f / 720.f), xf, 1.f / 120.f);
+        r = __fma_rn(widen_flush(t), x, 1.0 / 24.0);
+    } else if (a < 0x3fa00000u) {  // |x| < 2^-5
+        r = 1.0 / 40320.0;  // 1/8!
+        r = __fma_rn(r, x, 1.0 / 5040.0);
+        r = __fma_rn(r, x, 1.0 / 720.0);
+        r = __fma_rn(r, x, 1.0 / 120.0);
+        r = __fma_rn(r, x, 1.0 / 24.0);
+    } else {
+        return exp(x);
+    }
     r = __fma_rn(r, x, 1.0 / 6.0);
     r = __fma_rn(r, x, 0.5);
     r = __fma_rn(r, x, 1.0);
     return __fma_rn(r, x, 1.0);
 }
 __device__ __forceinline__ double expm1_fp64(double x) {
-    if (!small_arg(x)) return expm1(x);
-    double r = 1.0 / 362880.0;  // 1/9!: expm1(x) = x (1 + x/2! + x^2/3! + ... + x^8/9!)
-    r = __fma_rn(r, x, 1.0 / 40320.0);
-    r = __fma_rn(r, x, 1.0 / 5040.0);
-    r = __fma_rn(r, x, 1.0 / 720.0);
-    r = __fma_rn(r, x, 1.0 / 120.0);
-    r = __fma_rn(r, x, 1.0 / 24.0);
-    r = __fma_rn(r, x, 1.0 / 6.0);
+    const uint32_t a = abs_hi(x);
+    double r;
+    if (a < 0x3f500000u) {  // |x| < 2^-10
+        const float t = __fmaf_rn(narrow_flush(x), 1.f / 120.f, 1.f / 24.f);
+        r = __fma_rn(widen_flush(t), x, 1.0 / 6.0);
+    } else if (a < 0x3fa00000u) {  // |x| < 2^-5
+        r = 1.0 / 362880.0;  // 1/9!: expm1(x) = x (1 + x/2! + x^2/3! + ... + x^8/9!)
+        r = __fma_rn(r, x, 1.0 / 40320.0);
+        r = __fma_rn(r, x, 1.0 / 5040.0);
+        r = __fma_rn(r, x, 1.0 / 720.0);
+        r = __fma_rn(r, x, 1.0 / 120.0);
+        r = __fma_rn(r, x, 1.0 / 24.0);
+        r = __fma_rn(r, x, 1.0 / 6.0);
+    } else {
+        return expm1(x);
+    }
     r = __fma_rn(r, x, 0.5);
     r = __fma_rn(r, x, 1.0);
     return __dmul_rn(r, x);
@@ -205,8 +249,7 @@ __device__ __forceinline__ CellVal<double> make_cell(const PhysD& q, double p, d
     CellVal<double> c;
     c.p = p;
     c.z = z;
-    c.rho = __dmul_rn(q.rho_ref, exp_fp64(__dmul_rn(q.c_f, __dsub_rn(p, q.p_ref))));
-    c.drho = __dmul_rn(q.c_f, c.rho);
+    c.lam = __dmul_rn(q.lam_ref, exp_fp64(__dmul_rn(q.c_f, __dsub_rn(p, q.p_ref))));
     return c;
 }
 
@@ -217,6 +260,12 @@ struct LinkOut {
     T F;   // F_ab: mass outflow from a to b
     T Da;  // dF_ab / dp_a
     T Db;  // dF_ab / dp_b
+};
+// FP64 path: also the gravity parts, which the sums below need.
+template <>
+struct LinkOut<double> {
+    double F, Da, Db;
+    double u, rs;  // T lam_up c_f (g mu / 2)(z_a - z_b) and lam_a + lam_b
 };
 
 // Two-point flux of Eq. flux-calc seen from row a (z = depth, positive down):
@@ -247,22 +296,58 @@ __device__ __forceinline__ LinkOut<float> link(const PhysF& q, float T, const Ce
     return r;
 }
 
+// FP64: the same flux with the mobility lam = rho / mu,
+//   F = T lam_up dPhi,  dF/dp_a =  T lam_up (1 - c_f lam_a hg dz) + [up = a] c_f F
+//                       dF/dp_b = -T lam_up (1 + c_f lam_b hg dz) + [up = b] c_f F
+// (d lam / dp = c_f lam, so the mobility's term is c_f F).  Cells at one depth
+// have no gravity terms: FLAT leaves them out, which gives the same bits as
+// evaluating them with dz = 0 (a sum with an exact zero), so a kernel may
+// choose it for any set of links that link_flat() admits.
+template <bool FLAT>
+__device__ __forceinline__ LinkOut<double> link_d(const PhysD& q, double T, const CellVal<double>& a,
+                                                  const CellVal<double>& b) {
+    LinkOut<double> r;
+    double dphi = __dsub_rn(a.p, b.p);
+    double dz = 0.0;
+    r.rs = 0.0;
+    if (!FLAT) {
+        dz = __dsub_rn(a.z, b.z);
+        r.rs = __dadd_rn(a.lam, b.lam);
+        dphi = __fma_rn(-r.rs, __dmul_rn(q.hg, dz), dphi);
+    }
+    // dphi > 0 on the integer pipe: positive, not zero, not NaN
+    const long long bits = __double_as_longlong(dphi);
+    const bool up_a = bits > 0 && bits <= 0x7ff0000000000000ll;
+    const double Tl = __dmul_rn(T, up_a ? a.lam : b.lam);
+    r.F = __dmul_rn(Tl, dphi);
+    r.u = 0.0;
+    double da = Tl, db = -Tl;
+    if (!FLAT) {
+        r.u = __dmul_rn(__dmul_rn(q.chg, dz), Tl);
+        da = __fma_rn(-r.u, a.lam, Tl);
+        db = -__fma_rn(r.u, b.lam, Tl);
+    }
+    r.Da = __fma_rn(q.c_f, up_a ? r.F : 0.0, da);
+    r.Db = __fma_rn(q.c_f, up_a ? 0.0 : r.F, db);
+    return r;
+}
+// Whether FLAT gives the link's bits: equal finite depths and finite mobilities.
+__device__ __forceinline__ bool link_flat(const CellVal<double>& a, const CellVal<double>& b) {
+    return __double_as_longlong(a.z) == __double_as_longlong(b.z) && abs_hi(a.z) < 0x7ff00000u &&
+           abs_hi(a.lam) < 0x7ff00000u && abs_hi(b.lam) < 0x7ff00000u;
+}
 __device__ __forceinline__ LinkOut<double> link(const PhysD& q, double T, const CellVal<double>& a,
                                                 const CellVal<double>& b) {
-    const double dp = __dsub_rn(a.p, b.p);
-    const double hgdz = __dmul_rn(q.half_g, __dsub_rn(a.z, b.z));
-    const double dphi = __fma_rn(-__dadd_rn(a.rho, b.rho), hgdz, dp);
-    const bool up_a = dphi > 0.0;
-    const double Tm = __dmul_rn(T, q.inv_mu);
-    const double Tl = __dmul_rn(Tm, up_a ? a.rho : b.rho);
-    const double w = __dmul_rn(Tm, dphi);
-    LinkOut<double> r;
-    r.F = __dmul_rn(Tl, dphi);
-    const double dda = __fma_rn(-a.drho, hgdz, 1.0);
-    const double ddb = __fma_rn(-b.drho, hgdz, -1.0);
-    r.Da = __fma_rn(Tl, dda, __dmul_rn(up_a ? a.drho : 0.0, w));
-    r.Db = __fma_rn(Tl, ddb, __dmul_rn(up_a ? 0.0 : b.drho, w));
-    return r;
+    return link_d<false>(q, T, a, b);
+}
+// The link seen from its other end: exact except at a tie dPhi == 0, where
+// each end takes the other cell as upstream.
+__device__ __forceinline__ LinkOut<double> flip(const LinkOut<double>& l) {
+    return LinkOut<double>{-l.F, -l.Db, -l.Da, -l.u, l.rs};
+}
+// Whether a link may be an exact tie (zero flux; harmlessly also underflow).
+__device__ __forceinline__ bool zero_flux(const LinkOut<double>& l) {
+    return (__double_as_longlong(l.F) << 1) == 0;
 }
 
 // ---------------------------------------------------------------- packed FP32x2
@@ -369,23 +454,43 @@ struct AccD {
     double A, dA;
 };
 
+// `lam` is rho(p) / mu.  With c_r == 0, dA = c_f mn exp(c_f (p - p^n)) = c_f (mn + A).
 template <bool CR>
-__device__ __forceinline__ AccD accumulation(const PhysD& q, double p, double pn, double mn, double rho,
+__device__ __forceinline__ AccD accumulation(const PhysD& q, double p, double pn, double mn, double lam,
                                              double phi0) {
     const double dpn = __dsub_rn(p, pn);
     const double e = expm1_fp64(__dmul_rn(q.c_f, dpn));
     AccD r;
     r.A = __dmul_rn(mn, e);
     if (CR) {
-        const double vphi = __dmul_rn(q.V_dt, phi0);
-        r.A = __fma_rn(__dmul_rn(vphi, q.c_r), __dmul_rn(dpn, rho), r.A);
-        const double phi_rel = __fma_rn(q.c_r, __dsub_rn(p, q.p_ref), 1.0);
-        r.dA = __dmul_rn(__dmul_rn(vphi, rho), __fma_rn(phi_rel, q.c_f, q.c_r));
+        r.A = __fma_rn(__dmul_rn(phi0, q.vol_cr), __dmul_rn(dpn, lam), r.A);
+        r.dA = __dmul_rn(__dmul_rn(__dmul_rn(phi0, q.vol), lam), __fma_rn(q.cc, __dsub_rn(p, q.p_ref), q.cs));
     } else {
-        r.dA = __dmul_rn(__dmul_rn(q.c_f, mn), __dadd_rn(1.0, e));
+        r.dA = __dmul_rn(q.c_f, __dadd_rn(mn, r.A));
     }
     return r;
 }
+
+// Sums of an FP64 row over its links, in slot order.  The diagonal needs no
+// term of its own per link: dF/dp_a + dF/dp_b = c_f F - u (lam_a + lam_b), so
+//   sum dF/dp_a = -sum dF/dp_b + (c_f sum F - sum u rs),
+// the bracket and dA small beside the first sum, which they join last.
+struct RowAccD {
+    double F = 0.0, d = 0.0, grav = 0.0;  // sum F, -sum dF/dp_b, -sum u rs
+    template <bool JAC, bool FLAT = false>
+    __device__ __forceinline__ void add(const LinkOut<double>& l) {
+        F = __dadd_rn(F, l.F);
+        if (JAC) d = __dsub_rn(d, l.Db);
+        if (!FLAT) grav = __fma_rn(-l.u, l.rs, grav);
+    }
+    // sum dF/dp_a + sum dF/dp_b + dA, and the row's diagonal dR_K/dp_K
+    __device__ __forceinline__ double excess(const PhysD& q, double dA) const {
+        return __dadd_rn(__fma_rn(q.c_f, F, grav), dA);
+    }
+    __device__ __forceinline__ double diagonal(const PhysD& q, double dA) const {
+        return __dadd_rn(d, excess(q, dA));
+    }
+};
 
 // Non-finite test on the integer pipe (exponent all ones).
 __device__ __forceinline__ bool nonfinite(double x) {

@@ -22,9 +22,13 @@ enum class AsmKernel { Naive, YMarch, YMarchTma, XMarch };
 cudaError_t launch_assemble_mixed(AsmKernel kern, const GridGeom& g, const PhysF& q, bool crk,
                                   const AsmFields<float>& f, const AsmOut<float>& o, int JY, int W,
                                   cudaStream_t st, int k0 = 0, int k1 = -1);
+// FP64: the naive kernel, or for any other choice the tile kernel of
+// tpfa_fp64.cu (its tiles follow from the grid).
 cudaError_t launch_assemble_fp64(AsmKernel kern, const GridGeom& g, const PhysD& q, bool crk,
-                                 const AsmFields<double>& f, const AsmOut<double>& o, int JY, int W,
-                                 cudaStream_t st, int k0 = 0, int k1 = -1);
+                                 const AsmFields<double>& f, const AsmOut<double>& o, cudaStream_t st, int k0 = 0,
+                                 int k1 = -1);
+cudaError_t launch_cells_fp64(const GridGeom& g, const PhysD& q, bool crk, const AsmFields<double>& f,
+                              const AsmOut<double>& o, cudaStream_t st, int k0, int k1);
 // The mixed march with TMA row loads (same rows, same bits).  The maps come
 // from tma_encode_state (p, p^n: whenever the bound pointers change) and
 // tma_encode_static (the library-owned fields); both return false when the
@@ -65,6 +69,7 @@ cudaError_t launch_prev_mass_f64(const SetupPhys& s, const double* pn, const dou
                                  long long n, cudaStream_t st);
 // Adjoint (tpfa_vjp.cu).
 struct LinkGeo;
+struct LinkGeoD;
 // The mixed path's adjoint runs the y-march (JY rows per march, W warps per
 // block) or its naive gather twin; lg: distance over area per link direction.
 // vsplit: N float2 of workspace for the cotangent's FP32 pairs.
@@ -72,7 +77,7 @@ cudaError_t launch_vjp_mixed(AsmKernel kern, const GridGeom& g, const PhysF& q, 
                              const float* kperm, const LinkGeo& lg, const double* v, float2* vsplit, double* g_p,
                              double* g_lnk, unsigned int* status, int JY, int W, cudaStream_t st);
 cudaError_t launch_vjp_fp64(const GridGeom& g, const PhysD& q, bool crk, const AsmFields<double>& f,
-                            const double* kperm, const double* v, double* g_p, double* g_lnk,
+                            const double* kperm, const LinkGeoD& lg, const double* v, double* g_p, double* g_lnk,
                             unsigned int* status, cudaStream_t st);
 // Matrix-free J w (tpfa_jvp.cu); R may be null.  The mixed path runs the
 // y-march (JY rows per march, W warps per block) or the naive gather.

@@ -77,7 +77,7 @@ __global__ void __launch_bounds__(kRows) k_mesh_assemble(MeshFields<Real> f, lon
                 put(dpos, __fsub_rn(dsum.s, dsum.c));
             }
         } else {
-            double rsum = 0.0, dsum = 0.0;
+            RowAccD sum;
             for (long long e = rs; e < re; ++e) {
                 const long long c = ldm(f.col, e, nnz, o.status);
                 if (c == r) {
@@ -86,19 +86,15 @@ __global__ void __launch_bounds__(kRows) k_mesh_assemble(MeshFields<Real> f, lon
                 }
                 const CellVal<double> nb = make_cell(q, ldm(f.p, c, n, o.status), ldm(f.z, c, n, o.status));
                 const LinkOut<double> L = link(q, ldm(f.Tc, e, nnz, o.status), me, nb);
-                rsum = __dadd_rn(rsum, L.F);
-                if (JAC) {
-                    dsum = __dadd_rn(dsum, L.Da);
-                    put(e, L.Db);
-                }
+                sum.add<JAC>(L);
+                if (JAC) put(e, L.Db);
             }
-            const AccD acc = accumulation<CRK>(q, me.p, f.pn[r], f.mn[r], me.rho, CRK ? f.phi0[r] : 0.0);
-            out.R = __dadd_rn(rsum, acc.A);
+            const AccD acc = accumulation<CRK>(q, me.p, f.pn[r], f.mn[r], me.lam, CRK ? f.phi0[r] : 0.0);
+            out.R = __dadd_rn(sum.F, acc.A);
             out.diag64 = 0.0;
             if (JAC) {
-                dsum = __dadd_rn(dsum, acc.dA);
-                out.diag64 = dsum;
-                put(dpos, dsum);
+                out.diag64 = sum.diagonal(q, acc.dA);
+                put(dpos, out.diag64);
             }
         }
         if (o.R) o.R[r] = out.R;

@@ -97,27 +97,23 @@ template <bool CRK, bool JAC, typename Sink>
 __device__ __forceinline__ RowSums assemble_row(const PhysD& q, const CellVal<double>& me,
                                                 const CellVal<double> (&nb)[NSLOT], const double (&T)[NSLOT],
                                                 unsigned mask, double pn, double mn, double phi0, Sink&& sink) {
-    double rs = 0.0, ds = 0.0;
+    RowAccD sum;
 #pragma unroll
     for (int s = 0; s < NSLOT; ++s) {
         if (s == SLOT_SELF) continue;
         if (mask & (1u << s)) {
             const LinkOut<double> L = link(q, T[s], me, nb[s]);
-            rs = __dadd_rn(rs, L.F);
-            if (JAC) {
-                ds = __dadd_rn(ds, L.Da);
-                sink(slot_pos(mask, s), L.Db);
-            }
+            sum.add<JAC>(L);
+            if (JAC) sink(slot_pos(mask, s), L.Db);
         }
     }
-    const AccD acc = accumulation<CRK>(q, me.p, pn, mn, me.rho, phi0);
+    const AccD acc = accumulation<CRK>(q, me.p, pn, mn, me.lam, phi0);
     RowSums out;
-    out.R = __dadd_rn(rs, acc.A);
+    out.R = __dadd_rn(sum.F, acc.A);
     out.diag64 = 0.0;
     if (JAC) {
-        ds = __dadd_rn(ds, acc.dA);
-        out.diag64 = ds;
-        sink(slot_pos(mask, SLOT_SELF), ds);
+        out.diag64 = sum.diagonal(q, acc.dA);
+        sink(slot_pos(mask, SLOT_SELF), out.diag64);
     }
     out.bad = nonfinite(out.R) || (JAC && nonfinite(out.diag64));
     return out;

@@ -5,6 +5,7 @@
 
 #include "tpfa_common.cuh"
 #include "tpfa_impl.h"
+#include "tpfa_tile.h"
 
 namespace tpfa {
 
@@ -206,26 +207,32 @@ struct Tile<double> {
     }
 };
 
-constexpr int kTx = 32, kTy = 8;  // cells of a tile (one thread each)
+constexpr int kTileThreads = 256;  // cells of a tile at most (one thread each)
 constexpr int kTransRun = 4;      // planes a block walks (its next plane's own cells are already there)
 
-// Owned transmissibilities of a tile of 32 x 8 cells over kTransRun planes,
+// Owned transmissibilities of a tile of TX x TY cells over kTransRun planes,
 // and (kperm != null) the adjoint's copy of k.  Per plane the tile's
-// reciprocals with the cells its links reach (x - 1 .. x + 32, y .. y + 8) sit
+// reciprocals with the cells its links reach (one more row above, one more
+// column on each side) sit
 // in shared memory: 1.2 per cell instead of six.  Measured from ln k with the
 // copy of k (a kernel of its own before): mixed 128^3 704 -> 42 us, FP64
 // 97 x 83 x 50 144 -> 87 us (bound by the FP64 pipe: 1.5 exponentials and five
 // quotients per cell).  Runs of 8 planes instead of 4 measured the same on the
 // mixed path and 7 % slower in FP64 (fewer blocks).
 template <typename Real, bool LOG>
-__global__ void __launch_bounds__(kTx* kTy) k_trans(GridGeom g, Geo geo, const double* __restrict__ perm, Real* Tx,
-                                                    Real* Ty, Real* Tz, Real* Tpp, Real* Tmp, Real* kperm) {
+__global__ void __launch_bounds__(kTileThreads)
+    k_trans(GridGeom g, Geo geo, int TX, int TY, const double* __restrict__ perm, Real* Tx, Real* Ty, Real* Tz,
+            Real* Tpp, Real* Tmp, Real* kperm) {
     using R = Tile<Real>;
     using RT = typename R::type;
-    constexpr int PX = kTx + 2, PY = kTy + 1;
-    __shared__ RT tile[2][PY][PX];
+    // (TX + 2)(TY + 1) with TX TY <= 256 and TX <= 128 is at most 3 * 257
+    constexpr int kPlane = 3 * (kTileThreads + 1);
+    __shared__ RT tile[2][kPlane];
     __shared__ float2 eighth[8];
-    const int tx = threadIdx.x, ty = threadIdx.y, t = tx + kTx * ty;
+    const int PX = TX + 2;
+    const int t = threadIdx.x, nt = blockDim.x;
+    const bool in = t < TX * TY;
+    const int ty = in ? t / TX : 0, tx = in ? t - ty * TX : 0;
     if (sizeof(Real) == 4 && LOG && t < 8) {
         const float h = (float)kEighth[t];
         eighth[t] = make_float2(h, (float)(kEighth[t] - (double)h));
@@ -233,30 +240,30 @@ __global__ void __launch_bounds__(kTx* kTy) k_trans(GridGeom g, Geo geo, const d
     if (sizeof(Real) == 4 && LOG) __syncthreads();
     const int nx = g.nx, ny = g.ny;
     const long long nxy = (long long)nx * ny;
-    const unsigned bx = (unsigned)(nx + kTx - 1) / kTx, by = (unsigned)(ny + kTy - 1) / kTy;
+    const unsigned bx = (unsigned)(nx + TX - 1) / TX, by = (unsigned)(ny + TY - 1) / TY;
     const unsigned bt = blockIdx.x / bx;
-    const int i0 = (int)(blockIdx.x - bt * bx) * kTx, j0 = (int)(bt % by) * kTy;
+    const int i0 = (int)(blockIdx.x - bt * bx) * TX, j0 = (int)(bt % by) * TY;
     const int i = i0 + tx, j = j0 + ty;
-    const bool act = i < nx && j < ny;
+    const bool act = in && i < nx && j < ny;
     // in-range cell of tile position (x, y), x = 0 the cell left of the tile
     auto cell = [&](int x, int y) {
         const int ci = min(max(i0 + x - 1, 0), nx - 1), cj = min(j0 + y, ny - 1);
         return ci + (long long)nx * cj;
     };
     const long long own = cell(tx + 1, ty);
-    // the tile's other cells: the row above (34) and the columns left and right (8 each)
-    const bool edge = t < PX + 2 * kTy;
-    const int ex = t < PX ? t : (t - PX < kTy ? 0 : PX - 1);
-    const int ey = t < PX ? kTy : (t - PX) % kTy;
-    const long long ecell = cell(ex, ey);
+    const int sp = ty * PX + tx + 1;
     const int k0 = (int)(bt / by) * kTransRun, k1 = min(k0 + kTransRun, g.nz);
     double vc = R::template pre<LOG>(perm[own + nxy * k0]);  // own k (FP64 path) or the stored value
     RT rc = R::template of<LOG>(vc, eighth);
     for (int k = k0; k < k1; ++k) {
-        auto& P = tile[(k - k0) & 1];
+        RT* const P = tile[(k - k0) & 1];
         const long long base = nxy * k;
-        P[ty][tx + 1] = rc;
-        if (edge) P[ey][ex] = R::template of<LOG>(R::template pre<LOG>(perm[base + ecell]), eighth);
+        if (in) P[sp] = rc;
+        // the row above and the columns left and right of the tile
+        for (int h = t; h < PX + 2 * TY; h += nt) {
+            const int x = h < PX ? h : (((h - PX) & 1) ? PX - 1 : 0), y = h < PX ? TY : (h - PX) / 2;
+            P[y * PX + x] = R::template of<LOG>(R::template pre<LOG>(perm[base + cell(x, y)]), eighth);
+        }
         const bool zp = k + 1 < g.nz;
         const double vn = zp ? R::template pre<LOG>(perm[base + nxy + own]) : vc;
         const RT rn = zp ? R::template of<LOG>(vn, eighth) : rc;
@@ -270,13 +277,13 @@ __global__ void __launch_bounds__(kTx* kTy) k_trans(GridGeom g, Geo geo, const d
         };
         if (act) {
             const bool xp = i + 1 < nx, yp = j + 1 < ny;
-            put(Tx, xp, P[ty][tx + 2], geo.px, geo.ax, xp ? c + 1 : c);
-            put(Ty, yp, P[ty + 1][tx + 1], geo.py, geo.ay, yp ? c + nx : c);
+            put(Tx, xp, P[sp + 1], geo.px, geo.ax, xp ? c + 1 : c);
+            put(Ty, yp, P[sp + PX], geo.py, geo.ay, yp ? c + nx : c);
             put(Tz, zp, rn, geo.pz, geo.az, zp ? c + nxy : c);
             if (g.diag) {
                 const bool pp = yp && xp, mp = yp && i > 0;
-                put(Tpp, pp, P[ty + 1][tx + 2], geo.pd, geo.ad, pp ? c + nx + 1 : c);
-                put(Tmp, mp, P[ty + 1][tx], geo.pd, geo.ad, mp ? c + nx - 1 : c);
+                put(Tpp, pp, P[sp + PX + 1], geo.pd, geo.ad, pp ? c + nx + 1 : c);
+                put(Tmp, mp, P[sp + PX - 1], geo.pd, geo.ad, mp ? c + nx - 1 : c);
             }
             if (kperm) {
                 Real kv;
@@ -382,11 +389,14 @@ template <typename Real>
 static cudaError_t launch_trans_t(const GridGeom& g, const SetupPhys& s, const double* perm, Real* Tx, Real* Ty,
                                   Real* Tz, Real* Tpp, Real* Tmp, Real* kperm, cudaStream_t st, bool log_k) {
     // one block index for tiles and z-runs: any grid shape of fewer than 2^31 cells fits
-    const long long nb = (long long)((g.nx + kTx - 1) / kTx) * ((g.ny + kTy - 1) / kTy) *
+    int TX = 1, TY = 1;
+    tile_shape(g.nx, g.ny, kTileThreads, TX, TY);
+    const long long nb = (long long)((g.nx + TX - 1) / TX) * ((g.ny + TY - 1) / TY) *
                          ((g.nz + kTransRun - 1) / kTransRun);
-    const dim3 block(kTx, kTy, 1);
-    if (log_k) k_trans<Real, true><<<(unsigned)nb, block, 0, st>>>(g, make_geo(s), perm, Tx, Ty, Tz, Tpp, Tmp, kperm);
-    else k_trans<Real, false><<<(unsigned)nb, block, 0, st>>>(g, make_geo(s), perm, Tx, Ty, Tz, Tpp, Tmp, kperm);
+    const int block = (TX * TY + 31) / 32 * 32;
+    const Geo q = make_geo(s);
+    if (log_k) k_trans<Real, true><<<(unsigned)nb, block, 0, st>>>(g, q, TX, TY, perm, Tx, Ty, Tz, Tpp, Tmp, kperm);
+    else k_trans<Real, false><<<(unsigned)nb, block, 0, st>>>(g, q, TX, TY, perm, Tx, Ty, Tz, Tpp, Tmp, kperm);
     return cudaGetLastError();
 }
 

@@ -167,12 +167,12 @@ extern "C" int tpfa_assemble_jacobian_static(int nx, int ny, int nz, const tpfa_
                                             (double*)T[3], (double*)T[4], nullptr, st);
         if (e == cudaSuccess) e = launch_prev_mass_f64(sp, (const double*)p_prev_dev, poro_dev, mn, N, st);
         if (e == cudaSuccess) {
-            const PhysD q{prm->rho_ref, prm->p_ref, prm->c_f, 1.0 / prm->mu, prm->g, 0.5 * prm->g, V_dt, prm->c_r};
+            const PhysD q = make_phys_d(prm->rho_ref, prm->p_ref, prm->c_f, prm->mu, prm->g, V_dt, prm->c_r);
             AsmFields<double> f{(const double*)p_dev, (const double*)p_prev_dev, mn, depth_dev, poro_dev,
                                 (const double*)T[0], (const double*)T[1], (const double*)T[2],
                                 (const double*)(T[3] ? T[3] : T[0]), (const double*)(T[4] ? T[4] : T[0])};
             AsmOut<double> o{R_dev, (double*)vals_dev, nullptr, status};
-            e = launch_assemble_fp64(AsmKernel::YMarch, g, q, crk, f, o, 32, 4, st);
+            e = launch_assemble_fp64(AsmKernel::YMarch, g, q, crk, f, o, st);
         }
     }
     if (e != cudaSuccess) return report_error(TPFA_ERR_CUDA, cudaGetErrorString(e));

@@ -14,9 +14,7 @@
 // the forward assembly and this pass: densities, upwind choices and
 // mobilities are recomputed (gather form, no atomics).
 //
-// FP64 path: links, sums and outputs in FP64, one thread per cell.
-//
-// Mixed path: with dF_Li/dp_i = -dF_iL/dp_i except at an exact tie, and
+// The FP64 path's adjoint is in tpfa_fp64.cu.  Mixed path: with dF_Li/dp_i = -dF_iL/dp_i except at an exact tie, and
 // k_L / (k_i + k_L) = Upsilon_iL (d/A)_iL / (2 k_i) for the harmonic
 // two-point transmissibility,
 //   g_p[i]   = v_i dA_i/dp_i + sum_L dF_iL/dp_i (v_i - v_L) + sum_L v_L delta_iL
@@ -51,82 +49,6 @@ __device__ __forceinline__ T ld_chk(const T* p, long long idx, long long N, unsi
         return T{};
     }
     return __ldg(p + idx);
-}
-
-template <typename Real>
-__device__ __forceinline__ double to_f64(Real x) {
-    if constexpr (sizeof(Real) == 4) return widen(x);
-    else return x;
-}
-
-template <typename Real, bool CRK>
-__global__ void __launch_bounds__(256) k_vjp(GridGeom g, typename PhysOf<Real>::type q, AsmFields<Real> f,
-                                             const Real* __restrict__ kperm, const double* __restrict__ v,
-                                             double* __restrict__ g_p, double* __restrict__ g_lnk,
-                                             unsigned int* status) {
-    const int i = blockIdx.x * 32 + threadIdx.x;
-    const int j = blockIdx.y * 8 + threadIdx.y;
-    const int k = blockIdx.z;
-    if (i >= g.nx || j >= g.ny) return;
-    const int nx = g.nx, nxy = nx * g.ny;
-    const int c = i + nx * j + nxy * k;
-    const long long NN = (long long)nxy * g.nz;
-    const unsigned mask = slot_mask(g, i, j, k);
-    const int off[NSLOT] = {-nxy, -nx - 1, -nx, -nx + 1, -1, 0, 1, nx - 1, nx, nx + 1, nxy};
-    const CellVal<Real> me = make_cell(q, ld_chk(f.p, c, NN, status), ld_chk(f.z, c, NN, status));
-    const double vi = ld_chk(v, c, NN, status);
-    const Real ki = ld_chk(kperm, c, NN, status);
-    double diag = 0.0, offs = 0.0, glnk = 0.0;
-#pragma unroll
-    for (int s = 0; s < NSLOT; ++s) {
-        if (s == SLOT_SELF) continue;
-        const bool valid = (mask & (1u << s)) != 0;
-        // invalid slots keep an in-range index (the cell itself), so a load
-        // scheduled ahead of the guard still reads inside the arrays
-        const int d = valid ? c + off[s] : c;
-        if (!valid) continue;
-        const Real* Tp;
-        int ti;
-        switch (s) {
-            case 0: Tp = f.Tz; ti = d; break;
-            case 1: Tp = f.Tpp; ti = d; break;
-            case 2: Tp = f.Ty; ti = d; break;
-            case 3: Tp = f.Tmp; ti = d; break;
-            case 4: Tp = f.Tx; ti = d; break;
-            case 6: Tp = f.Tx; ti = c; break;
-            case 7: Tp = f.Tmp; ti = c; break;
-            case 8: Tp = f.Ty; ti = c; break;
-            case 9: Tp = f.Tpp; ti = c; break;
-            default: Tp = f.Tz; ti = c; break;
-        }
-        const Real T = ld_chk(Tp, ti, NN, status);
-        const CellVal<Real> nb = make_cell(q, ld_chk(f.p, d, NN, status), ld_chk(f.z, d, NN, status));
-        const LinkOut<Real> L = link(q, T, me, nb);
-        // row L's derivative with respect to p_i
-        const Real dLi = (L.F == Real(0) && T != Real(0)) ? link(q, T, nb, me).Db : -L.Da;
-        const double vl = ld_chk(v, d, NN, status);
-        const Real kl = ld_chk(kperm, d, NN, status);
-        diag += to_f64(L.Da);
-        offs = fma(vl, to_f64(dLi), offs);
-        const Real ratio = (ki + kl) > Real(0) ? kl / (ki + kl) : Real(0);
-        glnk = fma(vi - vl, to_f64(L.F) * to_f64(ratio), glnk);
-    }
-    Real pn = ld_chk(f.pn, c, NN, status);
-    if constexpr (sizeof(Real) == 4) {
-        const AccF acc = accumulation<CRK>(q, me.p, pn, ld_chk(f.mn, c, NN, status), me.rho, CRK ? ld_chk(f.phi0, c, NN, status) : 0.f);
-        diag += widen(acc.dA);
-    } else {
-        const AccD acc = accumulation<CRK>(q, me.p, pn, ld_chk(f.mn, c, NN, status), me.rho, CRK ? ld_chk(f.phi0, c, NN, status) : 0.0);
-        diag += acc.dA;
-    }
-    const double gp = fma(vi, diag, offs);
-    if (c < 0 || c >= NN || g_p == nullptr) {
-        atomicOr(status, STATUS_DEVICE_CHECK);
-        return;
-    }
-    g_p[c] = gp;
-    if (g_lnk) g_lnk[c] = glnk;
-    if (nonfinite(gp) || nonfinite(glnk)) atomicOr(status, STATUS_NONFINITE);
 }
 
 __device__ __forceinline__ float geo_of(const LinkGeo& lg, int s) {
@@ -216,7 +138,7 @@ __global__ void __launch_bounds__(256) k_vjp_mixed(GridGeom g, PhysF q, AsmField
 
 template <int W>
 constexpr int vjp_smem_bytes() {
-    using M = YMarch<float, true, false, false, W, false, true>;
+    using M = YMarch<true, false, false, W, false, true>;
     return W * (M::RING * M::NF * 32 * 4 + M::RING * 32 * 8 + M::RING * M::NW * 32 * 8);
 }
 
@@ -225,7 +147,7 @@ __global__ void __launch_bounds__(32 * W, 16 / W)
     k_vjp_ymarch(GridGeom g, PhysF q, AsmFields<float> f, AsmOut<float> o, const float* __restrict__ kperm,
                  LinkGeo lg, const float2* __restrict__ v, double* __restrict__ g_p, double* __restrict__ g_lnk,
                  int JY) {
-    using M_t = YMarch<float, DIAG, CRK, false, W, false, true>;
+    using M_t = YMarch<DIAG, CRK, false, W, false, true>;
     extern __shared__ __align__(16) unsigned char smem[];
     const int lane = threadIdx.x, wi = threadIdx.y;
     const int k = blockIdx.z * W + wi;
@@ -252,27 +174,27 @@ __global__ void __launch_bounds__(32 * W, 16 / W)
     M.issue_row(j0, 1);
     M.issue_row(j0 + 1, 2);
     M.wait_all_but_newest();
-    YRow<float> P = M.row_cells(0);
-    YRow<float> C = M.row_cells(1);
+    YRow P = M.row_cells(0);
+    YRow C = M.row_cells(1);
     YV vP = M.v_row(0);
     YV vC = M.v_row(1);
     float Ty_prev, Tpp_prev, Tmp_prev;
     {
-        const YIn<float> Dp = M.read_in(0);
+        const YIn Dp = M.read_in(0);
         Ty_prev = Dp.Ty;
         Tpp_prev = Dp.Tpp;
         Tmp_prev = Dp.Tmp;
     }
-    YUp<float> U = M.up_links(P, C, Ty_prev, Tpp_prev, Tmp_prev);
+    YUp U = M.up_links(P, C, Ty_prev, Tpp_prev, Tmp_prev);
     int s0 = 1, s1 = 2, s2 = 0;  // ring slots of rows j, j+1, j+2
     unsigned long long fix_rows = 0ull;  // rows with a zero flux, recomputed after the march
 
     for (int j = j0; j < j1; ++j) {
         M.issue_row(j + 2, s2);
         M.wait_all_but_newest();
-        const YRow<float> N = M.row_cells(s1);
+        const YRow N = M.row_cells(s1);
         const YV vN = M.v_row(s1);
-        const YIn<float> D = M.read_in(s0);
+        const YIn D = M.read_in(s0);
         const F2Split vzm = M.v_at(s0, 2), vzp = M.v_at(s0, 3);
         const float kC = ring[s0 * (M_t::NF * 32) + M_t::F_K * 32 + lane];
         const int st = s0;
@@ -398,17 +320,6 @@ bool aligned(const void* p, uintptr_t a) { return (reinterpret_cast<uintptr_t>(p
 
 }  // namespace
 
-template <typename Real>
-static cudaError_t launch_vjp_t(const GridGeom& g, const typename PhysOf<Real>::type& q, bool crk,
-                                const AsmFields<Real>& f, const Real* kperm, const double* v, double* g_p,
-                                double* g_lnk, unsigned int* status, cudaStream_t st) {
-    dim3 block(32, 8, 1);
-    dim3 grid((g.nx + 31) / 32, (g.ny + 7) / 8, g.nz);
-    if (crk) k_vjp<Real, true><<<grid, block, 0, st>>>(g, q, f, kperm, v, g_p, g_lnk, status);
-    else k_vjp<Real, false><<<grid, block, 0, st>>>(g, q, f, kperm, v, g_p, g_lnk, status);
-    return cudaGetLastError();
-}
-
 // The cotangent as FP32 pairs: v = hi + lo with hi the truncation of v and lo
 // the remainder truncated (F2Split), one pair per cell.
 __global__ void k_split_pairs(const double* __restrict__ v, float2* __restrict__ out, long long n) {
@@ -450,12 +361,6 @@ cudaError_t launch_vjp_mixed(AsmKernel kern, const GridGeom& g, const PhysF& q, 
     }
     return crk ? launch_vjp_ymarch_t<false, true>(g, q, f, kperm, lg, v, g_p, g_lnk, status, JY, W, st)
                : launch_vjp_ymarch_t<false, false>(g, q, f, kperm, lg, v, g_p, g_lnk, status, JY, W, st);
-}
-
-cudaError_t launch_vjp_fp64(const GridGeom& g, const PhysD& q, bool crk, const AsmFields<double>& f,
-                            const double* kperm, const double* v, double* g_p, double* g_lnk,
-                            unsigned int* status, cudaStream_t st) {
-    return launch_vjp_t<double>(g, q, crk, f, kperm, v, g_p, g_lnk, status, st);
 }
 
 }  // namespace tpfa

@@ -1,4 +1,4 @@
-// tpfa_ymarch.cuh -- the production assembly kernel (sm_103a).
+// tpfa_ymarch.cuh -- the mixed path's one-cell assembly march (sm_103a).
 //
 // A warp owns a 32-cell x-segment (cells i0 .. i0+31) of one z-plane k and
 // marches along y over a run of JY rows; a block stacks W warps on W
@@ -48,45 +48,38 @@
 
 namespace tpfa {
 
-template <typename Real>
 struct YRow {
-    CellVal<Real> c, m, p;  // cells (i, j), (i-1, j), (i+1, j) of this lane
+    CellVal<float> c, m, p;  // cells (i, j), (i-1, j), (i+1, j) of this lane
 };
 
-template <typename Real>
 struct YIn {  // inputs of one row other than p and z
-    Real Tx, Ty, Tz, Tpp, Tmp, pn, phi0;
+    float Tx, Ty, Tz, Tpp, Tmp, pn, phi0;
     double mn;
-    Real p_zm, z_zm, p_zp, z_zp, Tz_m;
-    Real hT1, hT2;  // lane 0: Tx(i0-1, j), Tpp(i0-1, j-1); lane 31: Tmp(i0+32, j-1)
+    float p_zm, z_zm, p_zp, z_zp, Tz_m;
+    float hT1, hT2;  // lane 0: Tx(i0-1, j), Tpp(i0-1, j-1); lane 31: Tmp(i0+32, j-1)
 };
 
-template <typename Real>
 struct YUp {  // a link from row j-1 into row j, seen from row j-1
-    LinkOut<Real> y, xy, mxy;  // to (i, j), (i+1, j), (i-1, j)
+    LinkOut<float> y, xy, mxy;  // to (i, j), (i+1, j), (i-1, j)
     bool tie;                  // any of the three had dPhi == 0 exactly
 };
 
-template <typename Real>
-__device__ __forceinline__ Real vshfl_up(Real v) {
+__device__ __forceinline__ float vshfl_up(float v) {
     return __shfl_up_sync(0xffffffffu, v, 1);
 }
-template <typename Real>
-__device__ __forceinline__ Real vshfl_down(Real v) {
+__device__ __forceinline__ float vshfl_down(float v) {
     return __shfl_down_sync(0xffffffffu, v, 1);
 }
 
 __device__ __forceinline__ float drho_of(const PhysF& q, float rho) { return __fmul_rn(q.c_f, rho); }
-__device__ __forceinline__ double drho_of(const PhysD& q, double rho) { return __dmul_rn(q.c_f, rho); }
 
 // A link and whether it may be an exact tie: dPhi == 0 forces F == 0, so
 // F == 0 on a link with T != 0 flags every tie (and, harmlessly, fluxes that
 // underflow to zero).
-template <typename Real, typename Phys>
-__device__ __forceinline__ LinkOut<Real> link_t(const Phys& q, Real T, const CellVal<Real>& a,
-                                                const CellVal<Real>& b, bool& tie) {
-    const LinkOut<Real> r = link(q, T, a, b);
-    tie = (r.F == Real(0)) && (T != Real(0));
+__device__ __forceinline__ LinkOut<float> link_t(const PhysF& q, float T, const CellVal<float>& a,
+                                                 const CellVal<float>& b, bool& tie) {
+    const LinkOut<float> r = link(q, T, a, b);
+    tie = (r.F == 0.f) && (T != 0.f);
     return r;
 }
 
@@ -103,17 +96,16 @@ struct YV {
     F2Split c, h;
 };
 
-template <typename Real, bool DIAG, bool CRK, bool JAC, int W, bool JV = false, bool VJ = false>
+template <bool DIAG, bool CRK, bool JAC, int W, bool JV = false, bool VJ = false>
 struct YMarch {
-    static_assert(!JV || (sizeof(Real) == 4 && !JAC), "the J w march is the mixed path's, without CSR values");
-    static_assert(!VJ || (sizeof(Real) == 4 && !JAC && !JV), "the adjoint march is the mixed path's");
-    using Phys = typename PhysOf<Real>::type;
-    static constexpr int VEC = 16 / (int)sizeof(Real);  // elements per 16-byte store
+    static_assert(!JV || !JAC, "the J w march writes no CSR values");
+    static_assert(!VJ || (!JAC && !JV), "the adjoint march writes no CSR values");
+    static constexpr int VEC = 4;  // elements per 16-byte store
 
     const GridGeom& g;
-    const Phys& q;
-    const AsmFields<Real>& f;
-    const AsmOut<Real>& o;
+    const PhysF& q;
+    const AsmFields<float>& f;
+    const AsmOut<float>& o;
     int lane, i0, i, k, nx, ny, nxy, kb, ih;
     bool act, hact, zm, zp, xint, v16;
     long long base_k;
@@ -121,8 +113,8 @@ struct YMarch {
     int X2;          // offset of this segment within a y-row whose j and k are interior
     int Sx0, ez;
 
-    __device__ __forceinline__ YMarch(const GridGeom& g_, const Phys& q_, const AsmFields<Real>& f_,
-                                      const AsmOut<Real>& o_, int lane_, int i0_, int k_)
+    __device__ __forceinline__ YMarch(const GridGeom& g_, const PhysF& q_, const AsmFields<float>& f_,
+                                      const AsmOut<float>& o_, int lane_, int i0_, int k_)
         : g(g_), q(q_), f(f_), o(o_), lane(lane_), i0(i0_), i(i0_ + lane_), k(k_) {
         nx = g.nx;
         ny = g.ny;
@@ -183,7 +175,7 @@ struct YMarch {
     enum { F_P, F_Z, F_HP, F_HZ, F_TX, F_TY, F_TZ, F_TPP, F_TMP, F_PN, F_PHI, F_PZM, F_ZZM, F_TZM, F_PZP, F_ZZP,
            F_HT1, F_HT2, F_K };
     static constexpr int NF = VJ ? F_K + 1 : F_K;  // the adjoint also prefetches the cell's k
-    Real* ring;      // RING * NF * 32 values
+    float* ring;      // RING * NF * 32 values
     double* ringm;   // RING * 32 values of m^n
     // J w mode: RING * NW * 32 values of w (own, halo, z-1, z+1), the
     // direction w and the output
@@ -192,18 +184,14 @@ struct YMarch {
     const double* wv = nullptr;
     double* Jw = nullptr;
     // adjoint mode: k of the field type, the link geometry, the two gradients
-    const Real* kperm = nullptr;
+    const float* kperm = nullptr;
     LinkGeo lg{};
     double* gP = nullptr;
     double* gK = nullptr;
 
-    __device__ __forceinline__ void cp4(Real* dst, const Real* src, bool valid) const {
+    __device__ __forceinline__ void cp4(float* dst, const float* src, bool valid) const {
         const uint32_t d = (uint32_t)__cvta_generic_to_shared(dst);
-        const int n = valid ? (int)sizeof(Real) : 0;
-        if constexpr (sizeof(Real) == 4)
-            asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(d), "l"(src), "r"(n) : "memory");
-        else
-            asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"(d), "l"(src), "r"(n) : "memory");
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(d), "l"(src), "r"(valid ? 4 : 0) : "memory");
     }
     __device__ __forceinline__ void cp8(double* dst, const double* src, bool valid) const {
         const uint32_t d = (uint32_t)__cvta_generic_to_shared(dst);
@@ -212,7 +200,7 @@ struct YMarch {
     // Request every input of row r into ring slot sl (a row outside the grid
     // requests nothing).
     __device__ __forceinline__ void issue_row(int r, int sl) const {
-        Real* R = ring + sl * (NF * 32) + lane;
+        float* R = ring + sl * (NF * 32) + lane;
         const bool rv = r >= 0 && r < ny;
         const int c = kb + nx * (rv ? r : 0) + (act ? i : 0);
         const bool a = rv && act;
@@ -257,16 +245,16 @@ struct YMarch {
     __device__ __forceinline__ void wait_all_but_newest() const {
         asm volatile("cp.async.wait_group 1;" ::: "memory");
     }
-    __device__ __forceinline__ YIn<Real> read_in(int sl) const {
-        const Real* R = ring + sl * (NF * 32) + lane;
-        YIn<Real> D;
+    __device__ __forceinline__ YIn read_in(int sl) const {
+        const float* R = ring + sl * (NF * 32) + lane;
+        YIn D;
         D.Tx = R[F_TX * 32];
         D.Ty = R[F_TY * 32];
         D.Tz = R[F_TZ * 32];
-        D.Tpp = DIAG ? R[F_TPP * 32] : Real(0);
-        D.Tmp = DIAG ? R[F_TMP * 32] : Real(0);
+        D.Tpp = DIAG ? R[F_TPP * 32] : 0.f;
+        D.Tmp = DIAG ? R[F_TMP * 32] : 0.f;
         D.pn = R[F_PN * 32];
-        D.phi0 = CRK ? R[F_PHI * 32] : Real(0);
+        D.phi0 = CRK ? R[F_PHI * 32] : 0.f;
         D.mn = ringm[sl * 32 + lane];
         D.p_zm = R[F_PZM * 32];
         D.z_zm = R[F_ZZM * 32];
@@ -274,11 +262,11 @@ struct YMarch {
         D.p_zp = R[F_PZP * 32];
         D.z_zp = R[F_ZZP * 32];
         D.hT1 = R[F_HT1 * 32];
-        D.hT2 = DIAG ? R[F_HT2 * 32] : Real(0);
+        D.hT2 = DIAG ? R[F_HT2 * 32] : 0.f;
         return D;
     }
-    __device__ __forceinline__ YRow<Real> row_cells(int sl) const {
-        const Real* R = ring + sl * (NF * 32) + lane;
+    __device__ __forceinline__ YRow row_cells(int sl) const {
+        const float* R = ring + sl * (NF * 32) + lane;
         return make_row(R[F_P * 32], R[F_Z * 32], R[F_HP * 32], R[F_HZ * 32]);
     }
 
@@ -373,7 +361,7 @@ struct YMarch {
     __device__ __forceinline__ const float* tma_slot(int sl) const {
         return reinterpret_cast<const float*>(tring + sl * TS::BYTES);
     }
-    __device__ __forceinline__ YRow<Real> tma_row_cells(int sl) const {
+    __device__ __forceinline__ YRow tma_row_cells(int sl) const {
         const float* S = tma_slot(sl);
         constexpr int P1 = TS::P / 4 + TS::HX, Z1 = TS::Z / 4 + TS::HX;  // plane k
         return make_row(S[P1 + xo + 4 + lane], S[Z1 + xo + 4 + lane], S[P1 + hx], S[Z1 + hx]);
@@ -381,31 +369,31 @@ struct YMarch {
     // The diagonal-link T of lanes 0 and 31 into row r - 1 (Tpp(i0 - 1, r - 1)
     // and Tmp(i0 + 32, r - 1)), read from the slot of row r - 1 before it is
     // refilled; 0 in the other lanes.
-    __device__ __forceinline__ Real tma_h2(int sl) const {
-        if (!DIAG) return Real(0);
+    __device__ __forceinline__ float tma_h2(int sl) const {
+        if (!DIAG) return 0.f;
         const float* S = tma_slot(sl);
         const float t = lane == 31 ? S[TS::TMP / 4 + xo + 36] : S[TS::TPP / 4 + xo + 3];
         return (lane == 0 || lane == 31) ? t : 0.f;
     }
-    __device__ __forceinline__ YIn<Real> tma_read_in(int sl, Real hT2) const {
+    __device__ __forceinline__ YIn tma_read_in(int sl, float hT2) const {
         const float* S = tma_slot(sl);
         constexpr int P0 = TS::P / 4, Z0 = TS::Z / 4, B = TS::HX;
         const int o = xo + lane, oh = o + 4;  // the lane's cell in a plain box row and in a halo box row
-        YIn<Real> D;
+        YIn D;
         D.Tx = S[TS::TX / 4 + oh];
         D.Ty = S[TS::TY / 4 + o];
         D.Tz = S[TS::TZ / 4 + TS::SX + o];
-        D.Tpp = DIAG ? S[TS::TPP / 4 + oh] : Real(0);
-        D.Tmp = DIAG ? S[TS::TMP / 4 + oh] : Real(0);
+        D.Tpp = DIAG ? S[TS::TPP / 4 + oh] : 0.f;
+        D.Tmp = DIAG ? S[TS::TMP / 4 + oh] : 0.f;
         D.pn = S[TS::PN / 4 + o];
-        D.phi0 = CRK ? S[TS::PHI / 4 + o] : Real(0);
+        D.phi0 = CRK ? S[TS::PHI / 4 + o] : 0.f;
         D.mn = reinterpret_cast<const double*>(tring + sl * TS::BYTES + TS::MN)[o];
         D.p_zm = S[P0 + oh];
         D.z_zm = S[Z0 + oh];
         D.Tz_m = S[TS::TZ / 4 + o];
         D.p_zp = S[P0 + 2 * B + oh];
         D.z_zp = S[Z0 + 2 * B + oh];
-        D.hT1 = lane == 0 ? S[TS::TX / 4 + xo + 3] : Real(0);  // Tx(i0 - 1, r)
+        D.hT1 = lane == 0 ? S[TS::TX / 4 + xo + 3] : 0.f;  // Tx(i0 - 1, r)
         D.hT2 = hT2;
         return D;
     }
@@ -441,10 +429,10 @@ struct YMarch {
         return lane == 31 ? v.h : t;
     }
 
-    __device__ __forceinline__ YRow<Real> make_row(Real po, Real zo, Real ph, Real zh) const {
-        YRow<Real> R;
+    __device__ __forceinline__ YRow make_row(float po, float zo, float ph, float zh) const {
+        YRow R;
         R.c = make_cell(q, po, zo);
-        const CellVal<Real> h = make_cell(q, ph, zh);
+        const CellVal<float> h = make_cell(q, ph, zh);
         R.m.p = vshfl_up(R.c.p);
         R.m.z = vshfl_up(R.c.z);
         R.m.rho = vshfl_up(R.c.rho);
@@ -458,9 +446,9 @@ struct YMarch {
         return R;
     }
     // Links from row r into row r+1, seen from row r (cells of rows r and r+1).
-    __device__ __forceinline__ YUp<Real> up_links(const YRow<Real>& R, const YRow<Real>& Nx, Real Ty, Real Tpp,
-                                                  Real Tmp) const {
-        YUp<Real> U;
+    __device__ __forceinline__ YUp up_links(const YRow& R, const YRow& Nx, float Ty, float Tpp,
+                                                  float Tmp) const {
+        YUp U;
         bool t0, t1 = false, t2 = false;
         U.y = link_t(q, Ty, R.c, Nx.c, t0);
         if (DIAG) {
@@ -476,60 +464,47 @@ struct YMarch {
     // the previous step's, exact except at a tie dPhi == 0 (where each end
     // takes the other cell as upstream): U.tie flags those, and the marches
     // recompute the affected rows afterwards.
-    __device__ __forceinline__ void eval_links(const YRow<Real>& P, const YRow<Real>& C, const YRow<Real>& N,
-                                               const YIn<Real>& D, const YUp<Real>& Uprev,
-                                               LinkOut<Real> (&S)[NSLOT], YUp<Real>& U) const {
-        Real Tx_m = vshfl_up(D.Tx);
+    __device__ __forceinline__ void eval_links(const YRow& P, const YRow& C, const YRow& N,
+                                               const YIn& D, const YUp& Uprev,
+                                               LinkOut<float> (&S)[NSLOT], YUp& U) const {
+        float Tx_m = vshfl_up(D.Tx);
         if (lane == 0) Tx_m = D.hT1;
-        const CellVal<Real> zmc = make_cell(q, D.p_zm, D.z_zm);
-        const CellVal<Real> zpc = make_cell(q, D.p_zp, D.z_zp);
+        const CellVal<float> zmc = make_cell(q, D.p_zm, D.z_zm);
+        const CellVal<float> zpc = make_cell(q, D.p_zp, D.z_zp);
 
         // slot order: 0 (0,0,-1) 1 (-1,-1) 2 (0,-1) 3 (+1,-1) 4 (-1,0) 5 self
         //             6 (+1,0) 7 (-1,+1) 8 (0,+1) 9 (+1,+1) 10 (0,0,+1)
-        LinkOut<Real> E;  // lane 0: its (-1,-1) link; lane 31: its (+1,-1) link
-        if constexpr (sizeof(Real) == 4) {
-            // eight links as four FP32x2 pairs
-            const Link2 x = link2(q, f2(Tx_m, D.Tx), C.c, C.m, C.p);
-            const Link2 yz = link2(q, f2(D.Ty, D.Tz), C.c, N.c, zpc);
-            S[4] = LinkOut<float>{x.F.x, x.Da.x, x.Db.x};
-            S[6] = LinkOut<float>{x.F.y, x.Da.y, x.Db.y};
-            S[8] = LinkOut<float>{yz.F.x, yz.Da.x, yz.Db.x};
-            S[10] = LinkOut<float>{yz.F.y, yz.Da.y, yz.Db.y};
-            if (DIAG) {
-                const Link2 d = link2(q, f2(D.Tmp, D.Tpp), C.c, N.m, N.p);
-                const Link2 ze = link2(q, f2(D.Tz_m, D.hT2), C.c, zmc, lane == 0 ? P.m : P.p);
-                S[7] = LinkOut<float>{d.F.x, d.Da.x, d.Db.x};
-                S[9] = LinkOut<float>{d.F.y, d.Da.y, d.Db.y};
-                S[0] = LinkOut<float>{ze.F.x, ze.Da.x, ze.Db.x};
-                E = LinkOut<float>{ze.F.y, ze.Da.y, ze.Db.y};
-            } else {
-                S[0] = link(q, D.Tz_m, C.c, zmc);
-            }
+        LinkOut<float> E;  // lane 0: its (-1,-1) link; lane 31: its (+1,-1) link
+        // eight links as four FP32x2 pairs
+        const Link2 x = link2(q, f2(Tx_m, D.Tx), C.c, C.m, C.p);
+        const Link2 yz = link2(q, f2(D.Ty, D.Tz), C.c, N.c, zpc);
+        S[4] = LinkOut<float>{x.F.x, x.Da.x, x.Db.x};
+        S[6] = LinkOut<float>{x.F.y, x.Da.y, x.Db.y};
+        S[8] = LinkOut<float>{yz.F.x, yz.Da.x, yz.Db.x};
+        S[10] = LinkOut<float>{yz.F.y, yz.Da.y, yz.Db.y};
+        if (DIAG) {
+            const Link2 d = link2(q, f2(D.Tmp, D.Tpp), C.c, N.m, N.p);
+            const Link2 ze = link2(q, f2(D.Tz_m, D.hT2), C.c, zmc, lane == 0 ? P.m : P.p);
+            S[7] = LinkOut<float>{d.F.x, d.Da.x, d.Db.x};
+            S[9] = LinkOut<float>{d.F.y, d.Da.y, d.Db.y};
+            S[0] = LinkOut<float>{ze.F.x, ze.Da.x, ze.Db.x};
+            E = LinkOut<float>{ze.F.y, ze.Da.y, ze.Db.y};
         } else {
             S[0] = link(q, D.Tz_m, C.c, zmc);
-            S[4] = link(q, Tx_m, C.c, C.m);
-            S[6] = link(q, D.Tx, C.c, C.p);
-            S[8] = link(q, D.Ty, C.c, N.c);
-            S[10] = link(q, D.Tz, C.c, zpc);
-            if (DIAG) {
-                S[7] = link(q, D.Tmp, C.c, N.m);
-                S[9] = link(q, D.Tpp, C.c, N.p);
-                E = link(q, D.hT2, C.c, lane == 0 ? P.m : P.p);
-            }
         }
         U.y = S[8];
         U.xy = S[9];
         U.mxy = S[7];
-        U.tie = (S[8].F == Real(0) && D.Ty != Real(0)) ||
-                (DIAG && ((S[9].F == Real(0) && D.Tpp != Real(0)) || (S[7].F == Real(0) && D.Tmp != Real(0))));
+        U.tie = (S[8].F == 0.f && D.Ty != 0.f) ||
+                (DIAG && ((S[9].F == 0.f && D.Tpp != 0.f) || (S[7].F == 0.f && D.Tmp != 0.f)));
 
         // links into row j-1: negations of Uprev (own +y, left's +x+y, right's -x+y)
-        S[2] = LinkOut<Real>{-Uprev.y.F, -Uprev.y.Db, -Uprev.y.Da};
+        S[2] = LinkOut<float>{-Uprev.y.F, -Uprev.y.Db, -Uprev.y.Da};
         if (DIAG) {
-            const Real f1 = vshfl_up(Uprev.xy.F), a1 = vshfl_up(Uprev.xy.Da), b1 = vshfl_up(Uprev.xy.Db);
-            const Real f3 = vshfl_down(Uprev.mxy.F), a3 = vshfl_down(Uprev.mxy.Da), b3 = vshfl_down(Uprev.mxy.Db);
-            S[1] = LinkOut<Real>{-f1, -b1, -a1};
-            S[3] = LinkOut<Real>{-f3, -b3, -a3};
+            const float f1 = vshfl_up(Uprev.xy.F), a1 = vshfl_up(Uprev.xy.Da), b1 = vshfl_up(Uprev.xy.Db);
+            const float f3 = vshfl_down(Uprev.mxy.F), a3 = vshfl_down(Uprev.mxy.Da), b3 = vshfl_down(Uprev.mxy.Db);
+            S[1] = LinkOut<float>{-f1, -b1, -a1};
+            S[3] = LinkOut<float>{-f3, -b3, -a3};
             if (lane == 0) S[1] = E;
             if (lane == 31) S[3] = E;
         }
@@ -539,15 +514,15 @@ struct YMarch {
     // into row j.  buf: this step's staging buffer.  Returns the links from
     // row j into row j+1.
     template <int PATH>
-    __device__ __forceinline__ YUp<Real> row(int j, const YRow<Real>& P, const YRow<Real>& C, const YRow<Real>& N,
-                                             const YIn<Real>& D, const YUp<Real>& Uprev, Real* buf,
+    __device__ __forceinline__ YUp row(int j, const YRow& P, const YRow& C, const YRow& N,
+                                             const YIn& D, const YUp& Uprev, float* buf,
                                              int rowbase) const {
         constexpr bool FULL = PATH == 2, INJK = PATH >= 1;
         constexpr int L = DIAG ? 11 : 7, LX = DIAG ? 3 : 1;  // interior row length; x links per side
         const int ey = INJK ? 2 : axis_links(j, ny);
         const unsigned mask = row_mask<PATH>(j);
-        LinkOut<Real> S[NSLOT];
-        YUp<Real> U;
+        LinkOut<float> S[NSLOT];
+        YUp U;
         eval_links(P, C, N, D, Uprev, S, U);
 
         // offsets of this row's CSR segment and of this lane's row in it
@@ -582,13 +557,13 @@ struct YMarch {
     // dF/dp_K w_K + dF/dp_L w_L is one FP32 fma; the terms and the residual's
     // fluxes share one FP32x2 Kahan sum in slot order, then dA/dp w_K.
     template <int PATH>
-    __device__ __forceinline__ YUp<Real> row_jvp(int j, const YRow<Real>& P, const YRow<Real>& C,
-                                                 const YRow<Real>& N, const YIn<Real>& D, const YUp<Real>& Uprev,
+    __device__ __forceinline__ YUp row_jvp(int j, const YRow& P, const YRow& C,
+                                                 const YRow& N, const YIn& D, const YUp& Uprev,
                                                  const YW& wP, const YW& wC, const YW& wN, float wzm,
                                                  float wzp) const {
         const unsigned mask = row_mask<PATH>(j);
-        LinkOut<Real> S[NSLOT];
-        YUp<Real> U;
+        LinkOut<float> S[NSLOT];
+        YUp U;
         eval_links(P, C, N, D, Uprev, S, U);
         const float ws[NSLOT] = {wzm, wP.m, wP.c, wP.p, wC.m, 0.f, wC.p, wN.m, wN.c, wN.p, wzp};
         Kahan2 ks;
@@ -625,16 +600,16 @@ struct YMarch {
     // where any link had F == 0, and the caller recomputes it after the march
     // with the full formulation (which adds the tie terms).
     template <int PATH>
-    __device__ __forceinline__ YUp<Real> row_vjp(int j, const YRow<Real>& P, const YRow<Real>& C,
-                                                 const YRow<Real>& N, const YIn<Real>& D, const YUp<Real>& Uprev,
-                                                 Real Ty_prev, Real Tpp_prev, Real Tmp_prev, const YV& vP,
+    __device__ __forceinline__ YUp row_vjp(int j, const YRow& P, const YRow& C,
+                                                 const YRow& N, const YIn& D, const YUp& Uprev,
+                                                 float Ty_prev, float Tpp_prev, float Tmp_prev, const YV& vP,
                                                  const YV& vC, const YV& vN, const F2Split& vzm, const F2Split& vzp,
                                                  float kC, bool& fix) const {
         const unsigned mask = row_mask<PATH>(j);
-        LinkOut<Real> S[NSLOT];
-        YUp<Real> U;
+        LinkOut<float> S[NSLOT];
+        YUp U;
         eval_links(P, C, N, D, Uprev, S, U);
-        Real Tx_m = vshfl_up(D.Tx), Tl = vshfl_up(Tpp_prev), Tr = vshfl_down(Tmp_prev);
+        float Tx_m = vshfl_up(D.Tx), Tl = vshfl_up(Tpp_prev), Tr = vshfl_down(Tmp_prev);
         if (lane == 0) Tx_m = D.hT1, Tl = D.hT2;
         if (lane == 31) Tr = D.hT2;
         const float Ts[NSLOT] = {D.Tz_m, Tl, Ty_prev, Tr, Tx_m, 0.f, D.Tx, D.Tmp, D.Ty, D.Tpp, D.Tz};
@@ -671,56 +646,30 @@ struct YMarch {
     }
 
     // Slot values go to rowbuf; residual and diagonal sums in slot order.
-    // FP32: one FP32x2 Kahan sum carries (residual, diagonal); FP64: plain sums.
-    __device__ __forceinline__ RowSums sum_row(const LinkOut<Real> (&S)[NSLOT], unsigned mask, const CellVal<Real>& me,
-                                               const YIn<Real>& D, Real* rowbuf) const {
-        if constexpr (sizeof(Real) == 4) {
-            Kahan2 ks;
+    // One FP32x2 Kahan sum carries (residual, diagonal).
+    __device__ __forceinline__ RowSums sum_row(const LinkOut<float> (&S)[NSLOT], unsigned mask, const CellVal<float>& me,
+                                               const YIn& D, float* rowbuf) const {
+        Kahan2 ks;
 #pragma unroll
-            for (int s = 0; s < NSLOT; ++s) {
-                if (s == SLOT_SELF) continue;
-                if (mask & (1u << s)) {
-                    ks.add(f2(S[s].F, JAC ? S[s].Da : 0.f));
-                    if (JAC && act) rowbuf[slot_pos(mask, s)] = S[s].Db;
-                }
+        for (int s = 0; s < NSLOT; ++s) {
+            if (s == SLOT_SELF) continue;
+            if (mask & (1u << s)) {
+                ks.add(f2(S[s].F, JAC ? S[s].Da : 0.f));
+                if (JAC && act) rowbuf[slot_pos(mask, s)] = S[s].Db;
             }
-            const AccF acc = accumulation<CRK>(q, me.p, D.pn, D.mn, me.rho, D.phi0);
-            RowSums out;
-            out.R = __dadd_rn(__dadd_rn(acc.A, widen(ks.s.x)), -widen(ks.c.x));
-            out.diag64 = 0.0;
-            if (JAC) {
-                Kahan32 ds{ks.s.y, ks.c.y};
-                ds.add(acc.dA);
-                out.diag64 = __dadd_rn(widen(ds.s), -widen(ds.c));
-                if (act) rowbuf[slot_pos(mask, SLOT_SELF)] = __fsub_rn(ds.s, ds.c);
-            }
-            out.bad = nonfinite(out.R) || (JAC && nonfinite(out.diag64));
-            return out;
-        } else {
-            double rs = 0.0, ds = 0.0;
-#pragma unroll
-            for (int s = 0; s < NSLOT; ++s) {
-                if (s == SLOT_SELF) continue;
-                if (mask & (1u << s)) {
-                    rs = __dadd_rn(rs, S[s].F);
-                    if (JAC) {
-                        ds = __dadd_rn(ds, S[s].Da);
-                        if (act) rowbuf[slot_pos(mask, s)] = S[s].Db;
-                    }
-                }
-            }
-            const AccD acc = accumulation<CRK>(q, me.p, D.pn, D.mn, me.rho, D.phi0);
-            RowSums out;
-            out.R = __dadd_rn(rs, acc.A);
-            out.diag64 = 0.0;
-            if (JAC) {
-                ds = __dadd_rn(ds, acc.dA);
-                out.diag64 = ds;
-                if (act) rowbuf[slot_pos(mask, SLOT_SELF)] = ds;
-            }
-            out.bad = nonfinite(out.R) || (JAC && nonfinite(out.diag64));
-            return out;
         }
+        const AccF acc = accumulation<CRK>(q, me.p, D.pn, D.mn, me.rho, D.phi0);
+        RowSums out;
+        out.R = __dadd_rn(__dadd_rn(acc.A, widen(ks.s.x)), -widen(ks.c.x));
+        out.diag64 = 0.0;
+        if (JAC) {
+            Kahan32 ds{ks.s.y, ks.c.y};
+            ds.add(acc.dA);
+            out.diag64 = __dadd_rn(widen(ds.s), -widen(ds.c));
+            if (act) rowbuf[slot_pos(mask, SLOT_SELF)] = __fsub_rn(ds.s, ds.c);
+        }
+        out.bad = nonfinite(out.R) || (JAC && nonfinite(out.diag64));
+        return out;
     }
 
     // Wait until the bulk store issued from this buffer two steps ago has
@@ -736,8 +685,8 @@ struct YMarch {
     // middle goes out as one bulk shared->global copy (issued by lane 0,
     // tracked as a bulk async-group); the at most 2 (VEC - 1) elements at the
     // ends are stored by single lanes.
-    __device__ __forceinline__ void write_segment(Real* buf, long long seg, int aoff, int len) const {
-        Real* dst = o.vals + (seg - aoff);  // 16-byte aligned when v16
+    __device__ __forceinline__ void write_segment(float* buf, long long seg, int aoff, int len) const {
+        float* dst = o.vals + (seg - aoff);  // 16-byte aligned when v16
         const int span = aoff + len;
         if (v16) {
             const int qlo = (aoff + VEC - 1) / VEC, qhi = span / VEC;
@@ -774,10 +723,9 @@ struct YMarch {
 
 // Dynamic shared memory of one block of W warps: per warp two CSR staging
 // buffers, the RING x NF input ring and the RING m^n values.
-template <typename Real, int W>
+template <int W>
 constexpr int ymarch_smem_bytes() {
-    return W * (2 * (32 * NSLOT + 16 / (int)sizeof(Real)) * (int)sizeof(Real) +
-                3 * 18 * 32 * (int)sizeof(Real) + 3 * 32 * (int)sizeof(double));
+    return W * (2 * (32 * NSLOT + 4) * 4 + 3 * 18 * 32 * 4 + 3 * 32 * 8);
 }
 
 // One block's work: x-segment bx, y-run by, z-block bz of one grid.  Shared
@@ -810,19 +758,19 @@ __device__ __forceinline__ void march_rows(int j0, int j1, int ny, bool zint, bo
 // 160 x 160 x 80 and on the 64-model ensemble: the ensemble's persistent
 // kernel gains 5 % with it, the single-grid kernel loses 4 %, so only the
 // ensemble uses it.
-template <typename Real, bool DIAG, bool CRK, bool JAC, int W, bool SPLIT = false>
-__device__ __forceinline__ void ymarch_tile(const GridGeom& g, const typename PhysOf<Real>::type& q,
-                                            const AsmFields<Real>& f, const AsmOut<Real>& o, int JY, int bx, int by,
+template <bool DIAG, bool CRK, bool JAC, int W, bool SPLIT = false>
+__device__ __forceinline__ void ymarch_tile(const GridGeom& g, const PhysF& q, const AsmFields<float>& f,
+                                            const AsmOut<float>& o, int JY, int bx, int by,
                                             int bz, unsigned char* smem, int kbase = 0, int kend = -1) {
-    using M_t = YMarch<Real, DIAG, CRK, JAC, W>;
-    constexpr int BUF = 32 * NSLOT + 16 / (int)sizeof(Real);
+    using M_t = YMarch<DIAG, CRK, JAC, W>;
+    constexpr int BUF = 32 * NSLOT + 4;
     const int lane = threadIdx.x, w = threadIdx.y;
     const int k = kbase + bz * W + w;  // planes [kbase, kend) of the grid (all by default)
     if (k >= (kend < 0 ? g.nz : kend)) return;  // warp-uniform
     // per warp: two staging buffers, then the input ring, then the m^n ring
-    Real* stage = reinterpret_cast<Real*>(smem) + w * 2 * BUF;
-    Real* ring = reinterpret_cast<Real*>(smem) + W * 2 * BUF + w * M_t::RING * M_t::NF * 32;
-    double* ringm = reinterpret_cast<double*>(reinterpret_cast<Real*>(smem) + W * 2 * BUF +
+    float* stage = reinterpret_cast<float*>(smem) + w * 2 * BUF;
+    float* ring = reinterpret_cast<float*>(smem) + W * 2 * BUF + w * M_t::RING * M_t::NF * 32;
+    double* ringm = reinterpret_cast<double*>(reinterpret_cast<float*>(smem) + W * 2 * BUF +
                                               W * M_t::RING * M_t::NF * 32) + w * M_t::RING * 32;
     M_t M(g, q, f, o, lane, bx * 32, k);
     M.ring = ring;
@@ -837,16 +785,16 @@ __device__ __forceinline__ void ymarch_tile(const GridGeom& g, const typename Ph
     M.issue_row(j0, 1);
     M.issue_row(j0 + 1, 2);
     M.wait_all_but_newest();
-    YRow<Real> P = M.row_cells(0);
-    YRow<Real> C = M.row_cells(1);
-    Real Ty_prev, Tpp_prev, Tmp_prev;
+    YRow P = M.row_cells(0);
+    YRow C = M.row_cells(1);
+    float Ty_prev, Tpp_prev, Tmp_prev;
     {
-        const YIn<Real> Dp = M.read_in(0);
+        const YIn Dp = M.read_in(0);
         Ty_prev = Dp.Ty;
         Tpp_prev = Dp.Tpp;
         Tmp_prev = Dp.Tmp;
     }
-    YUp<Real> U = M.up_links(P, C, Ty_prev, Tpp_prev, Tmp_prev);
+    YUp U = M.up_links(P, C, Ty_prev, Tpp_prev, Tmp_prev);
     int s0 = 1, s1 = 2, s2 = 0;  // ring slots of rows j, j+1, j+2
     int rowbase = M.row_base(j0);
     // rows whose links into the previous row (reused by negation) met an
@@ -859,13 +807,13 @@ __device__ __forceinline__ void ymarch_tile(const GridGeom& g, const typename Ph
             // row j+2 is requested now and used two steps later; row j+1 arrived
             M.issue_row(j + 2, s2);
             M.wait_all_but_newest();
-            const YRow<Real> N = M.row_cells(s1);
-            const YIn<Real> D = M.read_in(s0);
+            const YRow N = M.row_cells(s1);
+            const YIn D = M.read_in(s0);
             const int st = s0;
             s0 = s1;
             s1 = s2;
             s2 = st;
-            Real* buf = stage + ((j - j0) & 1) * BUF;
+            float* buf = stage + ((j - j0) & 1) * BUF;
             M.buffer_ready();
             if (__any_sync(0xffffffffu, U.tie)) tie_rows |= 1ull << (j - j0);
             U = M.template row<PATH>(j, P, C, N, D, U, buf, rowbase);
@@ -878,13 +826,13 @@ __device__ __forceinline__ void ymarch_tile(const GridGeom& g, const typename Ph
             // row j+2 is requested now and used two steps later; row j+1 arrived
             M.issue_row(j + 2, s2);
             M.wait_all_but_newest();
-            const YRow<Real> N = M.row_cells(s1);
-            const YIn<Real> D = M.read_in(s0);
+            const YRow N = M.row_cells(s1);
+            const YIn D = M.read_in(s0);
             const int st = s0;
             s0 = s1;
             s1 = s2;
             s2 = st;
-            Real* buf = stage + ((j - j0) & 1) * BUF;
+            float* buf = stage + ((j - j0) & 1) * BUF;
             M.buffer_ready();
             if (__any_sync(0xffffffffu, U.tie)) tie_rows |= 1ull << (j - j0);
             const bool injk = zint && j > 0 && j + 1 < M.ny;
@@ -901,7 +849,7 @@ __device__ __forceinline__ void ymarch_tile(const GridGeom& g, const typename Ph
     if (tie_rows) {  // warp-uniform; every bulk store of the warp has completed
         __syncwarp();
         for (int b = 0; b < 64; ++b)
-            if ((tie_rows >> b) & 1ull) naive_row<Real, CRK, JAC>(g, q, f, o, M.act, M.i, j0 + b, k);
+            if ((tie_rows >> b) & 1ull) naive_row<float, CRK, JAC>(g, q, f, o, M.act, M.i, j0 + b, k);
     }
 }
 
@@ -925,7 +873,7 @@ template <bool DIAG, bool CRK, bool JAC, int W>
 __device__ __forceinline__ void ymarch_tile_tma(const GridGeom& g, const PhysF& q, const AsmFields<float>& f,
                                                 const AsmOut<float>& o, const TmaMaps* maps, int JY, int bx,
                                                 int by, int k, unsigned char* smem) {
-    using M_t = YMarch<float, DIAG, CRK, JAC, W>;
+    using M_t = YMarch<DIAG, CRK, JAC, W>;
     using TS = TmaSlot<W>;
     constexpr int BUF = 32 * NSLOT + 4, TR = M_t::TRING;
     const int lane = threadIdx.x, w = threadIdx.y;
@@ -949,11 +897,11 @@ __device__ __forceinline__ void ymarch_tile_tma(const GridGeom& g, const PhysF& 
     ok = ok && M.tma_wait(1);
     unsigned long long tie_rows = 0ull;
     if (ok) {
-        YRow<float> P = M.tma_row_cells(0);
-        YRow<float> C = M.tma_row_cells(1);
-        YUp<float> U;
+        YRow P = M.tma_row_cells(0);
+        YRow C = M.tma_row_cells(1);
+        YUp U;
         {
-            const YIn<float> Dp = M.tma_read_in(0, 0.f);
+            const YIn Dp = M.tma_read_in(0, 0.f);
             U = M.up_links(P, C, Dp.Ty, Dp.Tpp, Dp.Tmp);
         }
         int sp = 0;  // slot of row j-1; rows j, j+1, ... follow in the next slots (mod TR)
@@ -969,8 +917,8 @@ __device__ __forceinline__ void ymarch_tile_tma(const GridGeom& g, const PhysF& 
                 ok = false;
                 break;
             }
-            const YRow<float> N = M.tma_row_cells(s1);
-            const YIn<float> D = M.tma_read_in(s0, hT2);
+            const YRow N = M.tma_row_cells(s1);
+            const YIn D = M.tma_read_in(s0, hT2);
             sp = s0;
             if (live) {
                 float* buf = stage + ((j - j0) & 1) * BUF;
@@ -1007,12 +955,11 @@ __global__ void __launch_bounds__(32 * W, 16 / W)
     ymarch_tile_tma<DIAG, CRK, JAC, W>(g, q, f, o, &tm, JY, blockIdx.x, blockIdx.y, k0 + (int)blockIdx.z, smem);
 }
 
-template <typename Real, bool DIAG, bool CRK, bool JAC, int W>
-__global__ void __launch_bounds__(32 * W, (sizeof(Real) == 4 ? 16 : 8) / W)
-    k_assemble_ymarch(GridGeom g, typename PhysOf<Real>::type q, AsmFields<Real> f, AsmOut<Real> o, int JY,
-                      int k0, int k1) {
+template <bool DIAG, bool CRK, bool JAC, int W>
+__global__ void __launch_bounds__(32 * W, 16 / W)
+    k_assemble_ymarch(GridGeom g, PhysF q, AsmFields<float> f, AsmOut<float> o, int JY, int k0, int k1) {
     extern __shared__ __align__(16) unsigned char smem[];
-    ymarch_tile<Real, DIAG, CRK, JAC, W>(g, q, f, o, JY, blockIdx.x, blockIdx.y, blockIdx.z, smem, k0, k1);
+    ymarch_tile<DIAG, CRK, JAC, W>(g, q, f, o, JY, blockIdx.x, blockIdx.y, blockIdx.z, smem, k0, k1);
 }
 
 }  // namespace tpfa
