@@ -411,8 +411,8 @@ typedef struct {
  * again when x_dev or check_every change); a `stream` that is itself being
  * captured gets plain launches.  Returns TPFA_ERR_NO_CONVERGENCE when the
  * tolerance was not met (x_dev then holds the last iterate).  The first
- * call allocates the workspace: nnz values, 12 FP64 vectors of N (and, on
- * TPFA_MIXED, four FP32 vectors), and creates the stream and two events.
+ * call allocates the workspace (14 FP64 vectors of N and 6 or 10 values of the
+ * field type per cell) and creates the stream and two events.
  */
 int tpfa_linear_solve(tpfa_handle h, const double* b_dev, double* x_dev, const tpfa_krylov_opts* opts,
                       tpfa_krylov_stats* stats, void* stream);

@@ -147,12 +147,15 @@ struct tpfa_grid {
     cudaStream_t h_up = nullptr, h_down = nullptr;
     cudaEvent_t h_ev[2 * kMaxSlabs + 2] = {};
     // Newton / Krylov workspace, allocated on first use
-    void* kv_vals = nullptr;
+    // The vectors are slices of one pool, which first holds the assembled CSR
+    // values: they are copied by slots into kv_dia before the vectors are used.
+    double* kv_pool = nullptr;
+    void* kv_dia = nullptr;    // off-diagonals by stencil slots
     double* kv_diag = nullptr;
     double* kv_R = nullptr;
-    double* kv_vec[12] = {};  // x, r, r^, p, p^, v, s, s^, t, M^-1 (and z-line multipliers, super-diagonal)
-    float* kv_f32[4] = {};    // p^ and s^ split into FP32 pairs (mixed path)
+    double* kv_x = nullptr;
     double* kv_part = nullptr;
+    unsigned int* kv_arrived = nullptr;
     KrylovScalars* kv_S = nullptr;
     KrylovScalars* kv_S_host = nullptr;  // pinned
     // the solve's batches of iterations as one CUDA graph, launched on a
@@ -164,6 +167,19 @@ struct tpfa_grid {
     int kv_exec_every = 0;
     bool kv_exec_line = false;
 
+    void release_krylov() {
+        dev_free(kv_pool);
+        dev_free(kv_dia);
+        dev_free(kv_diag);
+        dev_free(kv_R);
+        dev_free(kv_x);
+        dev_free(kv_part);
+        dev_free(kv_arrived);
+        dev_free(kv_S);
+        if (kv_S_host) cudaFreeHost(kv_S_host);
+        kv_pool = nullptr, kv_dia = nullptr, kv_diag = nullptr, kv_R = nullptr, kv_x = nullptr, kv_part = nullptr;
+        kv_arrived = nullptr, kv_S = nullptr, kv_S_host = nullptr;
+    }
     void release() {
         for (auto& ev : h_ev) {
             if (ev) cudaEventDestroy(ev);
@@ -172,15 +188,7 @@ struct tpfa_grid {
         if (h_up) cudaStreamDestroy(h_up);
         if (h_down) cudaStreamDestroy(h_down);
         h_up = h_down = nullptr;
-        dev_free(kv_vals);
-        dev_free(kv_diag);
-        dev_free(kv_R);
-        for (auto& v : kv_vec) dev_free(v), v = nullptr;
-        for (auto& v : kv_f32) dev_free(v), v = nullptr;
-        dev_free(kv_part);
-        dev_free(kv_S);
-        if (kv_S_host) cudaFreeHost(kv_S_host);
-        kv_vals = nullptr, kv_diag = nullptr, kv_R = nullptr, kv_part = nullptr, kv_S = nullptr, kv_S_host = nullptr;
+        release_krylov();
         if (kv_exec) cudaGraphExecDestroy(kv_exec);
         for (auto& ev : kv_ev)
             if (ev) cudaEventDestroy(ev), ev = nullptr;
@@ -336,33 +344,27 @@ int march_rows2(const tpfa_grid* h) {
     return jy;
 }
 
-// Newton / Krylov workspace: the assembled Jacobian, R, twelve FP64 vectors,
-// the partial sums and the scalar record (device and pinned host copies).
+// Newton / Krylov workspace: the Jacobian by slots with its FP64 diagonal, R,
+// x, the pool of ten FP64 vectors (and the FP32 pairs, as wide as one), the
+// partial sums and the scalar record (device and pinned host copies).
+constexpr int kPoolVectors = 11;  // r, r^, p, p^, v, s^, t, M^-1 (three), pairs
+
 int krylov_workspace(tpfa_grid* h) {
     if (h->kv_S_host) return TPFA_OK;
     const size_t nb = sizeof(double) * (size_t)h->N;
-    bool ok = dev_alloc(&h->kv_vals, h->real_size * (size_t)h->nnz) == cudaSuccess;
-    if (ok && h->prec == TPFA_MIXED) ok = dev_alloc((void**)&h->kv_diag, nb) == cudaSuccess;
+    // the CSR values need at most eleven entries of 8 bytes per cell: they fit
+    bool ok = dev_alloc((void**)&h->kv_pool, kPoolVectors * nb) == cudaSuccess;
+    ok = ok && dev_alloc(&h->kv_dia, h->real_size * (size_t)krylov_slot_values(h->geom, h->N)) == cudaSuccess;
+    ok = ok && dev_alloc((void**)&h->kv_diag, nb) == cudaSuccess;
     ok = ok && dev_alloc((void**)&h->kv_R, nb) == cudaSuccess;
-    for (auto& v : h->kv_vec) ok = ok && dev_alloc((void**)&v, nb) == cudaSuccess;
-    if (h->prec == TPFA_MIXED)
-        for (auto& v : h->kv_f32) ok = ok && dev_alloc((void**)&v, sizeof(float) * (size_t)h->N) == cudaSuccess;
-    ok = ok && dev_alloc((void**)&h->kv_part, sizeof(double) * 2 * (size_t)krylov_partials(h->geom, h->N)) ==
-                   cudaSuccess;
+    ok = ok && dev_alloc((void**)&h->kv_x, nb) == cudaSuccess;
+    ok = ok && dev_alloc((void**)&h->kv_part, sizeof(double) * 2 * (size_t)krylov_partials()) == cudaSuccess;
+    ok = ok && dev_alloc((void**)&h->kv_arrived, sizeof(unsigned int)) == cudaSuccess;
     ok = ok && dev_alloc((void**)&h->kv_S, sizeof(KrylovScalars)) == cudaSuccess;
     ok = ok && cudaMallocHost((void**)&h->kv_S_host, sizeof(KrylovScalars)) == cudaSuccess;
     if (!ok) {
         cudaGetLastError();
-        dev_free(h->kv_vals);
-        dev_free(h->kv_diag);
-        dev_free(h->kv_R);
-        for (auto& v : h->kv_vec) dev_free(v), v = nullptr;
-        for (auto& v : h->kv_f32) dev_free(v), v = nullptr;
-        dev_free(h->kv_part);
-        dev_free(h->kv_S);
-        if (h->kv_S_host) cudaFreeHost(h->kv_S_host);
-        h->kv_vals = nullptr, h->kv_diag = nullptr, h->kv_R = nullptr, h->kv_part = nullptr, h->kv_S = nullptr;
-        h->kv_S_host = nullptr;
+        h->release_krylov();
         return fail(TPFA_ERR_OOM, "device allocation failed for the Newton/Krylov workspace");
     }
     return TPFA_OK;
@@ -378,30 +380,20 @@ int krylov_solve(tpfa_grid* h, const double* b, double sign, double* x, const tp
     const bool mixed = h->prec == TPFA_MIXED;
     KrylovWork w;
     w.x = x;
-    w.r = h->kv_vec[1];
-    w.rh = h->kv_vec[2];
-    w.p = h->kv_vec[3];
-    w.ph = h->kv_vec[4];
-    w.v = h->kv_vec[5];
-    w.s = h->kv_vec[6];
-    w.sh = h->kv_vec[7];
-    w.t = h->kv_vec[8];
-    w.dinv = h->kv_vec[9];
-    w.lmul = h->kv_vec[10];
-    w.up = h->kv_vec[11];
-    w.phh = h->kv_f32[0];
-    w.phl = h->kv_f32[1];
-    w.shh = h->kv_f32[2];
-    w.shl = h->kv_f32[3];
-    w.part = h->kv_part;
-    w.S = h->kv_S;
+    double** const vec[] = {&w.r, &w.rh, &w.p, &w.ph, &w.v, &w.sh, &w.t, &w.dinv, &w.lmul, &w.up};
+    double* next = h->kv_pool;
+    for (double** v : vec) *v = next, next += h->N;
+    w.pair = reinterpret_cast<float2*>(next);
+    w.dia = h->kv_dia;
+    w.diag = h->kv_diag;
+    w.sums = KrylovSums{h->kv_part, h->kv_arrived, h->kv_S};
     KrylovScalars* Sh = h->kv_S_host;
     *Sh = KrylovScalars{};
     Sh->tol2 = rtol * rtol;
     Sh->max_iters = max_iters;
     // The iterations run on the library's stream as CUDA-graph launches of
-    // `every` iterations each (ten kernels per iteration: one launch per
-    // batch instead of ten per iteration); that stream waits for `st`
+    // `every` iterations each (five kernels per iteration: one launch per
+    // batch instead of five per iteration); that stream waits for `st`
     // before the solve and `st` for it after.  A stream that is being
     // captured gets the plain launches instead.
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
@@ -443,7 +435,7 @@ int krylov_solve(tpfa_grid* h, const double* b, double sign, double* x, const tp
             e = cudaStreamBeginCapture(ks, cudaStreamCaptureModeThreadLocal);
             cudaError_t el = cudaSuccess;
             for (int q = 0; q < every && e == cudaSuccess && el == cudaSuccess; ++q)
-                el = krylov_iteration(h->geom, h->N, mixed, h->kv_vals, h->kv_diag, w, line, ks);
+                el = krylov_iteration(h->geom, h->N, mixed, w, line, ks);
             if (e == cudaSuccess) e = cudaStreamEndCapture(ks, &gr);
             if (e == cudaSuccess) e = el;
             if (e == cudaSuccess) e = cudaGraphInstantiate(&h->kv_exec, gr, 0);
@@ -458,9 +450,9 @@ int krylov_solve(tpfa_grid* h, const double* b, double sign, double* x, const tp
             h->kv_exec_line = line;
         }
     }
-    e = cudaMemcpyAsync(w.S, Sh, sizeof(KrylovScalars), cudaMemcpyHostToDevice, ks);
-    if (e == cudaSuccess) e = krylov_dinv(h->geom, mixed, h->kv_vals, h->kv_diag, w.dinv, w.lmul, w.up, line, ks);
-    if (e == cudaSuccess) e = krylov_start(h->geom, h->N, b, sign, w, ks);
+    e = cudaMemcpyAsync(w.sums.S, Sh, sizeof(KrylovScalars), cudaMemcpyHostToDevice, ks);
+    if (e == cudaSuccess) e = cudaMemsetAsync(w.sums.arrived, 0, sizeof(unsigned int), ks);
+    if (e == cudaSuccess) e = krylov_start(h->geom, h->N, mixed, h->kv_pool, b, sign, w, line, ks);
     if (e != cudaSuccess) {
         join();
         return cuda_fail(e, "Krylov start");
@@ -472,8 +464,8 @@ int krylov_solve(tpfa_grid* h, const double* b, double sign, double* x, const tp
     for (int it = 0; it <= max_iters + every; it += every) {
         if (graph) e = cudaGraphLaunch(h->kv_exec, ks);
         for (int q = 0; !graph && q < every && e == cudaSuccess; ++q)
-            e = krylov_iteration(h->geom, h->N, mixed, h->kv_vals, h->kv_diag, w, line, ks);
-        if (e == cudaSuccess) e = cudaMemcpyAsync(Sh, w.S, sizeof(KrylovScalars), cudaMemcpyDeviceToHost, ks);
+            e = krylov_iteration(h->geom, h->N, mixed, w, line, ks);
+        if (e == cudaSuccess) e = cudaMemcpyAsync(Sh, w.sums.S, sizeof(KrylovScalars), cudaMemcpyDeviceToHost, ks);
         if (e == cudaSuccess) e = cudaStreamSynchronize(ks);
         if (e != cudaSuccess) {
             join();
@@ -996,7 +988,7 @@ int tpfa_linear_solve(tpfa_handle h, const double* b_dev, double* x_dev, const t
     rc = krylov_workspace(h);
     if (rc) return rc;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    rc = launch(h, auto_kernel(h), nullptr, h->kv_vals, h->prec == TPFA_MIXED ? h->kv_diag : nullptr, st);
+    rc = launch(h, auto_kernel(h), nullptr, h->kv_pool, h->prec == TPFA_MIXED ? h->kv_diag : nullptr, st);
     if (rc) return rc;
     return krylov_solve(h, b_dev, 1.0, x_dev, opts, stats, st);
 }
@@ -1014,8 +1006,8 @@ int tpfa_newton_step(tpfa_handle h, void* p_dev, const tpfa_krylov_opts* opts, t
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     h->p = p_dev;
     double* R = R_dev ? R_dev : h->kv_R;
-    double* x = delta_dev ? delta_dev : h->kv_vec[0];
-    rc = launch(h, auto_kernel(h), R, h->kv_vals, h->prec == TPFA_MIXED ? h->kv_diag : nullptr, st);
+    double* x = delta_dev ? delta_dev : h->kv_x;
+    rc = launch(h, auto_kernel(h), R, h->kv_pool, h->prec == TPFA_MIXED ? h->kv_diag : nullptr, st);
     if (rc) return rc;
     rc = krylov_solve(h, R, -1.0, x, opts, stats, st);
     if (rc) return rc;

@@ -93,24 +93,32 @@ struct KrylovScalars {
     double rho, alpha, omega, beta, rr, bb, tol2;
     int done, breakdown, iter, max_iters;
 };
-struct KrylovWork {
-    double *x, *r, *rh, *p, *ph, *v, *s, *sh, *t, *dinv;
-    float *phh, *phl, *shh, *shl;  // p^ and s^ split into FP32 pairs (mixed path), else null
-    double *lmul, *up;  // z-line factorisation: multipliers and super-diagonal
-    double* part;       // 2 * krylov_partials() per-block partial sums
+// What the reducing kernels end in: partial sums, the count of finished
+// blocks (zero between kernels) and the scalars.
+struct KrylovSums {
+    double* part;  // 2 * krylov_partials() per-block partial sums
+    unsigned int* arrived;
     KrylovScalars* S;
 };
-long long krylov_vec_blocks(long long n);
-long long krylov_partials(const GridGeom& g, long long n);
-// M^-1 data: the inverse diagonal (Jacobi) or the inverse pivots of the z-line
-// factorisation (line).
-cudaError_t krylov_dinv(const GridGeom& g, bool mixed, const void* vals, const double* diag64, double* dinv,
-                        double* lmul, double* up, bool line, cudaStream_t st);
-// x = 0, r = r^ = sign * b, scalars initialised (S->tol2, S->max_iters set by the caller)
-cudaError_t krylov_start(const GridGeom& g, long long n, const double* b, double sign, const KrylovWork& w,
-                         cudaStream_t st);
-cudaError_t krylov_iteration(const GridGeom& g, long long n, bool mixed, const void* vals, const double* diag64,
-                             const KrylovWork& w, bool line, cudaStream_t st);
+struct KrylovWork {
+    double *x, *r, *rh, *p, *ph, *v, *sh, *t;  // s is held in r
+    double *dinv, *lmul, *up;  // M^-1 data (inverse diagonal or pivots; z-line: multipliers, super-diagonal)
+    float2* pair;              // p^ or s^ split into FP32 pairs (mixed path)
+    void* dia;                 // the off-diagonals by slots, krylov_slot_values() values of the field type
+    double* diag;              // the FP64 diagonal
+    KrylovSums sums;
+};
+long long krylov_partials();
+long long krylov_slot_values(const GridGeom& g, long long n);
+// The matrix by slots from its CSR values (`vals` may lie in the memory of r,
+// rh, p, ph, v, sh, t, pair, dinv, lmul and up: nothing there is written while
+// it is read; on the mixed path w.diag already holds the diagonal), M^-1's
+// data, x = 0, r = r^ = sign * b, the scalars (S->tol2 and S->max_iters are
+// the caller's).
+cudaError_t krylov_start(const GridGeom& g, long long n, bool mixed, const void* vals, const double* b, double sign,
+                         const KrylovWork& w, bool line, cudaStream_t st);
+cudaError_t krylov_iteration(const GridGeom& g, long long n, bool mixed, const KrylovWork& w, bool line,
+                             cudaStream_t st);
 cudaError_t krylov_add_delta(long long n, bool mixed, void* p, const double* d, cudaStream_t st);
 
 // General meshes (tpfa_mesh.cu).
