@@ -324,7 +324,16 @@ bool aligned(const void* p, uintptr_t a) { return (reinterpret_cast<uintptr_t>(p
 // the remainder truncated (F2Split), one pair per cell.
 __global__ void k_split_pairs(const double* __restrict__ v, float2* __restrict__ out, long long n) {
     for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < n; c += (long long)gridDim.x * blockDim.x) {
-        const F2Split t = split_f2(v[c]);
+        const double d = v[c];
+        const uint32_t a = abs_hi(d);
+        // a normal hi whose remainder is normal or zero: no general conversion
+        F2Split t;
+        if (__all_sync(__activemask(), a == 0u || (a >= 0x3c000000u && a < 0x47e00000u))) {
+            t.hi = narrow_flush(d);
+            t.lo = narrow_flush(__dadd_rn(d, -widen_flush(t.hi)));
+        } else {
+            t = split_f2(d);
+        }
         out[c] = make_float2(t.hi, t.lo);
     }
 }

@@ -89,16 +89,16 @@ __device__ __forceinline__ void kahan2_masked(Kahan2& k, float2 x, bool va, bool
     k.c.y = vb ? t.c.y : k.c.y;
 }
 
-// accumulation() of Eq. vk for cells a and b at once: each half performs
-// the scalar function's operations in its order (FP32x2 halves round as the
-// scalar instructions do), so the results are its bits.  Returns the FP64
-// terms A of both cells and the pair of dA/dp.
+// accumulation() of Eq. vk (PLAIN) for cells a and b at once: each half
+// performs the scalar function's operations in its order (FP32x2 halves round
+// as the scalar instructions do), so the results are its bits.  Returns the
+// FP64 terms A of both cells and the pair of dA/dp.
 template <bool CRK>
 __device__ __forceinline__ float2 accumulation2(const PhysF& q, float2 p, float2 pn, double2 mn, float2 rho,
                                                 float2 phi0, double& Aa, double& Ab) {
     if constexpr (CRK) {
-        const AccF a = accumulation<true>(q, p.x, pn.x, mn.x, rho.x, phi0.x);
-        const AccF b = accumulation<true>(q, p.y, pn.y, mn.y, rho.y, phi0.y);
+        const AccF a = accumulation<true, true>(q, p.x, pn.x, mn.x, rho.x, phi0.x);
+        const AccF b = accumulation<true, true>(q, p.y, pn.y, mn.y, rho.y, phi0.y);
         Aa = a.A;
         Ab = b.A;
         return f2(a.dA, b.dA);
@@ -106,17 +106,20 @@ __device__ __forceinline__ float2 accumulation2(const PhysF& q, float2 p, float2
         const float2 m1 = f2(-1.f);
         const float2 x = __fmul2_rn(f2(q.c_f), __ffma2_rn(pn, m1, p));  // c_f (p - p^n)
         float2 e;
+        double ea, eb;
         if (fabsf(x.x) < 0.0078125f && fabsf(x.y) < 0.0078125f) {  // expm1_f32's series for both
             float2 r = __ffma2_rn(x, f2(1.f / 24.f), f2(1.f / 6.f));
             r = __ffma2_rn(x, r, f2(0.5f));
             r = __ffma2_rn(x, r, f2(1.f));
             e = __fmul2_rn(r, x);
+            ea = widen_flush(e.x);
+            eb = widen_flush(e.y);
         } else {
-            e = f2(expm1_f32(x.x), expm1_f32(x.y));
+            e = f2(expm1_wide<true>(x.x, ea), expm1_wide<true>(x.y, eb));
         }
-        Aa = __dmul_rn(mn.x, widen(e.x));
-        Ab = __dmul_rn(mn.y, widen(e.y));
-        return __fmul2_rn(__fmul2_rn(f2(q.c_f), f2(narrow_rz(mn.x), narrow_rz(mn.y))), __fadd2_rn(f2(1.f), e));
+        Aa = __dmul_rn(mn.x, ea);
+        Ab = __dmul_rn(mn.y, eb);
+        return __fmul2_rn(__fmul2_rn(f2(q.c_f), f2(narrow_flush(mn.x), narrow_flush(mn.y))), __fadd2_rn(f2(1.f), e));
     }
 }
 
@@ -532,7 +535,7 @@ struct XState {
         // (on an interior segment every lane's +x and diagonal links exist)
         const bool kb2 = PATH == 2 ? true : okb, ka2 = PATH == 2 ? true : oka;
         const bool tie_x = on && (LX_.F.x == 0.f || (kb2 && LX_.F.y == 0.f));
-        const bool tie = __any_sync(0xffffffffu, tie_up || tie_x);
+        const bool tie_here = tie_up || tie_x;
         tie_up = on && (LY.F.x == 0.f || LY.F.y == 0.f ||
                          (DIAG && (LXY.F.x == 0.f || (kb2 && LXY.F.y == 0.f) || (ka2 && LMXY.F.x == 0.f) ||
                                    LMXY.F.y == 0.f)));
@@ -541,14 +544,23 @@ struct XState {
         R.gather();
         double Aa, Ab;
         const float2 dA = accumulation2<CRK>(q, Cc.p, pn, mn, Cc.rho, phi, Aa, Ab);
-        const double Ra = __dadd_rn(__dadd_rn(Aa, widen(R.kr.s.x)), -widen(R.kr.c.x));
-        const double Rb = __dadd_rn(__dadd_rn(Ab, widen(R.kr.s.y)), -widen(R.kr.c.y));
+        const double Ra = __dadd_rn(__dadd_rn(Aa, widen_flush(R.kr.s.x)), -widen_flush(R.kr.c.x));
+        const double Rb = __dadd_rn(__dadd_rn(Ab, widen_flush(R.kr.s.y)), -widen_flush(R.kr.c.y));
         Kahan2 dd = R.kd;  // the diagonals: dA joins each compensated sum last
         dd.add(dA);
-        const double Da64 = __dadd_rn(widen(dd.s.x), -widen(dd.c.x));
-        const double Db64 = __dadd_rn(widen(dd.s.y), -widen(dd.c.y));
+        const double Da64 = __dadd_rn(widen_flush(dd.s.x), -widen_flush(dd.c.x));
+        const double Db64 = __dadd_rn(widen_flush(dd.s.y), -widen_flush(dd.c.y));
         const float2 dg = __ffma2_rn(dd.c, f2(-1.f), dd.s);  // s - c, the FP32 diagonal values
         R.put_diag(dg.x, dg.y, on);
+        // rows that need exact conversions (odd_sum; min_abs is NaN if a sum is)
+        const float rmin = min_abs(R.kr.s.x, R.kr.s.y), dmin = min_abs(dd.s.x, dd.s.y);
+        const uint32_t hi = max(max(max(abs_hi(Ra), abs_hi(Rb)), max(abs_hi(Da64), abs_hi(Db64))),
+                                max(abs_hi(mn.x), abs_hi(mn.y)));
+        bool odd = hi >= kOddHigh;
+        if (!(rmin >= 0x1p-60f && dmin >= 0x1p-60f))  // small, zero or NaN: which
+            odd = odd || odd_sum(R.kr.s.x) || odd_sum(R.kr.s.y) || odd_sum(dd.s.x) || odd_sum(dd.s.y) ||
+                  nan_sum(rmin) || nan_sum(dmin);
+        const bool tie = __any_sync(0xffffffffu, tie_here || (on && odd));
         if (on) {
             const int c = kb + nx * j + ia;
             if (FAST || o.R) {
@@ -559,12 +571,6 @@ struct XState {
                 if (r16) *reinterpret_cast<double2*>(o.diag64 + c) = make_double2(Da64, Db64);
                 else o.diag64[c] = Da64, o.diag64[c + 1] = Db64;
             }
-            // a non-finite value has an all-ones exponent: one test for the four
-            const uint32_t ex = max(max((uint32_t)__double2hiint(Ra) & 0x7ff00000u,
-                                        (uint32_t)__double2hiint(Rb) & 0x7ff00000u),
-                                    max((uint32_t)__double2hiint(Da64) & 0x7ff00000u,
-                                        (uint32_t)__double2hiint(Db64) & 0x7ff00000u));
-            if (ex == 0x7ff00000u) atomicOr(o.status, STATUS_NONFINITE);
         }
 
         // ---- the segment's CSR values: one bulk copy (ends by single lanes)

@@ -62,6 +62,7 @@ struct YIn {  // inputs of one row other than p and z
 struct YUp {  // a link from row j-1 into row j, seen from row j-1
     LinkOut<float> y, xy, mxy;  // to (i, j), (i+1, j), (i-1, j)
     bool tie;                  // any of the three had dPhi == 0 exactly
+    bool odd = false;          // row j-1's results need exact conversions
 };
 
 __device__ __forceinline__ float vshfl_up(float v) {
@@ -398,6 +399,12 @@ struct YMarch {
         return D;
     }
 
+    // The bits of tie_rows for row j and the row before it (whose `odd` is
+    // known only now): j - j0 = e.
+    static __device__ __forceinline__ unsigned long long rows_before(int e) {
+        return (1ull << e) | (e > 0 ? 1ull << (e - 1) : 0ull);
+    }
+
     // w of the row in ring slot sl, narrowed to FP32 on the integer pipe
     // (truncation, below one float ulp), x-neighbours by shuffles.
     __device__ __forceinline__ YW w_row(int sl) const {
@@ -539,8 +546,8 @@ struct YMarch {
         if (act) {
             if (o.R) o.R[c] = out.R;
             if (JAC && o.diag64) o.diag64[c] = out.diag64;
-            if (out.bad) atomicOr(o.status, STATUS_NONFINITE);
         }
+        U.odd = out.bad;
         if (JAC) {
             const int iend = min(i0 + 32, nx);
             int seg_len;
@@ -629,15 +636,15 @@ struct YMarch {
         }
         fix = __any_sync(0xffffffffu, zero_flux);
         const AccF acc = accumulation<CRK>(q, C.c.p, D.pn, D.mn, C.c.rho, D.phi0);
+        // the diagonal's own term v_i dA_i/dp_i joins the compensated FP32
+        // sum last; + 0.0 is the twin's tie correction when no link has
+        // zero flux (it turns a -0 into +0 as that addition does)
+        Kahan32 kp{ks.s.x, ks.c.x};
+        kp.add(__fmaf_rn(vC.c.hi, acc.dA, __fmul_rn(vC.c.lo, acc.dA)));
+        const double gp = __dadd_rn(__dadd_rn(widen(kp.s), -widen(kp.c)), 0.0);
+        const double gk = __dadd_rn(widen(ks.s.y), -widen(ks.c.y));
         if (act) {
             const int c = kb + nx * j + i;
-            // the diagonal's own term v_i dA_i/dp_i joins the compensated FP32
-            // sum last; + 0.0 is the twin's tie correction when no link has
-            // zero flux (it turns a -0 into +0 as that addition does)
-            Kahan32 kp{ks.s.x, ks.c.x};
-            kp.add(__fmaf_rn(vC.c.hi, acc.dA, __fmul_rn(vC.c.lo, acc.dA)));
-            const double gp = __dadd_rn(__dadd_rn(widen(kp.s), -widen(kp.c)), 0.0);
-            const double gk = __dadd_rn(widen(ks.s.y), -widen(ks.c.y));
             gP[c] = gp;
             if (gK) gK[c] = gk;
             if (nonfinite(gp) || nonfinite(gk)) atomicOr(o.status, STATUS_NONFINITE);
@@ -658,17 +665,20 @@ struct YMarch {
                 if (JAC && act) rowbuf[slot_pos(mask, s)] = S[s].Db;
             }
         }
-        const AccF acc = accumulation<CRK>(q, me.p, D.pn, D.mn, me.rho, D.phi0);
+        const AccF acc = accumulation<CRK, true>(q, me.p, D.pn, D.mn, me.rho, D.phi0);
         RowSums out;
-        out.R = __dadd_rn(__dadd_rn(acc.A, widen(ks.s.x)), -widen(ks.c.x));
-        out.diag64 = 0.0;
+        Kahan32 ds{ks.s.y, ks.c.y};
         if (JAC) {
-            Kahan32 ds{ks.s.y, ks.c.y};
             ds.add(acc.dA);
-            out.diag64 = __dadd_rn(widen(ds.s), -widen(ds.c));
             if (act) rowbuf[slot_pos(mask, SLOT_SELF)] = __fsub_rn(ds.s, ds.c);
         }
-        out.bad = nonfinite(out.R) || (JAC && nonfinite(out.diag64));
+        out.R = __dadd_rn(__dadd_rn(acc.A, widen_flush(ks.s.x)), -widen_flush(ks.c.x));
+        out.diag64 = JAC ? __dadd_rn(widen_flush(ds.s), -widen_flush(ds.c)) : 0.0;
+        uint32_t hi = max(abs_hi(out.R), abs_hi(D.mn));
+        if (JAC) hi = max(hi, abs_hi(out.diag64));
+        // `bad` here: the row needs exact conversions
+        out.bad = act && (hi >= kOddHigh || odd_sum(ks.s.x) || nan_sum(ks.s.x) ||
+                          (JAC && (odd_sum(ds.s) || nan_sum(ds.s))));
         return out;
     }
 
@@ -815,7 +825,7 @@ __device__ __forceinline__ void ymarch_tile(const GridGeom& g, const PhysF& q, c
             s2 = st;
             float* buf = stage + ((j - j0) & 1) * BUF;
             M.buffer_ready();
-            if (__any_sync(0xffffffffu, U.tie)) tie_rows |= 1ull << (j - j0);
+            if (__any_sync(0xffffffffu, U.tie || U.odd)) tie_rows |= M_t::rows_before(j - j0);
             U = M.template row<PATH>(j, P, C, N, D, U, buf, rowbase);
             rowbase += M.row_base_step(j);
             P = C;
@@ -834,7 +844,7 @@ __device__ __forceinline__ void ymarch_tile(const GridGeom& g, const PhysF& q, c
             s2 = st;
             float* buf = stage + ((j - j0) & 1) * BUF;
             M.buffer_ready();
-            if (__any_sync(0xffffffffu, U.tie)) tie_rows |= 1ull << (j - j0);
+            if (__any_sync(0xffffffffu, U.tie || U.odd)) tie_rows |= M_t::rows_before(j - j0);
             const bool injk = zint && j > 0 && j + 1 < M.ny;
             if (injk && M.xint) U = M.template row<2>(j, P, C, N, D, U, buf, rowbase);
             else if (injk) U = M.template row<1>(j, P, C, N, D, U, buf, rowbase);
@@ -846,6 +856,7 @@ __device__ __forceinline__ void ymarch_tile(const GridGeom& g, const PhysF& q, c
     }
     asm volatile("cp.async.wait_group 0;" ::: "memory");
     M.drain();
+    if (__any_sync(0xffffffffu, U.odd)) tie_rows |= 1ull << (j1 - 1 - j0);
     if (tie_rows) {  // warp-uniform; every bulk store of the warp has completed
         __syncwarp();
         for (int b = 0; b < 64; ++b)
@@ -923,7 +934,7 @@ __device__ __forceinline__ void ymarch_tile_tma(const GridGeom& g, const PhysF& 
             if (live) {
                 float* buf = stage + ((j - j0) & 1) * BUF;
                 M.buffer_ready();
-                if (__any_sync(0xffffffffu, U.tie)) tie_rows |= 1ull << (j - j0);
+                if (__any_sync(0xffffffffu, U.tie || U.odd)) tie_rows |= M_t::rows_before(j - j0);
                 const bool injk = zint && j > 0 && j + 1 < M.ny;
                 if (injk && M.xint) U = M.template row<2>(j, P, C, N, D, U, buf, rowbase);
                 else if (injk) U = M.template row<1>(j, P, C, N, D, U, buf, rowbase);
@@ -933,6 +944,7 @@ __device__ __forceinline__ void ymarch_tile_tma(const GridGeom& g, const PhysF& 
             P = C;
             C = N;
         }
+        if (__any_sync(0xffffffffu, U.odd)) tie_rows |= 1ull << (j1 - 1 - j0);
     }
     ok = M.tma_drain() && ok;
     M.drain();
