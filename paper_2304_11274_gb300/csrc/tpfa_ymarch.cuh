@@ -634,7 +634,7 @@ struct YMarch {
             ks.add(f2(__fmul_rn(S[s].Da, dv), __fmul_rn(__fmul_rn(S[s].F, ratio), dv)));
             zero_flux |= S[s].F == 0.f;
         }
-        fix = __any_sync(0xffffffffu, zero_flux);
+        fix = __any_sync(0xffffffffu, act && zero_flux);  // lanes past the grid's edge work on zeros
         const AccF acc = accumulation<CRK>(q, C.c.p, D.pn, D.mn, C.c.rho, D.phi0);
         // the diagonal's own term v_i dA_i/dp_i joins the compensated FP32
         // sum last; + 0.0 is the twin's tie correction when no link has
