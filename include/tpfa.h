@@ -347,8 +347,10 @@ int tpfa_slab_exchange(tpfa_handle lower, void* p_lower_dev, tpfa_handle upper, 
  * `warps_per_block` (4 or 8) consecutive z-planes.  Results do not depend on
  * the tiling (every row is summed in the same order); only speed does.  The
  * J w and adjoint marches use the same tiling, with the rows per march
- * halved (down to 8) while the launch has fewer than four blocks per
- * multiprocessor.
+ * halved (down to 8) while the launch has fewer than three or four blocks per
+ * multiprocessor.  Until a tiling is set or autotuned, the marches choose
+ * fewer than the default 32 rows on grids whose blocks would not fill the
+ * GPU.  The FP64 path's tiles follow from the grid alone.
  */
 int tpfa_set_tiling(tpfa_handle h, int rows_per_march, int warps_per_block);
 int tpfa_get_tiling(tpfa_handle h, int* rows_per_march, int* warps_per_block);

@@ -119,7 +119,8 @@ struct tpfa_grid {
     const void* p = nullptr;
     const void* pn = nullptr;
     bool has_state = false;
-    int JY = 32;  // rows per warp march (tpfa_autotune may change it)
+    int JY = 32;  // rows per warp march (tpfa_set_tiling, tpfa_autotune)
+    bool tiling_set = false;  // JY was set by one of them; else the launches choose (rows_for)
     int sms = 0;  // multiprocessors of the grid's device
     int W = 4;    // warps (z-planes) per block
     // a z-slab of a larger grid (tpfa_create_slab): the handle's planes are
@@ -271,8 +272,8 @@ bool tma_ready(tpfa_grid* h) {
 // The library's choice of assembly kernel: the march with two cells per lane
 // on grids at least 256 cells wide, or 128 or 192 wide (whole 64-cell
 // segments), else the one-cell march (the dispatch runs the one-cell march
-// where the two-cell one does not apply: residual-only calls, the FP64 path,
-// odd nx, fields not pair-aligned).  A ragged last segment leaves lanes idle
+// where the two-cell one does not apply: the FP64 path, odd nx, fields not
+// pair-aligned).  A ragged last segment leaves lanes idle
 // and the x-boundary segments cost their lanes masked sums, so narrow grids
 // whose width is not a multiple of 64 do better one cell per lane: measured
 // (G cells/s, one-cell vs two-cell, best rows per march each) 26.4 vs 28.3 at
@@ -284,6 +285,48 @@ bool tma_ready(tpfa_grid* h) {
 AsmKernel auto_kernel(tpfa_grid* h) {
     const int nx = h->nx;
     return nx >= 256 || nx == 128 || nx == 192 ? AsmKernel::XMarch : AsmKernel::YMarch;
+}
+
+// Rows per march of a launch over `planes` planes with `seg`-cell x-segments
+// whose kernel keeps `resident` blocks per multiprocessor: the tiling's if it
+// was set, else the choice of least estimated time.  A march's start costs
+// about 2.5 rows; blocks run in waves of `resident` per multiprocessor, the
+// last of which takes 0.45 of a full one's time and more with the blocks of
+// its busiest multiprocessor; a single wave has nothing to even out its blocks
+// with (8 %).  Large grids get the 32 rows of the default tiling.  Measured
+// against 32 rows everywhere (one-cell R + J, 10 links): 24 x 20 x 16 33.9 ->
+// 10.3 us, 64^3 51 -> 21 us, 201 x 117 x 75 81 -> 72 us; the best of ten fixed
+// choices is at most 20 % better (64^3) and mostly equal or worse.
+int rows_for(const tpfa_grid* h, int seg, int planes, int resident) {
+    if (h->tiling_set || h->sms <= 0) return h->JY;
+    const long long col = (long long)((h->nx + seg - 1) / seg) * ((planes + h->W - 1) / h->W);
+    const long long slots = (long long)h->sms * resident;
+    int best = h->JY;
+    double cost = 1e300;
+    for (int r = h->JY; r >= 2; --r) {
+        const long long blocks = col * ((h->ny + r - 1) / r), full = blocks / slots, rest = blocks % slots;
+        const double busiest = (double)((rest + h->sms - 1) / h->sms) / resident;
+        const double waves = (double)full + (rest ? 0.45 + 0.55 * busiest : 0.0);
+        const double c = (r + 2.5) * (blocks <= slots ? 1.08 * waves : waves);
+        if (c < 0.99 * cost) cost = c, best = r;
+    }
+    return best;
+}
+
+// R alone: the two-cell march on every grid at least one segment wide (nx even;
+// the dispatch falls back).  Measured (G cells/s, 10 links, one-cell vs two-
+// cell): 16.1 vs 27.8 at 64^3, 43.0 vs 58.6 at 160 x 160 x 80, 35.4 vs 50.2 at
+// 224 x 96 x 48, 59.3 vs 91.0 at 512 x 512 x 128.
+AsmKernel residual_kernel(const tpfa_grid* h) { return h->nx >= 64 ? AsmKernel::XMarch : AsmKernel::YMarch; }
+
+// J w: two cells per lane where a row's last segment is not mostly idle (an
+// even number of 32-cell segments) or the row is long.  Measured (10 links, one-
+// cell vs two-cell): 33.2 vs 37.4 at 128^3, 33.0 vs 29.9 at 160 x 160 x 80, 34.1
+// vs 36.8 at 192 x 160 x 80, 27.6 vs 22.2 at 224 x 96 x 48, 40.0 vs 48.3 at
+// 256 x 256 x 128, 44.8 vs 58.0 at 512 x 512 x 128.
+AsmKernel jvp_kernel(const tpfa_grid* h) {
+    const int nx = h->nx;
+    return nx >= 256 || (nx >= 128 && (nx + 31) / 32 % 2 == 0) ? AsmKernel::XMarch : AsmKernel::YMarch;
 }
 
 int launch(tpfa_grid* h, AsmKernel kern, double* R, void* vals, double* diag64, cudaStream_t st, int k0 = 0,
@@ -299,11 +342,13 @@ int launch(tpfa_grid* h, AsmKernel kern, double* R, void* vals, double* diag64, 
                     "the TMA march needs the mixed path, nx a multiple of 4 and 16-byte aligned p and p^n");
     if (h->prec == TPFA_MIXED) {
         AsmOut<float> o{R, static_cast<float*>(vals), diag64, h->status};
+        const bool two = kern == AsmKernel::XMarch && xmarch_ok(h->geom, fields_of<float>(h));
+        const int rows = rows_for(h, two ? 64 : 32, (k1 < 0 ? h->nz : k1) - k0, two && vals ? 3 : 4);
         if (kern == AsmKernel::YMarchTma)
-            e = launch_assemble_mixed_tma(h->geom, h->qf, h->crk, fields_of<float>(h), o, h->tm, h->JY, h->W, st, k0,
+            e = launch_assemble_mixed_tma(h->geom, h->qf, h->crk, fields_of<float>(h), o, h->tm, rows, h->W, st, k0,
                                           k1);
         else
-            e = launch_assemble_mixed(kern, h->geom, h->qf, h->crk, fields_of<float>(h), o, h->JY, h->W, st, k0, k1);
+            e = launch_assemble_mixed(kern, h->geom, h->qf, h->crk, fields_of<float>(h), o, rows, h->W, st, k0, k1);
     } else {
         AsmOut<double> o{R, static_cast<double*>(vals), nullptr, h->status};
         e = launch_assemble_fp64(kern, h->geom, h->qd, h->crk, fields_of<double>(h), o, st, k0, k1);
@@ -325,22 +370,14 @@ int check_handle(tpfa_handle h) {
     return TPFA_OK;
 }
 
-// Rows per march for the J w and adjoint marches: the grid's tiling, halved
-// (down to 8) until the launch has at least four blocks per multiprocessor,
-// so that small grids still fill the GPU.
-int march_rows(const tpfa_grid* h) {
-    int jy = h->JY;
-    const long long bx = (h->nx + 31) / 32, bz = (h->nz + h->W - 1) / h->W;
-    while (jy > 8 && h->sms > 0 && bx * ((h->ny + jy - 1) / jy) * bz < 4LL * h->sms) jy /= 2;
-    return jy;
-}
-
-// The same for the two-cell marches (64-cell x-segments, three blocks of
-// four warps per multiprocessor).
-int march_rows2(const tpfa_grid* h) {
-    int jy = h->JY;
-    const long long bx = (h->nx + 63) / 64, bz = (h->nz + h->W - 1) / h->W;
-    while (jy > 8 && h->sms > 0 && bx * ((h->ny + jy - 1) / jy) * bz < 3LL * h->sms) jy /= 2;
+// Rows per march for the J w and adjoint marches: rows_for's choice, or the
+// tiling's halved (down to 8) until the launch has at least `per_sm` blocks per
+// multiprocessor, so that small grids still fill the GPU.
+int march_rows(const tpfa_grid* h, int seg, int per_sm) {
+    int jy = rows_for(h, seg, h->nz, per_sm);
+    if (!h->tiling_set) return jy;
+    const long long bx = (h->nx + seg - 1) / seg, bz = (h->nz + h->W - 1) / h->W;
+    while (jy > 8 && h->sms > 0 && bx * ((h->ny + jy - 1) / jy) * bz < (long long)per_sm * h->sms) jy /= 2;
     return jy;
 }
 
@@ -734,7 +771,7 @@ int tpfa_assemble_residual(tpfa_handle h, double* R_dev, void* stream) {
     if (!R_dev) return fail(TPFA_ERR_INVALID_ARG, "R must be non-NULL");
     if (!h->has_state) return fail(TPFA_ERR_NO_STATE, "tpfa_set_state has not been called");
     DeviceGuard dg(h->device);
-    return launch(h, auto_kernel(h), R_dev, nullptr, nullptr, static_cast<cudaStream_t>(stream));
+    return launch(h, residual_kernel(h), R_dev, nullptr, nullptr, static_cast<cudaStream_t>(stream));
 }
 
 int tpfa_assemble_jacobian_kernel(tpfa_handle h, tpfa_kernel kern, double* R_dev, void* vals_dev,
@@ -935,7 +972,7 @@ int tpfa_vjp_kernel(tpfa_handle h, tpfa_kernel kern, const double* v_dev, double
     if (h->prec == TPFA_MIXED)
         e = launch_vjp_mixed(k, h->geom, h->qf, h->crk, fields_of<float>(h), (const float*)h->kperm, h->lg, v_dev,
                              h->vsplit, g_p_dev, g_lnk_dev, h->status,
-                             k == AsmKernel::XMarch ? march_rows2(h) : march_rows(h), h->W, st);
+                             k == AsmKernel::XMarch ? march_rows(h, 64, 3) : march_rows(h, 32, 4), h->W, st);
     else
         e = launch_vjp_fp64(h->geom, h->qd, h->crk, fields_of<double>(h), (const double*)h->kperm, h->lgd, v_dev,
                             g_p_dev, g_lnk_dev, h->status, st);
@@ -956,7 +993,7 @@ int tpfa_jvp_kernel(tpfa_handle h, tpfa_kernel kern, const double* w_dev, double
     if (h->slab) return fail(TPFA_ERR_INVALID_ARG, "this call is not available on a slab handle (assembly only)");
     AsmKernel k;
     switch (kern) {
-        case TPFA_KERNEL_AUTO:
+        case TPFA_KERNEL_AUTO: k = jvp_kernel(h); break;
         case TPFA_KERNEL_TILED: k = AsmKernel::YMarch; break;
         case TPFA_KERNEL_NAIVE: k = AsmKernel::Naive; break;
         default: return fail(TPFA_ERR_INVALID_ARG, "bad kernel variant %d", (int)kern);
@@ -966,7 +1003,7 @@ int tpfa_jvp_kernel(tpfa_handle h, tpfa_kernel kern, const double* w_dev, double
     cudaError_t e;
     if (h->prec == TPFA_MIXED)
         e = launch_jvp_mixed(k, h->geom, h->qf, h->crk, fields_of<float>(h), w_dev, Jw_dev, R_dev, h->status,
-                             march_rows(h), h->W, st);
+                             k == AsmKernel::XMarch ? march_rows(h, 64, 3) : march_rows(h, 32, 4), h->W, st);
     else
         e = launch_jvp_fp64(h->geom, h->qd, h->crk, fields_of<double>(h), w_dev, Jw_dev, R_dev, h->status, st);
     if (e != cudaSuccess) return cuda_fail(e, "jvp launch");
@@ -1574,6 +1611,7 @@ int tpfa_set_tiling(tpfa_handle h, int rows_per_march, int warps_per_block) {
         return fail(TPFA_ERR_INVALID_ARG, "rows_per_march must be in [1, 64] and warps_per_block 4 or 8");
     h->JY = rows_per_march;
     h->W = warps_per_block;
+    h->tiling_set = true;
     return TPFA_OK;
 }
 
@@ -1598,6 +1636,7 @@ int tpfa_autotune(tpfa_handle h, const char* cache_path, void* stream) {
     if (it != cache.end()) {
         h->JY = it->second.first;
         h->W = it->second.second;
+        h->tiling_set = true;
         return TPFA_OK;
     }
     cudaStream_t st = static_cast<cudaStream_t>(stream);
@@ -1610,6 +1649,8 @@ int tpfa_autotune(tpfa_handle h, const char* cache_path, void* stream) {
     if (e == cudaSuccess) e = cudaEventCreate(&b);
     float best = 1e30f;
     int bj = h->JY, bw = h->W;
+    const bool was_set = h->tiling_set;
+    h->tiling_set = true;  // the candidates are launched as they are
     for (int jy : kTuneJY) {
         for (int w : kTuneW) {
             if (e != cudaSuccess) break;
@@ -1635,6 +1676,7 @@ int tpfa_autotune(tpfa_handle h, const char* cache_path, void* stream) {
     cudaStreamSynchronize(st);
     h->JY = bj;
     h->W = bw;
+    if (rc || e != cudaSuccess) h->tiling_set = was_set;
     if (rc) return rc;
     if (e != cudaSuccess) return cuda_fail(e, "autotune");
     cache[key] = {bj, bw};

@@ -71,35 +71,38 @@ static cudaError_t launch_ymarch_t(const GridGeom& g, const PhysF& q, const AsmF
 
 // ------------------------------------------------------------------ two cells per lane
 
-template <bool DIAG, bool CRK, int W, bool FAST>
+template <bool DIAG, bool CRK, int W, bool FAST, XOp OP>
 static cudaError_t launch_xmarch_f(const GridGeom& g, const PhysF& q, const AsmFields<float>& f,
                                    const AsmOut<float>& o, int JY, int k0, int k1, cudaStream_t st) {
-    constexpr int smem = xmarch_smem_bytes<DIAG, CRK, W>();
+    constexpr int smem = xmarch_smem_bytes<DIAG, CRK, W, OP>();
     const cudaError_t e =
-        ensure_smem_limit(reinterpret_cast<const void*>(&k_assemble_xmarch<DIAG, CRK, W, FAST>), smem);
+        ensure_smem_limit(reinterpret_cast<const void*>(&k_assemble_xmarch<DIAG, CRK, W, FAST, OP>), smem);
     if (e != cudaSuccess) return e;
     dim3 block(32, W, 1);
     dim3 grid((g.nx + 63) / 64, (g.ny + JY - 1) / JY, (k1 - k0 + W - 1) / W);
-    k_assemble_xmarch<DIAG, CRK, W, FAST><<<grid, block, smem, st>>>(g, q, f, o, JY, k0, k1);
+    k_assemble_xmarch<DIAG, CRK, W, FAST, OP><<<grid, block, smem, st>>>(g, q, f, o, JY, k0, k1);
     return cudaGetLastError();
 }
 
-// FAST: R and diag64 given, and R, diag64 and vals 16-byte aligned.
-template <bool DIAG, bool CRK, int W>
+// FAST: R and (with the Jacobian) diag64 given, and R, diag64 and vals 16-byte
+// aligned.
+template <bool DIAG, bool CRK, int W, XOp OP>
 static cudaError_t launch_xmarch_w(const GridGeom& g, const PhysF& q, const AsmFields<float>& f,
                                    const AsmOut<float>& o, int JY, int k0, int k1, cudaStream_t st) {
-    const bool fast = o.R && o.diag64 &&
+    const bool fast = o.R && (OP == XOp::Res || o.diag64) &&
                       ((reinterpret_cast<uintptr_t>(o.R) | reinterpret_cast<uintptr_t>(o.diag64) |
                         reinterpret_cast<uintptr_t>(o.vals)) & 15u) == 0;
-    if (fast) return launch_xmarch_f<DIAG, CRK, W, true>(g, q, f, o, JY, k0, k1, st);
-    return launch_xmarch_f<DIAG, CRK, W, false>(g, q, f, o, JY, k0, k1, st);
+    if (fast) return launch_xmarch_f<DIAG, CRK, W, true, OP>(g, q, f, o, JY, k0, k1, st);
+    return launch_xmarch_f<DIAG, CRK, W, false, OP>(g, q, f, o, JY, k0, k1, st);
 }
 
-template <bool DIAG, bool CRK>
-static cudaError_t launch_xmarch_t(const GridGeom& g, const PhysF& q, const AsmFields<float>& f,
-                                   const AsmOut<float>& o, int JY, int W, int k0, int k1, cudaStream_t st) {
-    if (W == 8) return launch_xmarch_w<DIAG, CRK, 8>(g, q, f, o, JY, k0, k1, st);
-    return launch_xmarch_w<DIAG, CRK, 4>(g, q, f, o, JY, k0, k1, st);
+template <XOp OP, int W>
+static cudaError_t launch_xmarch_op(const GridGeom& g, const PhysF& q, bool crk, const AsmFields<float>& f,
+                                    const AsmOut<float>& o, int JY, int k0, int k1, cudaStream_t st) {
+    if (g.diag) return crk ? launch_xmarch_w<true, true, W, OP>(g, q, f, o, JY, k0, k1, st)
+                           : launch_xmarch_w<true, false, W, OP>(g, q, f, o, JY, k0, k1, st);
+    return crk ? launch_xmarch_w<false, true, W, OP>(g, q, f, o, JY, k0, k1, st)
+               : launch_xmarch_w<false, false, W, OP>(g, q, f, o, JY, k0, k1, st);
 }
 
 static bool aligned_to(const void* p, uintptr_t a) { return (reinterpret_cast<uintptr_t>(p) & (a - 1)) == 0; }
@@ -230,13 +233,13 @@ cudaError_t launch_assemble_mixed(AsmKernel kern, const GridGeom& g, const PhysF
     const bool jac = o.vals != nullptr;
     clamp_planes(g, k0, k1);
     if (kern == AsmKernel::Naive) return launch_naive<float>(g, q, crk, f, o, st);
-    // two cells per lane: fused R + J on grids with nx even and pair-aligned
-    // fields; otherwise (and for residual-only calls) the one-cell march
-    if (kern == AsmKernel::XMarch && jac && xmarch_ok(g, f)) {
-        if (g.diag) return crk ? launch_xmarch_t<true, true>(g, q, f, o, JY, W, k0, k1, st)
-                               : launch_xmarch_t<true, false>(g, q, f, o, JY, W, k0, k1, st);
-        return crk ? launch_xmarch_t<false, true>(g, q, f, o, JY, W, k0, k1, st)
-                   : launch_xmarch_t<false, false>(g, q, f, o, JY, W, k0, k1, st);
+    // two cells per lane on grids with nx even and pair-aligned fields, else
+    // the one-cell march (R alone: always four warps per block, which its
+    // registers allow four blocks of per multiprocessor)
+    if (kern == AsmKernel::XMarch && xmarch_ok(g, f)) {
+        if (!jac) return launch_xmarch_op<XOp::Res, 4>(g, q, crk, f, o, JY, k0, k1, st);
+        return W == 8 ? launch_xmarch_op<XOp::Jac, 8>(g, q, crk, f, o, JY, k0, k1, st)
+                      : launch_xmarch_op<XOp::Jac, 4>(g, q, crk, f, o, JY, k0, k1, st);
     }
     if (g.diag) {
         if (crk) return jac ? launch_ymarch_t<true, true, true>(g, q, f, o, JY, W, k0, k1, st)

@@ -22,6 +22,7 @@
 
 #include "tpfa_impl.h"
 #include "tpfa_ymarch.cuh"
+#include "tpfa_xmarch.cuh"
 
 namespace tpfa {
 
@@ -196,6 +197,56 @@ cudaError_t launch_jvp_ymarch_t(const GridGeom& g, const PhysF& q, const AsmFiel
     return launch_jvp_ymarch_w<DIAG, CRK, 4>(g, q, f, w, Jw, R, status, JY, st);
 }
 
+// ---------------------------------------------------------------- two-cell J w march (mixed)
+
+constexpr int kXWarps = 4;
+
+template <bool DIAG, bool CRK, XOp OP>
+__global__ void __launch_bounds__(32 * kXWarps, xmarch_blocks(OP, DIAG))
+    k_jvp_xmarch(GridGeom g, PhysF q, AsmFields<float> f, AsmOut<float> o, const double* __restrict__ w,
+                 double* __restrict__ Jw, int JY, bool out16) {
+    using X = XMarch<DIAG, CRK, kXWarps, OP>;
+    extern __shared__ __align__(16) unsigned char smem[];
+    int bx, by, bz;
+    segment_major(bx, by, bz);
+    const int lane = threadIdx.x, wi = threadIdx.y, k = bz * kXWarps + wi;
+    if (k >= g.nz) return;  // warp-uniform
+    XState<DIAG, CRK, kXWarps, false, OP> M(
+        g, q, f, o, reinterpret_cast<float*>(smem) + wi * X::smem_floats_per_warp(), lane, k, bx);
+    M.wv = w;
+    M.Jw = Jw;
+    M.r16 = out16;
+    const int j0 = by * JY;
+    const unsigned long long rows = xmarch_rows(M, j0, min(j0 + JY, g.ny));
+    if (rows) {  // warp-uniform
+        for (int b = 0; b < 64; ++b)
+            if (((rows >> b) & 1ull) && M.act) {
+                jvp_row<CRK>(g, q, f, w, Jw, o.R, o.status, M.ia, j0 + b, k);
+                jvp_row<CRK>(g, q, f, w, Jw, o.R, o.status, M.ib, j0 + b, k);
+            }
+    }
+}
+
+template <bool DIAG, bool CRK, XOp OP>
+cudaError_t launch_jvp_xmarch_t(const GridGeom& g, const PhysF& q, const AsmFields<float>& f, const double* w,
+                                double* Jw, double* R, unsigned int* status, int JY, cudaStream_t st) {
+    constexpr int smem = xmarch_smem_bytes<DIAG, CRK, kXWarps, OP>();
+    const cudaError_t e = ensure_smem_limit(reinterpret_cast<const void*>(&k_jvp_xmarch<DIAG, CRK, OP>), smem);
+    if (e != cudaSuccess) return e;
+    const bool out16 = ((reinterpret_cast<uintptr_t>(Jw) | reinterpret_cast<uintptr_t>(R)) & 15u) == 0;
+    dim3 grid((g.nx + 63) / 64, (g.ny + JY - 1) / JY, (g.nz + kXWarps - 1) / kXWarps);
+    AsmOut<float> o{R, nullptr, nullptr, status};
+    k_jvp_xmarch<DIAG, CRK, OP><<<grid, dim3(32, kXWarps, 1), smem, st>>>(g, q, f, o, w, Jw, JY, out16);
+    return cudaGetLastError();
+}
+
+template <bool DIAG, bool CRK>
+cudaError_t launch_jvp_xmarch(const GridGeom& g, const PhysF& q, const AsmFields<float>& f, const double* w, double* Jw,
+                              double* R, unsigned int* status, int JY, cudaStream_t st) {
+    return R ? launch_jvp_xmarch_t<DIAG, CRK, XOp::JvpR>(g, q, f, w, Jw, R, status, JY, st)
+             : launch_jvp_xmarch_t<DIAG, CRK, XOp::Jvp>(g, q, f, w, Jw, R, status, JY, st);
+}
+
 cudaError_t launch_jvp_naive(const GridGeom& g, const PhysF& q, bool crk, const AsmFields<float>& f, const double* w,
                              double* Jw, double* R, unsigned int* status, cudaStream_t st) {
     dim3 block(32, 8, 1);
@@ -211,6 +262,13 @@ cudaError_t launch_jvp_mixed(AsmKernel kern, const GridGeom& g, const PhysF& q, 
                              const double* w, double* Jw, double* R, unsigned int* status, int JY, int W,
                              cudaStream_t st) {
     if (kern == AsmKernel::Naive) return launch_jvp_naive(g, q, crk, f, w, Jw, R, status, st);
+    // two cells per lane: nx even, pair-aligned fields, w 16-byte aligned
+    if (kern == AsmKernel::XMarch && xmarch_ok(g, f) && (reinterpret_cast<uintptr_t>(w) & 15u) == 0) {
+        if (g.diag) return crk ? launch_jvp_xmarch<true, true>(g, q, f, w, Jw, R, status, JY, st)
+                               : launch_jvp_xmarch<true, false>(g, q, f, w, Jw, R, status, JY, st);
+        return crk ? launch_jvp_xmarch<false, true>(g, q, f, w, Jw, R, status, JY, st)
+                   : launch_jvp_xmarch<false, false>(g, q, f, w, Jw, R, status, JY, st);
+    }
     if (g.diag) {
         return crk ? launch_jvp_ymarch_t<true, true>(g, q, f, w, Jw, R, status, JY, W, st)
                    : launch_jvp_ymarch_t<true, false>(g, q, f, w, Jw, R, status, JY, W, st);

@@ -123,14 +123,21 @@ __device__ __forceinline__ float2 accumulation2(const PhysF& q, float2 p, float2
     }
 }
 
-template <bool DIAG, bool CRK, int W>
+// What the march computes per row: R and the Jacobian row; R alone; J w; J w
+// and R.
+enum class XOp { Jac, Res, Jvp, JvpR };
+
+template <bool DIAG, bool CRK, int W, XOp OP = XOp::Jac>
 struct XMarch {
+    static constexpr bool JAC = OP == XOp::Jac, JV = OP == XOp::Jvp || OP == XOp::JvpR;
     // ---- ring layout (floats, per warp and slot)
     enum { P_P, P_Z, P_TX, P_TY, P_TZ, P_TPP, P_TMP, P_PN, P_PZM, P_ZZM, P_TZM, P_PZP, P_ZZP, P_PHI };
     static constexpr int NP = CRK ? P_PHI + 1 : P_PHI;  // pair fields, 64 floats each
     static constexpr int OFF_MN = NP * 64;              // 32 lanes x 2 doubles
     static constexpr int OFF_H = OFF_MN + 128;          // halo singles: p, z, T1, T2 x {lane 0, lane 31}
-    static constexpr int SLOT = OFF_H + 8;              // floats per slot (a multiple of 4)
+    static constexpr int OFF_W = OFF_H + 8;             // J w: w of the row, of planes k - 1 and k + 1 (32 x 2
+                                                        // doubles each), w of the halo cells (2 doubles)
+    static constexpr int SLOT = OFF_W + (JV ? 3 * 128 + 4 : 0);  // floats per slot (a multiple of 4)
     static constexpr int RING = 2;
     static constexpr int L = DIAG ? 11 : 7;             // interior row length
     static constexpr int LX = DIAG ? 3 : 1;             // x-side links of a row per side
@@ -140,12 +147,12 @@ struct XMarch {
     static constexpr unsigned kXPlus = 0x248u;  // slots 3, 6, 9
     static_assert(SLOT % 4 == 0, "16-byte aligned slots");
 
-    static constexpr int smem_floats_per_warp() { return RING * SLOT + 2 * BUF; }
+    static constexpr int smem_floats_per_warp() { return RING * SLOT + (JAC ? 2 * BUF : 0); }
 };
 
-template <bool DIAG, bool CRK, int W>
+template <bool DIAG, bool CRK, int W, XOp OP = XOp::Jac>
 constexpr int xmarch_smem_bytes() {
-    return W * XMarch<DIAG, CRK, W>::smem_floats_per_warp() * 4;
+    return W * XMarch<DIAG, CRK, W, OP>::smem_floats_per_warp() * 4;
 }
 
 __device__ __forceinline__ void cpa8(float* dst, const float* src, bool valid) {
@@ -165,6 +172,13 @@ __device__ __forceinline__ void cpa4_if(float* dst, const float* src, bool valid
                  "l"(src), "r"(valid ? 4 : 0), "r"((unsigned)lane_on)
                  : "memory");
 }
+__device__ __forceinline__ void cpa8d_if(double* dst, const double* src, bool valid, bool lane_on) {
+    const uint32_t d = (uint32_t)__cvta_generic_to_shared(dst);
+    asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.u32 q, %3, 0;\n\t"
+                 "@q cp.async.ca.shared.global [%0], [%1], 8, %2;\n\t}" ::"r"(d),
+                 "l"(src), "r"(valid ? 8 : 0), "r"((unsigned)lane_on)
+                 : "memory");
+}
 __device__ __forceinline__ void cpa16(void* dst, const void* src, bool valid) {
     const uint32_t d = (uint32_t)__cvta_generic_to_shared(dst);
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(d), "l"(src), "r"(valid ? 16 : 0) : "memory");
@@ -176,32 +190,38 @@ __device__ __forceinline__ void cpa16(void* dst, const void* src, bool valid) {
 // lacks slots 1, 4, 7; cell b at i = nx - 1 lacks 3, 6, 9); PATH 0: per-cell
 // masks.  Each half of the Kahan pairs is the cell's own sum in slot order,
 // so the sums equal assemble_row's bit for bit.
-template <bool DIAG, int PATH>
+template <bool DIAG, int PATH, XOp OP>
 struct XRow {
     static constexpr unsigned kFull = DIAG ? 0x7ffu : 0x575u;
     static constexpr unsigned kXMinus = 0x92u & kFull;  // slots 1, 4, 7
     static constexpr unsigned kXPlus = 0x248u & kFull;  // slots 3, 6, 9
     static constexpr int L = DIAG ? 11 : 7;
-    Kahan2 kr, kd;       // residual (F) and diagonal (dF/dp_K) sums of a and b
+    static constexpr bool JAC = OP == XOp::Jac, RES = OP != XOp::Jvp, JV = OP == XOp::Jvp || OP == XOp::JvpR;
+    Kahan2 kr, kd;       // residual (F) and diagonal (dF/dp_K) or J w sums of a and b
     Kahan32 ka, kb, kda, kdb;  // PATH 0: the same sums per cell
     float* ra;           // staging position of row a's first value
     float* rb;           // ... of row b's
     unsigned ma, mb;     // PATH 0: slot masks
     bool bnd_a, bnd_b;   // PATH 1: a at i = 0, b at i = nx - 1
+    float2 wc;           // J w: w of a and b
 
     template <int S>
     static constexpr int full_pos() {
         return __builtin_popcount(kFull & ((1u << S) - 1u));
     }
+    // One slot of both cells; wl: w of the two neighbours (J w).  The second
+    // sum takes dF/dp_K, or for J w dF/dp_K w_K + dF/dp_L w_L.
     template <int S>
-    __device__ __forceinline__ void put(const LinkOut<float>& a, const LinkOut<float>& b, bool act) {
+    __device__ __forceinline__ void put(const LinkOut<float>& a, const LinkOut<float>& b, bool act, float2 wl) {
         static_assert(S != SLOT_SELF, "the diagonal is not a link");
         if constexpr (!((kFull >> S) & 1u)) return;
-        const float2 F = f2(a.F, b.F), Da = f2(a.Da, b.Da);
+        const float2 F = f2(a.F, b.F);
+        float2 D = f2(a.Da, b.Da);
+        if constexpr (JV) D = __ffma2_rn(D, wc, __fmul2_rn(f2(a.Db, b.Db), wl));
         if constexpr (PATH == 2) {
-            kr.add(F);
-            kd.add(Da);
-            if (act) {
+            if (RES) kr.add(F);
+            if (JAC || JV) kd.add(D);
+            if (JAC && act) {
                 ra[full_pos<S>()] = a.Db;
                 rb[full_pos<S>()] = b.Db;
             }
@@ -211,13 +231,13 @@ struct XRow {
             constexpr int sb = __builtin_popcount(kXPlus & ((1u << S) - 1u));
             const bool va = !(xm && bnd_a), vb = !(xp && bnd_b);
             if constexpr (xm || xp) {
-                kahan2_masked(kr, F, va, vb);
-                kahan2_masked(kd, Da, va, vb);
+                if (RES) kahan2_masked(kr, F, va, vb);
+                if (JAC || JV) kahan2_masked(kd, D, va, vb);
             } else {
-                kr.add(F);
-                kd.add(Da);
+                if (RES) kr.add(F);
+                if (JAC || JV) kd.add(D);
             }
-            if (act) {
+            if (JAC && act) {
                 if (va) ra[full_pos<S>() - (bnd_a ? sa : 0)] = a.Db;
                 if (vb) rb[full_pos<S>() - (bnd_b ? sb : 0)] = b.Db;
             }
@@ -225,14 +245,14 @@ struct XRow {
             // general rows: each cell's own scalar sums, skipping its absent slots
             const bool va = (ma >> S) & 1u, vb = (mb >> S) & 1u;
             if (va) {
-                ka.add(a.F);
-                kda.add(a.Da);
-                if (act) ra[slot_pos(ma, S)] = a.Db;
+                if (RES) ka.add(F.x);
+                if (JAC || JV) kda.add(D.x);
+                if (JAC && act) ra[slot_pos(ma, S)] = a.Db;
             }
             if (vb) {
-                kb.add(b.F);
-                kdb.add(b.Da);
-                if (act) rb[slot_pos(mb, S)] = b.Db;
+                if (RES) kb.add(F.y);
+                if (JAC || JV) kdb.add(D.y);
+                if (JAC && act) rb[slot_pos(mb, S)] = b.Db;
             }
         }
     }
@@ -264,9 +284,16 @@ struct XRow {
 };
 
 // Per-warp state of the two-cell march.
-template <bool DIAG, bool CRK, int W, bool FAST>
+// w of one row (FP32): the lane's two cells, the cells left and right of them.
+struct XW {
+    float2 c;
+    float m, p;
+};
+
+template <bool DIAG, bool CRK, int W, bool FAST, XOp OP = XOp::Jac>
 struct XState {
-    using X = XMarch<DIAG, CRK, W>;
+    using X = XMarch<DIAG, CRK, W, OP>;
+    static constexpr bool JAC = X::JAC, JV = X::JV, RES = OP != XOp::Jvp;
     const GridGeom& g;
     const PhysF& q;
     const AsmFields<float>& f;
@@ -283,6 +310,11 @@ struct XState {
     CellVal<float> Ch, Ph, Cm, Cp;
     Link2 Uy, Uxy, Umxy;
     bool tie_up;
+    // J w: the direction, the output, w of rows j - 1 and j
+    const double* wv = nullptr;
+    double* Jw = nullptr;
+    XW wP, wC;
+    bool w_odd = false;  // a w of rows up to j + 1 lies outside the FP32 normal range
 
     __device__ __forceinline__ XState(const GridGeom& g_, const PhysF& q_, const AsmFields<float>& f_,
                                       const AsmOut<float>& o_, float* ring_, int lane_, int k_, int bx)
@@ -304,6 +336,7 @@ struct XState {
         okb = act && ib + 1 < nx;  // b's +x and +x+y links exist
         oka = act && ia > 0;       // a's -x+y link exists
         v16 = FAST || (reinterpret_cast<uintptr_t>(o.vals) & 15u) == 0;
+        // (the J w march's caller sets it, from R and J w)
         r16 = FAST || ((reinterpret_cast<uintptr_t>(o.R) | reinterpret_cast<uintptr_t>(o.diag64)) & 15u) == 0;
         const long long Ex = 2LL * (nx - 1), Ey = 2LL * (ny - 1), D = g.diag;
         const long long plane = (long long)nx * ny + Ex * ny + (long long)nx * Ey + D * Ex * Ey;
@@ -353,7 +386,37 @@ struct XState {
                 cpa4_if(H + 6, (hl ? f.Tmp : f.Tpp) + (t2 ? ch - nx : 0), t2, hlane);
             }
         }
+        if constexpr (JV) {
+            double* Wd = reinterpret_cast<double*>(S + X::OFF_W);
+            cpa16(Wd + 2 * lane, wv + c, a);
+            cpa16(Wd + 64 + 2 * lane, wv + cm, a && zm);
+            cpa16(Wd + 128 + 2 * lane, wv + cp, a && zp);
+            const int ch = kb + nx * (rv ? r : 0) + (hact ? ih : 0);
+            cpa8d_if(Wd + 192 + (hl ? 1 : 0), wv + ch, rv && hact, lane == 0 || hl);
+        }
         asm volatile("cp.async.commit_group;" ::: "memory");
+    }
+    // w as FP32 (truncated), and whether the cheap narrowing is exact for it
+    __device__ __forceinline__ float narrow_w(double x) {
+        const uint32_t a = abs_hi(x);
+        w_odd = w_odd || (a - 0x38100000u >= 0x0fe00000u && a != 0u);
+        return narrow_flush(x);
+    }
+    __device__ __forceinline__ float2 w_pair(int sl, int plane) {
+        const double2 d = *reinterpret_cast<const double2*>(ring + sl * X::SLOT + X::OFF_W + 128 * plane + 4 * lane);
+        return f2(narrow_w(d.x), narrow_w(d.y));
+    }
+    __device__ __forceinline__ XW w_row(int sl) {
+        XW r;
+        r.c = w_pair(sl, 0);
+        const double* Wh = reinterpret_cast<const double*>(ring + sl * X::SLOT + X::OFF_W) + 192;
+        float h = 0.f;
+        if (hact) h = narrow_w(Wh[hl ? 1 : 0]);
+        r.m = __shfl_up_sync(0xffffffffu, r.c.y, 1);
+        r.p = __shfl_down_sync(0xffffffffu, r.c.x, 1);
+        if (lane == 0) r.m = h;
+        if (hl) r.p = h;
+        return r;
     }
     __device__ __forceinline__ float2 pair_at(int sl, int fld) const {
         return *reinterpret_cast<const float2*>(ring + sl * X::SLOT + fld * 64 + 2 * lane);
@@ -393,6 +456,20 @@ struct XState {
     static __device__ __forceinline__ CellPair shift_right(const CellVal<float>& prv, const CellPair& c) {
         return CellPair{f2(prv.p, c.p.x), f2(prv.z, c.z.x), f2(prv.rho, c.rho.x), f2(prv.drho, c.drho.x)};
     }
+    // The left (right) neighbour lane's link of its cell b (a), seen from this
+    // lane's cell a (b).  R alone needs the flux only.
+    static __device__ __forceinline__ LinkOut<float> from_left(const Link2& l) {
+        const float f = __shfl_up_sync(0xffffffffu, l.F.y, 1);
+        if constexpr (!JAC && !JV) return flip(f, 0.f, 0.f);
+        const float a = __shfl_up_sync(0xffffffffu, l.Da.y, 1), b = __shfl_up_sync(0xffffffffu, l.Db.y, 1);
+        return flip(f, a, b);
+    }
+    static __device__ __forceinline__ LinkOut<float> from_right(const Link2& l) {
+        const float f = __shfl_down_sync(0xffffffffu, l.F.x, 1);
+        if constexpr (!JAC && !JV) return flip(f, 0.f, 0.f);
+        const float a = __shfl_down_sync(0xffffffffu, l.Da.x, 1), b = __shfl_down_sync(0xffffffffu, l.Db.x, 1);
+        return flip(f, a, b);
+    }
     static __device__ __forceinline__ LinkOut<float> half(const Link2& l, int h) {
         return h == 0 ? LinkOut<float>{l.F.x, l.Da.x, l.Db.x} : LinkOut<float>{l.F.y, l.Da.y, l.Db.y};
     }
@@ -417,6 +494,10 @@ struct XState {
                  (Uy.F.x == 0.f || Uy.F.y == 0.f ||
                   (DIAG && (Uxy.F.x == 0.f || (okb && Uxy.F.y == 0.f) || (oka && Umxy.F.x == 0.f) ||
                             Umxy.F.y == 0.f)));
+        if constexpr (JV) {
+            wP = w_row(0);
+            wC = w_row(1);
+        }
         issue(j0 + 1, 0);
     }
 
@@ -438,13 +519,21 @@ struct XState {
         const float2 pzp = pair_at(sD, X::P_PZP), zzp = pair_at(sD, X::P_ZZP);
         const double2 mn = *reinterpret_cast<const double2*>(ring + sD * X::SLOT + X::OFF_MN + 4 * lane);
         const float hT1 = halo_at(sD, 2), hT2 = DIAG ? halo_at(sD, 3) : 0.f;
+        XW wN{};
+        float2 wzm = f2(0.f), wzp = f2(0.f);
+        if constexpr (JV) {
+            wN = w_row(sN);
+            wzm = w_pair(sD, 1);
+            wzp = w_pair(sD, 2);
+        }
         issue(j + 2, sD);
 
         // ---- CSR offsets of the two rows
         constexpr int L = X::L, LX = X::LX;
         const int ey = PATH >= 1 ? 2 : axis_links(j, ny);
         const int per = 1 + ey + ez, perx = 1 + g.diag * ey;
-        XRow<DIAG, PATH> R;
+        XRow<DIAG, PATH, OP> R;
+        R.wc = wC.c;
         int off_a, len_a;
         if constexpr (PATH == 2) {
             off_a = 2 * lane * L;
@@ -462,13 +551,15 @@ struct XState {
         }
         const long long seg = base_k + rowbase + (long long)i0 * per + (long long)Sx0 * perx;
         const int aoff = (int)(seg & 3);
-        R.ra = buf + aoff + off_a;
-        R.rb = R.ra + len_a;
-        // the bulk copy issued from this buffer two steps ago has read it
-        // (lane 0 issued it; in the other lanes, which have no bulk groups, the
-        // wait returns at once)
-        if (v16) asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory");
-        __syncwarp();
+        if constexpr (JAC) {
+            R.ra = buf + aoff + off_a;
+            R.rb = R.ra + len_a;
+            // the bulk copy issued from this buffer two steps ago has read it
+            // (lane 0 issued it; in the other lanes, which have no bulk groups,
+            // the wait returns at once)
+            if (v16) asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory");
+            __syncwarp();
+        }
 
         // ---- links and slot values, in slot order
         {
@@ -478,7 +569,7 @@ struct XState {
                 Zm = pair2(a0, b0);
             }
             const Link2 LZM = link_pp(q, tzm, Cc, Zm);
-            R.template put<0>(half(LZM, 0), half(LZM, 1), on);
+            R.template put<0>(half(LZM, 0), half(LZM, 1), on, wzm);
         }
         // the segment's halo links: lane 0 -> a's -x (halo of row j) and -x-y
         // (halo of row j-1); lane 31 -> b's +x-y (halo of row j-1)
@@ -489,36 +580,33 @@ struct XState {
             LH = link_pp(q, hl ? f2(hT2, 0.f) : f2(hT1, hT2), pair2(own, own), pair2(hl ? Ph : Ch, Ph));
         }
         if (DIAG) {
-            const float f1 = __shfl_up_sync(0xffffffffu, Uxy.F.y, 1), a1 = __shfl_up_sync(0xffffffffu, Uxy.Da.y, 1),
-                        b1 = __shfl_up_sync(0xffffffffu, Uxy.Db.y, 1);
-            R.template put<1>(lane == 0 ? half(LH, 1) : flip(f1, a1, b1), flip(Uxy.F.x, Uxy.Da.x, Uxy.Db.x), on);
+            const LinkOut<float> l1 = from_left(Uxy);  // every lane shuffles
+            R.template put<1>(lane == 0 ? half(LH, 1) : l1, flip(Uxy.F.x, Uxy.Da.x, Uxy.Db.x), on,
+                              f2(wP.m, wP.c.x));
         }
-        R.template put<2>(flip(Uy.F.x, Uy.Da.x, Uy.Db.x), flip(Uy.F.y, Uy.Da.y, Uy.Db.y), on);
+        R.template put<2>(flip(Uy.F.x, Uy.Da.x, Uy.Db.x), flip(Uy.F.y, Uy.Da.y, Uy.Db.y), on, wP.c);
         if (DIAG) {
-            const float f3 = __shfl_down_sync(0xffffffffu, Umxy.F.x, 1),
-                        a3 = __shfl_down_sync(0xffffffffu, Umxy.Da.x, 1),
-                        b3 = __shfl_down_sync(0xffffffffu, Umxy.Db.x, 1);
-            R.template put<3>(flip(Umxy.F.y, Umxy.Da.y, Umxy.Db.y), hl ? half(LH, 0) : flip(f3, a3, b3), on);
+            const LinkOut<float> l3 = from_right(Umxy);
+            R.template put<3>(flip(Umxy.F.y, Umxy.Da.y, Umxy.Db.y), hl ? half(LH, 0) : l3, on,
+                              f2(wP.c.y, wP.p));
         }
         const Link2 LX_ = link_pp(q, Tx, Cc, shift_left(Cc, Cp));
-        {
-            const float f4 = __shfl_up_sync(0xffffffffu, LX_.F.y, 1), a4 = __shfl_up_sync(0xffffffffu, LX_.Da.y, 1),
-                        b4 = __shfl_up_sync(0xffffffffu, LX_.Db.y, 1);
-            R.template put<4>(lane == 0 ? half(LH, 0) : flip(f4, a4, b4), flip(LX_.F.x, LX_.Da.x, LX_.Db.x), on);
-        }
-        R.template put<6>(half(LX_, 0), half(LX_, 1), on);
+        const LinkOut<float> l4 = from_left(LX_);
+        R.template put<4>(lane == 0 ? half(LH, 0) : l4, flip(LX_.F.x, LX_.Da.x, LX_.Db.x), on,
+                          f2(wC.m, wC.c.x));
+        R.template put<6>(half(LX_, 0), half(LX_, 1), on, f2(wC.c.y, wC.p));
         CellVal<float> Nm, Np;
         neighbours(Nc, Nh, Nm, Np);
         Link2 LMXY, LXY;
         if (DIAG) {
             LMXY = link_pp(q, Tmp, Cc, shift_right(Nm, Nc));
-            R.template put<7>(half(LMXY, 0), half(LMXY, 1), on);
+            R.template put<7>(half(LMXY, 0), half(LMXY, 1), on, f2(wN.m, wN.c.x));
         }
         const Link2 LY = link_pp(q, Ty, Cc, Nc);
-        R.template put<8>(half(LY, 0), half(LY, 1), on);
+        R.template put<8>(half(LY, 0), half(LY, 1), on, wN.c);
         if (DIAG) {
             LXY = link_pp(q, Tpp, Cc, shift_left(Nc, Np));
-            R.template put<9>(half(LXY, 0), half(LXY, 1), on);
+            R.template put<9>(half(LXY, 0), half(LXY, 1), on, f2(wN.c.y, wN.p));
         }
         {
             CellPair Zp;
@@ -527,7 +615,7 @@ struct XState {
                 Zp = pair2(a1, b1);
             }
             const Link2 LZP = link_pp(q, Tz, Cc, Zp);
-            R.template put<10>(half(LZP, 0), half(LZP, 1), on);
+            R.template put<10>(half(LZP, 0), half(LZP, 1), on, wzp);
         }
 
         // ties on this row's reused links: the previous step's up-links and
@@ -535,8 +623,9 @@ struct XState {
         // (on an interior segment every lane's +x and diagonal links exist)
         const bool kb2 = PATH == 2 ? true : okb, ka2 = PATH == 2 ? true : oka;
         const bool tie_x = on && (LX_.F.x == 0.f || (kb2 && LX_.F.y == 0.f));
-        const bool tie_here = tie_up || tie_x;
-        tie_up = on && (LY.F.x == 0.f || LY.F.y == 0.f ||
+        // (a tie's flux is zero from either end: R alone needs none of this)
+        const bool tie_here = (JAC || JV) && (tie_up || tie_x);
+        if (JAC || JV) tie_up = on && (LY.F.x == 0.f || LY.F.y == 0.f ||
                          (DIAG && (LXY.F.x == 0.f || (kb2 && LXY.F.y == 0.f) || (ka2 && LMXY.F.x == 0.f) ||
                                    LMXY.F.y == 0.f)));
 
@@ -546,35 +635,50 @@ struct XState {
         const float2 dA = accumulation2<CRK>(q, Cc.p, pn, mn, Cc.rho, phi, Aa, Ab);
         const double Ra = __dadd_rn(__dadd_rn(Aa, widen_flush(R.kr.s.x)), -widen_flush(R.kr.c.x));
         const double Rb = __dadd_rn(__dadd_rn(Ab, widen_flush(R.kr.s.y)), -widen_flush(R.kr.c.y));
-        Kahan2 dd = R.kd;  // the diagonals: dA joins each compensated sum last
-        dd.add(dA);
-        const double Da64 = __dadd_rn(widen_flush(dd.s.x), -widen_flush(dd.c.x));
-        const double Db64 = __dadd_rn(widen_flush(dd.s.y), -widen_flush(dd.c.y));
-        const float2 dg = __ffma2_rn(dd.c, f2(-1.f), dd.s);  // s - c, the FP32 diagonal values
-        R.put_diag(dg.x, dg.y, on);
+        Kahan2 dd = R.kd;  // dA (J w: times w) joins the second sums last
+        double Da64 = 0.0, Db64 = 0.0;
+        if constexpr (JAC) {
+            dd.add(dA);
+            Da64 = __dadd_rn(widen_flush(dd.s.x), -widen_flush(dd.c.x));
+            Db64 = __dadd_rn(widen_flush(dd.s.y), -widen_flush(dd.c.y));
+            const float2 dg = __ffma2_rn(dd.c, f2(-1.f), dd.s);  // s - c, the FP32 diagonal values
+            R.put_diag(dg.x, dg.y, on);
+        } else if constexpr (JV) {
+            // exact conversions: J w scales with w, which may be small everywhere
+            dd.add(__fmul2_rn(dA, wC.c));
+            Da64 = __dadd_rn(widen(dd.s.x), -widen(dd.c.x));
+            Db64 = __dadd_rn(widen(dd.s.y), -widen(dd.c.y));
+        }
         // rows that need exact conversions (odd_sum; min_abs is NaN if a sum is)
-        const float rmin = min_abs(R.kr.s.x, R.kr.s.y), dmin = min_abs(dd.s.x, dd.s.y);
-        const uint32_t hi = max(max(max(abs_hi(Ra), abs_hi(Rb)), max(abs_hi(Da64), abs_hi(Db64))),
-                                max(abs_hi(mn.x), abs_hi(mn.y)));
-        bool odd = hi >= kOddHigh;
-        if (!(rmin >= 0x1p-60f && dmin >= 0x1p-60f))  // small, zero or NaN: which
-            odd = odd || odd_sum(R.kr.s.x) || odd_sum(R.kr.s.y) || odd_sum(dd.s.x) || odd_sum(dd.s.y) ||
-                  nan_sum(rmin) || nan_sum(dmin);
+        uint32_t hi = max(abs_hi(mn.x), abs_hi(mn.y));
+        float rmin = 1.f, dmin = 1.f;
+        if (RES) hi = max(hi, max(abs_hi(Ra), abs_hi(Rb))), rmin = min_abs(R.kr.s.x, R.kr.s.y);
+        if (JAC || JV) hi = max(hi, max(abs_hi(Da64), abs_hi(Db64)));
+        if (JAC) dmin = min_abs(dd.s.x, dd.s.y);
+        bool odd = hi >= kOddHigh || (JV && w_odd);
+        if (!(rmin >= 0x1p-60f && dmin >= 0x1p-60f)) {  // small, zero or NaN: which
+            if (RES) odd = odd || odd_sum(R.kr.s.x) || odd_sum(R.kr.s.y) || nan_sum(rmin);
+            if (JAC) odd = odd || odd_sum(dd.s.x) || odd_sum(dd.s.y) || nan_sum(dmin);
+        }
         const bool tie = __any_sync(0xffffffffu, tie_here || (on && odd));
         if (on) {
             const int c = kb + nx * j + ia;
-            if (FAST || o.R) {
+            if (RES && (FAST || o.R)) {
                 if (r16) *reinterpret_cast<double2*>(o.R + c) = make_double2(Ra, Rb);
                 else o.R[c] = Ra, o.R[c + 1] = Rb;
             }
-            if (FAST || o.diag64) {
+            if (JAC && (FAST || o.diag64)) {
                 if (r16) *reinterpret_cast<double2*>(o.diag64 + c) = make_double2(Da64, Db64);
                 else o.diag64[c] = Da64, o.diag64[c + 1] = Db64;
+            }
+            if (JV) {
+                if (r16) *reinterpret_cast<double2*>(Jw + c) = make_double2(Da64, Db64);
+                else Jw[c] = Da64, Jw[c + 1] = Db64;
             }
         }
 
         // ---- the segment's CSR values: one bulk copy (ends by single lanes)
-        {
+        if constexpr (JAC) {
             const int iend = min(i0 + 64, nx);
             int seg_len;
             if constexpr (PATH == 2) seg_len = 64 * L;
@@ -619,6 +723,10 @@ struct XState {
             Uxy = LXY;
             Umxy = LMXY;
         }
+        if constexpr (JV) {
+            wP = wC;
+            wC = wN;
+        }
         return tie;
     }
 };
@@ -650,25 +758,14 @@ __device__ __forceinline__ void xmarch_row(State& M, int j, int j0, int& rowbase
     rowbase += M.rowA + (PATH >= 1 ? 2 : axis_links(j, M.ny)) * M.rowB;
 }
 
-// One block's work: x-segment bx (64 cells), y-run by, z-block bz.  Shared by
-// the single-grid kernel and the persistent ensemble kernel.  FAST: R and
-// diag64 given and, with vals, 16-byte aligned (checked by the launcher).
-template <bool DIAG, bool CRK, int W, bool FAST>
-__device__ __forceinline__ void xmarch_tile(const GridGeom& g, const PhysF& q, const AsmFields<float>& f,
-                                            const AsmOut<float>& o, int JY, int bx, int by, int bz,
-                                            unsigned char* smem, int kbase = 0, int kend = -1) {
-    using X = XMarch<DIAG, CRK, W>;
-    const int lane = threadIdx.x, w = threadIdx.y;
-    const int k = kbase + bz * W + w;  // planes [kbase, kend) of the grid (all by default)
-    if (k >= (kend < 0 ? g.nz : kend)) return;  // warp-uniform
-    XState<DIAG, CRK, W, FAST> M(g, q, f, o, reinterpret_cast<float*>(smem) + w * X::smem_floats_per_warp(), lane,
-                                 k, bx);
-    const int j0 = by * JY;
-    const int j1 = min(j0 + JY, g.ny);
+// The march of one warp over rows [j0, j1); returns the rows to recompute.
+template <class State>
+__device__ __forceinline__ unsigned long long xmarch_rows(State& M, int j0, int j1) {
+    const int ny = M.ny;
     const bool zint = M.zm && M.zp;
-    const bool xint = M.i0 > 0 && M.i0 + 64 < g.nx;
+    const bool xint = M.i0 > 0 && M.i0 + 64 < M.nx;
     M.start(j0);
-    int rowbase = j0 * M.rowA + (int)axis_links_before(j0, g.ny) * M.rowB;
+    int rowbase = j0 * M.rowA + (int)axis_links_before(j0, ny) * M.rowB;
     unsigned long long tie_rows = 0ull;
     // the warp's path is fixed for its interior rows (j and k interior): the
     // rows at j = 0 and j = ny - 1, and every row of a boundary plane, take
@@ -678,7 +775,7 @@ __device__ __forceinline__ void xmarch_tile(const GridGeom& g, const PhysF& q, c
     int j = j0;
     if (zint) {
         if (j == 0 && j < j1) xmarch_row<0>(M, j++, j0, rowbase, tie_rows);
-        const int jend = min(j1, g.ny - 1);
+        const int jend = min(j1, ny - 1);
         if (xint) {
 #pragma unroll 1
             for (; j < jend; ++j) xmarch_row<2>(M, j, j0, rowbase, tie_rows);
@@ -689,24 +786,48 @@ __device__ __forceinline__ void xmarch_tile(const GridGeom& g, const PhysF& q, c
     }
     for (; j < j1; ++j) xmarch_row<0>(M, j, j0, rowbase, tie_rows);
     asm volatile("cp.async.wait_group 0;" ::: "memory");
-    if (M.v16) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
+    return tie_rows;
+}
+
+// One block's work: x-segment bx (64 cells), y-run by, z-block bz of planes
+// [k0, k1).  FAST: R and diag64 (R alone: R) given and, with vals, 16-byte
+// aligned (checked by the launcher).
+template <bool DIAG, bool CRK, int W, bool FAST, XOp OP>
+__device__ __forceinline__ void xmarch_tile(const GridGeom& g, const PhysF& q, const AsmFields<float>& f,
+                                            const AsmOut<float>& o, int JY, int bx, int by, int bz,
+                                            unsigned char* smem, int k0, int k1) {
+    using X = XMarch<DIAG, CRK, W, OP>;
+    const int lane = threadIdx.x, w = threadIdx.y;
+    const int k = k0 + bz * W + w;
+    if (k >= k1) return;  // warp-uniform
+    XState<DIAG, CRK, W, FAST, OP> M(g, q, f, o, reinterpret_cast<float*>(smem) + w * X::smem_floats_per_warp(), lane,
+                                     k, bx);
+    const int j0 = by * JY;
+    const unsigned long long tie_rows = xmarch_rows(M, j0, min(j0 + JY, g.ny));
+    if (X::JAC && M.v16) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
     if (tie_rows) {  // warp-uniform; every bulk store of the warp has completed
         __syncwarp();
         for (int b = 0; b < 64; ++b)
             if ((tie_rows >> b) & 1ull) {
-                naive_row<float, CRK, true>(g, q, f, o, M.act, M.ia, j0 + b, k);
-                naive_row<float, CRK, true>(g, q, f, o, M.act, M.ib, j0 + b, k);
+                naive_row<float, CRK, X::JAC>(g, q, f, o, M.act, M.ia, j0 + b, k);
+                naive_row<float, CRK, X::JAC>(g, q, f, o, M.act, M.ib, j0 + b, k);
             }
     }
 }
 
-template <bool DIAG, bool CRK, int W, bool FAST>
-__global__ void __launch_bounds__(32 * W, W == 4 ? 3 : 1)
+// Blocks per multiprocessor (4 warps each).  R alone fits 128 registers
+// without spills (five blocks: 3 % slower with 10 links), J w with 6 links
+// too (3 % faster than three blocks at 512 x 512 x 128); with 10 links it
+// would spill half its window (58.0 -> 30.3 G cells/s).
+constexpr int xmarch_blocks(XOp op, bool diag) { return op == XOp::Res || (op != XOp::Jac && !diag) ? 4 : 3; }
+
+template <bool DIAG, bool CRK, int W, bool FAST, XOp OP>
+__global__ void __launch_bounds__(32 * W, W == 4 ? xmarch_blocks(OP, DIAG) : 1)
     k_assemble_xmarch(GridGeom g, PhysF q, AsmFields<float> f, AsmOut<float> o, int JY, int k0, int k1) {
     extern __shared__ __align__(16) unsigned char smem[];
     int bx, by, bz;
     segment_major(bx, by, bz);
-    xmarch_tile<DIAG, CRK, W, FAST>(g, q, f, o, JY, bx, by, bz, smem, k0, k1);
+    xmarch_tile<DIAG, CRK, W, FAST, OP>(g, q, f, o, JY, bx, by, bz, smem, k0, k1);
 }
 
 }  // namespace tpfa
