@@ -20,13 +20,18 @@ from ._capi import TPFA_FP64, TPFA_MIXED, TPFAError, check
 PRECISIONS = {"fp64": TPFA_FP64, "mixed": TPFA_MIXED}
 
 
+# The library's functions declare their argument types, so addresses and
+# stream handles are passed as plain integers.  The current stream is asked
+# for as a raw handle: torch.cuda.current_stream() builds a Stream object,
+# 3 us of the 10 to 15 us that a call on a small grid costs the host.
 def _ptr(t: torch.Tensor | None):
-    return ctypes.c_void_p(t.data_ptr()) if t is not None else None
+    return t.data_ptr() if t is not None else None
 
 
 def _stream(stream=None):
-    s = stream if stream is not None else torch.cuda.current_stream()
-    return ctypes.c_void_p(s.cuda_stream)
+    if stream is not None:
+        return stream.cuda_stream
+    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
 
 
 def _unused_mesh_params() -> dict:
@@ -41,6 +46,8 @@ def params_struct(phys: dict) -> _capi.TPFAParams:
 
 def _dev_f64(x, device):
     if isinstance(x, torch.Tensor):
+        if x.dtype == torch.float64 and x.device == device and x.is_contiguous():
+            return x
         return x.to(device=device, dtype=torch.float64).contiguous()
     return torch.as_tensor(np.ascontiguousarray(x, dtype=np.float64), device=device)
 
@@ -77,6 +84,7 @@ class Grid:
         self.nnz = int(nnz.value)
         self._p = None
         self._pn = None
+        self._perm_set = 0  # how often the permeability was replaced
 
     def _create(self, h, prm, k, ph, z):
         check(self.lib.tpfa_create_grid(ctypes.byref(h), self.nx, self.ny, self.nz, ctypes.byref(prm),
@@ -159,6 +167,7 @@ class Grid:
         k = _dev_f64(perm, self.device)
         if k.numel() != self.n:
             raise ValueError(f"expected {self.n} values, got {k.numel()}")
+        self._perm_set += 1
         check(self.lib.tpfa_set_permeability(self.handle, _ptr(k), _stream(stream)))
         self._perm = k  # read asynchronously: keep it alive
 
@@ -168,6 +177,7 @@ class Grid:
         lk = _dev_f64(log_k, self.device)
         if lk.numel() != self.n:
             raise ValueError(f"expected {self.n} values, got {lk.numel()}")
+        self._perm_set += 1
         check(self.lib.tpfa_set_log_permeability(self.handle, _ptr(lk), _stream(stream)))
         self._perm = lk  # read asynchronously: keep it alive
 
@@ -506,13 +516,16 @@ class TPFAResidual(torch.autograd.Function):
     """R(p, ln k) of Eq. vk on a Grid whose previous-step state is bound.
 
     forward(grid, p, log_k) -> R (FP64, N).  log_k is the natural log of the
-    permeability; the grid's transmissibilities are recomputed when it
-    changes.  backward runs the library's adjoint kernel (checkpoint-free:
-    nothing is saved but p and log_k)."""
+    permeability; the grid's transmissibilities are recomputed from it in the
+    forward pass, and again in the backward pass if the grid's permeability
+    was replaced in between (by another forward, or by the caller).  backward
+    runs the library's adjoint kernel (checkpoint-free: nothing is saved but p
+    and log_k)."""
 
     @staticmethod
     def forward(ctx, grid, p, log_k):
-        _apply_log_k(grid, log_k)
+        grid.set_log_permeability(log_k.detach())
+        ctx.perm_set = grid._perm_set
         grid.set_pressure(p.detach())
         R = grid.assemble_residual()
         ctx.grid = grid
@@ -521,20 +534,15 @@ class TPFAResidual(torch.autograd.Function):
 
     @staticmethod
     def backward(ctx, gR):
-        p, log_k = ctx.saved_tensors
+        p, log_k = ctx.saved_tensors  # raises if one was modified in place
         grid = ctx.grid
-        _apply_log_k(grid, log_k)
+        if grid._perm_set != ctx.perm_set:
+            grid.set_log_permeability(log_k.detach())
         grid.set_pressure(p.detach())
-        g_p, g_lnk = grid.vjp(gR.detach().to(torch.float64).contiguous(), want_lnk=ctx.needs_input_grad[2])
+        g_p, g_lnk = grid.vjp(gR.detach(), want_lnk=ctx.needs_input_grad[2])
         gp = g_p.to(p.dtype) if ctx.needs_input_grad[1] else None
         gk = g_lnk.to(log_k.dtype) if ctx.needs_input_grad[2] else None
         return None, gp, gk
-
-
-def _apply_log_k(grid, log_k):
-    # Always re-applied: a tensor's address and version do not identify its
-    # contents (the caching allocator reuses addresses).
-    grid.set_log_permeability(log_k.detach())
 
 
 def residual(grid, p, log_k):
