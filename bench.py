@@ -42,9 +42,9 @@ CONN = 10
 WORKLOAD = "tpfa_residual_jacobian_512x512x256_10pt_mixed"
 KERNEL_SOURCES = ["tpfa_assemble.cu", "tpfa_xmarch.cuh", "tpfa_ymarch.cuh", "tpfa_row.cuh", "tpfa_common.cuh",
                   "tpfa_grid.h"]
-JVP_SOURCES = ["tpfa_jvp.cu", "tpfa_ymarch.cuh", "tpfa_row.cuh", "tpfa_common.cuh", "tpfa_grid.h"]
+JVP_SOURCES = ["tpfa_jvp.cu", "tpfa_xmarch.cuh", "tpfa_ymarch.cuh", "tpfa_row.cuh", "tpfa_common.cuh", "tpfa_grid.h"]
 MESH_SOURCES = ["tpfa_mesh.cu", "tpfa_mesh.h", "tpfa_row.cuh", "tpfa_common.cuh", "tpfa_grid.h"]
-FP64_SOURCES = ["tpfa_assemble.cu", "tpfa_ymarch.cuh", "tpfa_row.cuh", "tpfa_common.cuh", "tpfa_grid.h"]
+FP64_SOURCES = ["tpfa_fp64.cu", "tpfa_tile.h", "tpfa_row.cuh", "tpfa_common.cuh", "tpfa_grid.h"]
 VJP_SOURCES = ["tpfa_vjp.cu", "tpfa_ymarch.cuh", "tpfa_row.cuh", "tpfa_common.cuh", "tpfa_grid.h"]
 # kernel names of the assembly variants, as the launch list shows them
 VARIANT_KERNELS = {"tiled2": "k_assemble_xmarch<DIAG,!CRK,W>", "tiled": "k_assemble_ymarch<float,DIAG,!CR,JAC,W>",
@@ -656,7 +656,7 @@ def measure_jvp(g, prob, dev, stream, peak, reps=10):
                          "traffic_source": "ncu DRAM bytes per cell at 256x256x128 (profiles/jvp_mixed_256x256x128.md) x cells",
                          "warp_instructions_per_cell": profile_number(prof, "warp_instructions_per_cell"),
                          "kernel_source_sha256_16": khash},
-            "kernel": "k_jvp_ymarch<DIAG,!CR,W=%d>" % tiling[1],
+            "kernel": "k_jvp_xmarch<DIAG,!CR>",
             "tiling": {"rows_per_march": tiling[0], "warps_per_block": tiling[1]},
             "outputs": "J w (FP64)"}
 
@@ -744,7 +744,7 @@ def measure_newton(dev, stream, reps=3):
                                        "achieved": per_iter_bytes / (ms_iter * 1e-3) / 1e9, "peak": peak,
                                        "unit": "GB/s", "frac": per_iter_bytes / (ms_iter * 1e-3) / 1e9 / peak},
             "preconditioner": "z-line (tridiagonal along z, per column)",
-            "note": "includes one assembly and the update; 10 kernels per BiCGStab iteration, 8 iterations per CUDA-graph launch and host poll"}
+            "note": "includes one assembly and the update; 5 kernels per BiCGStab iteration, 8 iterations per CUDA-graph launch and host poll"}
 
 
 def measure_adjoint(dev, stream, reps=20):

@@ -360,9 +360,9 @@ int launch(tpfa_grid* h, AsmKernel kern, double* R, void* vals, double* diag64, 
 // The adjoint's kernel for TPFA_KERNEL_AUTO: the one-cell march.  The
 // two-cell adjoint march issues 18 % fewer instructions per cell but needs
 // 168 registers (12 warps per multiprocessor, a few spilled values) against
-// 119 (16 warps): measured (G cells/s per call, one-cell vs two-cell) 21.4
-// vs 17.2 at 128^3, 28.4 vs 26.2 at 256 x 256 x 128, 32.7 vs 32.5 at
-// 512 x 512 x 256.
+// 119 (16 warps): measured (us per call, one-cell vs two-cell, 10 links) 90
+// vs 98 at 128^3, 275 vs 308 at 256 x 256 x 128, 963 vs 992 at
+// 512 x 512 x 128 (6 links: 71 vs 73, 220 vs 210, 764 vs 726).
 AsmKernel vjp_auto_kernel(tpfa_grid*) { return AsmKernel::YMarch; }
 
 int check_handle(tpfa_handle h) {

@@ -13,9 +13,9 @@
 // link the term dF/dp_K w_K + dF/dp_L w_L is one FP32 fma of the link's FP32
 // derivatives; the terms are Kahan-summed in FP32 in slot order, then
 // dA/dp w_K, and the sum is combined in FP64.  The error is a few float ulps
-// of sum_L |J_KL| |w_L|.  Two kernels give identical bits: the y-march (the
-// production kernel, the assembly's march with w in its prefetch ring) and a
-// one-thread-per-cell gather with checked loads.
+// of sum_L |J_KL| |w_L|.  Three kernels give identical bits: the assembly's
+// marches with w in their prefetch rings (two cells per lane on wide grids, one
+// on others) and a one-thread-per-cell gather with checked loads.
 //
 // The FP64 path's J w is in tpfa_fp64.cu.
 #include <cuda_runtime.h>

@@ -6,7 +6,8 @@
 // a = i0 + 2l and b = a + 1 of each row, so every per-cell quantity of a
 // lane is an FP32 pair and every link it evaluates is one half of an FP32x2
 // instruction whose other half is the same link of its other cell.  Per row
-// j each lane assembles rows (a, j, k) and (b, j, k) of Algorithm 1 / Eq. vk:
+// j each lane assembles rows (a, j, k) and (b, j, k) of Algorithm 1 / Eq. vk
+// (R and the Jacobian, R alone, or J w with or without R: XOp below):
 //
 //   * links evaluated from the lane's side, as pairs (cell a, cell b):
 //       +x (a -> b, b -> lane+1's a), +y, +x+y, -x+y, +z, -z
