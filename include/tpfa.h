@@ -505,8 +505,9 @@ int tpfa_ensemble_set_outputs(tpfa_ensemble e, int m, double* R_dev, void* vals_
  * output changed since the last call, then launches the graph on `stream`. */
 int tpfa_assemble_batch(tpfa_ensemble e, void* stream);
 
-/* The ensemble's tiling (see tpfa_set_tiling), its number of tiles and of
- * persistent blocks (the latter known after the first batch call). */
+/* The ensemble's tiling (see tpfa_set_tiling; rows_per_march: the most rows, as
+ * the last models' marches are shorter), its number of tiles and of persistent
+ * blocks (the latter known after the first batch call). */
 int tpfa_ensemble_tiling(tpfa_ensemble e, int* rows_per_march, int* warps_per_block, long long* tiles,
                          int* blocks);
 

@@ -20,8 +20,7 @@ namespace {
 
 template <bool DIAG, bool CRK, int W>
 __global__ void __launch_bounds__(32 * W, 16 / W)
-    k_assemble_batch(const BatchModel* __restrict__ models, int M, long long total, int JY,
-                     unsigned long long* ticket) {
+    k_assemble_batch(const BatchModel* __restrict__ models, int M, long long total, unsigned long long* ticket) {
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ BatchModel sm;
     __shared__ long long s_tile;
@@ -48,7 +47,7 @@ __global__ void __launch_bounds__(32 * W, 16 / W)
         }
         __syncthreads();
         if (s_tile >= total) break;
-        ymarch_tile<DIAG, CRK, true, W, true>(sm.g, sm.q, sm.f, sm.o, JY, s_bx, s_by, s_bz, smem);
+        ymarch_tile<DIAG, CRK, true, W, true>(sm.g, sm.q, sm.f, sm.o, sm.rows, s_bx, s_by, s_bz, smem);
         __syncthreads();  // every warp is done with this tile's descriptor and buffers
     }
 }

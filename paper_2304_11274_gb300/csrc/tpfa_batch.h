@@ -10,13 +10,13 @@ namespace tpfa {
 
 // One model of an ensemble as the persistent kernel sees it: its grid, its
 // physics, its fields and outputs, and its tiles (32-cell x-segments, runs of
-// JY rows, blocks of W planes), numbered from `first`.
+// `rows` rows, blocks of W planes), numbered from `first`.
 struct BatchModel {
     GridGeom g;
     PhysF q;
     AsmFields<float> f;
     AsmOut<float> o;
-    int tx, ty, tz;
+    int tx, ty, tz, rows;
     int crk;  // c_r != 0
     long long first;
 };
