@@ -475,6 +475,18 @@ struct XState {
         return h == 0 ? LinkOut<float>{l.F.x, l.Da.x, l.Db.x} : LinkOut<float>{l.F.y, l.Da.y, l.Db.y};
     }
 
+    // Whether either cell's link is an exact tie: a zero flux with a derivative.
+    // A link of an impermeable cell (T = 0) has neither, from either end, and is
+    // reused as it is.  |F| 2^100 < |dF/dp_b| asks both at once: true of every
+    // tie, never of T = 0, and of a non-zero flux only where |dPhi| < 2^-100 or so
+    // (that row is then merely computed again).  va, vb: the cell's link exists.
+    // Measured at 512 x 512 x 128, 10 links, 5 % of the cells impermeable, against
+    // F == 0 alone: J w 4726 -> 604 us (597 without such cells), R + J 3139 -> 746 us (739).
+    static __device__ __forceinline__ bool ties(const Link2& l, bool va = true, bool vb = true) {
+        const float2 F = __fmul2_rn(l.F, f2(0x1p100f));
+        return (va && fabsf(F.x) < fabsf(l.Db.x)) || (vb && fabsf(F.y) < fabsf(l.Db.y));
+    }
+
     // Prologue of a march starting at row j0: rows j0-1 and j0, the links
     // of row j0-1 into row j0; row j0+1 requested.
     __device__ __forceinline__ void start(int j0) {
@@ -491,10 +503,7 @@ struct XState {
             Umxy = link_pp(q, pair_at(0, X::P_TMP), Pc, shift_right(Cm, Cc));
         }
         // zero flux on a link reused next (only links that exist; none from row -1)
-        tie_up = j0 > 0 && act &&
-                 (Uy.F.x == 0.f || Uy.F.y == 0.f ||
-                  (DIAG && (Uxy.F.x == 0.f || (okb && Uxy.F.y == 0.f) || (oka && Umxy.F.x == 0.f) ||
-                            Umxy.F.y == 0.f)));
+        tie_up = j0 > 0 && act && (ties(Uy) || (DIAG && (ties(Uxy, true, okb) || ties(Umxy, oka))));
         if constexpr (JV) {
             wP = w_row(0);
             wC = w_row(1);
@@ -623,12 +632,10 @@ struct XState {
         // the +x links (a's -x comes from lane-1's b, b's -x from a)
         // (on an interior segment every lane's +x and diagonal links exist)
         const bool kb2 = PATH == 2 ? true : okb, ka2 = PATH == 2 ? true : oka;
-        const bool tie_x = on && (LX_.F.x == 0.f || (kb2 && LX_.F.y == 0.f));
+        const bool tie_x = on && ties(LX_, true, kb2);
         // (a tie's flux is zero from either end: R alone needs none of this)
         const bool tie_here = (JAC || JV) && (tie_up || tie_x);
-        if (JAC || JV) tie_up = on && (LY.F.x == 0.f || LY.F.y == 0.f ||
-                         (DIAG && (LXY.F.x == 0.f || (kb2 && LXY.F.y == 0.f) || (ka2 && LMXY.F.x == 0.f) ||
-                                   LMXY.F.y == 0.f)));
+        if (JAC || JV) tie_up = on && (ties(LY) || (DIAG && (ties(LXY, true, kb2) || ties(LMXY, ka2))));
 
         // ---- accumulation (Eq. vk) and the FP64 combinations
         R.gather();
