@@ -83,13 +83,14 @@ __device__ __forceinline__ float narrow_rz(double x) {
     return (float)x;
 }
 
-// The two conversions above without their general branch: its conversion
-// instruction is predicated, not jumped over, and takes its time on the FP64
-// pipe even when no lane needs it.  Measured without it: the two-cell assembly
-// at 512 x 512 x 256 1430 -> 1378 us, an ensemble of 20 models 1692 -> 1624 us.
-// narrow_flush: |x| < 2^128, values below 2^-126 give zero.  narrow_any: the
-// same for any x (larger values infinite, NaN kept).  widen_flush: finite x,
-// subnormals give zero.
+// The two conversions above without the conversion instruction: it is
+// predicated, not jumped over, and takes its time on the FP64 pipe even when no
+// lane needs it.  Measured without it: the two-cell assembly at 512 x 512 x 256
+// 1430 -> 1378 us, an ensemble of 20 models 1692 -> 1624 us.
+//   narrow_flush, widen_flush: |x| < 2^128; what would be or is an FP32
+//     subnormal gives zero;
+//   narrow_any: every x, with the bits of narrow_rz (NaN payloads aside); the
+//     rare values by integer operations behind a branch.
 __device__ __forceinline__ float narrow_flush(double x) {
     const uint32_t hi = (uint32_t)__double2hiint(x);
     const uint32_t lo = (uint32_t)__double2loint(x);
@@ -97,12 +98,23 @@ __device__ __forceinline__ float narrow_flush(double x) {
     const uint32_t f = ((a - 0x38000000u) << 3) | (lo >> 29);
     return __uint_as_float((hi & 0x80000000u) | (a >= 0x38100000u ? f : 0u));
 }
+// Magnitude bits of (float)x for |x| outside [2^-126, 2^128), from its words.
+__device__ __forceinline__ uint32_t narrow_rare(uint32_t a, uint32_t lo) {
+    if (a >= 0x47f00000u) return a > 0x7ff00000u || (a == 0x7ff00000u && lo) ? 0x7fc00000u : 0x7f800000u;
+    // units of 2^-149, rounded to nearest even: x = m 2^-149 / 2^s
+    const int s = 926 - (int)(a >> 20);
+    if (s > 53) return 0u;
+    const uint64_t m = ((uint64_t)((a & 0x000fffffu) | 0x00100000u) << 32) | lo;
+    const uint64_t rest = m & ((1ull << s) - 1u), half = 1ull << (s - 1);
+    const uint32_t n = (uint32_t)(m >> s);
+    return n + (rest > half || (rest == half && (n & 1u)));
+}
 __device__ __forceinline__ float narrow_any(double x) {
     const uint32_t hi = (uint32_t)__double2hiint(x);
     const uint32_t lo = (uint32_t)__double2loint(x);
     const uint32_t a = hi & 0x7fffffffu;
-    uint32_t f = a >= 0x38100000u ? ((a - 0x38000000u) << 3) | (lo >> 29) : 0u;
-    if (a >= 0x47f00000u) f = 0x7f800000u | (a >= 0x7ff00000u ? (a & 0x000fffffu) << 3 : 0u);
+    uint32_t f = a ? ((a - 0x38000000u) << 3) | (lo >> 29) : 0u;
+    if (a - 0x38100000u >= 0x0fe00000u && a) f = narrow_rare(a, lo);
     return __uint_as_float((hi & 0x80000000u) | f);
 }
 __device__ __forceinline__ double widen_flush(float x) {
@@ -112,6 +124,10 @@ __device__ __forceinline__ double widen_flush(float x) {
     const uint32_t hi = (n ? (a >> 3) + 0x38000000u : 0u) | (u & 0x80000000u);
     return __hiloint2double((int)hi, n ? (int)(u << 29) : 0);
 }
+__device__ __forceinline__ bool finite_f32(float x) { return fabsf(x) < __int_as_float(0x7f800000); }
+// Below kSubnormal: x is subnormal (twice its bits: no sign; zero wraps round).
+constexpr uint32_t kSubnormal = 2u * 0x007fffffu;
+__device__ __forceinline__ uint32_t sub_word(float x) { return 2u * __float_as_uint(x) - 2u; }
 
 // A double as an unevaluated FP32 pair v = hi + lo (hi the truncation of v,
 // lo the exact remainder narrowed; |lo| < ulp(hi)), so differences of nearby
@@ -439,6 +455,9 @@ __device__ __forceinline__ float expm1_f32(float x) {
 struct AccF {
     double A;  // FP64 accumulation term
     float dA;  // its pressure derivative (a term of the FP32 diagonal sum)
+    // PLAIN (below): the least sub_word and the sum of A's FP32 factors
+    uint32_t low;
+    float all;
 };
 
 // expm1 of the accumulation term with its value as a double: in PLAIN rows
@@ -458,11 +477,13 @@ __device__ __forceinline__ AccF accumulation(const PhysF& q, float p, float pn, 
     double e64;
     const float e = expm1_wide<PLAIN>(__fmul_rn(q.c_f, dpn), e64);
     r.A = __dmul_rn(mn, e64);
+    if (PLAIN) r.low = sub_word(e), r.all = e;
     if (CR) {
         // (V/dt) phi0 c_r (p - p^n) rho(p), and dA = (V/dt)(phi0 c_r rho + phi(p) c_f rho)
         const float vphi = __fmul_rn(q.V_dt, phi0);
         const float g = __fmul_rn(__fmul_rn(vphi, q.c_r), __fmul_rn(dpn, rho));
         r.A = __dadd_rn(r.A, PLAIN ? widen_flush(g) : widen(g));
+        if (PLAIN) r.low = min(r.low, sub_word(g)), r.all = __fadd_rn(e, g);
         const float phi_rel = __fmaf_rn(q.c_r, __fsub_rn(p, q.p_ref), 1.f);
         r.dA = __fmul_rn(__fmul_rn(vphi, rho), __fmaf_rn(phi_rel, q.c_f, q.c_r));
     } else {
@@ -472,24 +493,22 @@ __device__ __forceinline__ AccF accumulation(const PhysF& q, float p, float pn, 
     return r;
 }
 
-// The marches form a row's FP64 results from its compensated FP32 sums with
-// the cheap widening, which is exact for normal values and zero, and record
-// the rows where that may not do: a sum so small that a flushed subnormal (its
-// compensation, or a factor of A) could reach the result's last bit; a result
-// (or m^n) so large that an infinite or NaN sum, which the cheap widening
-// turns into about 2^128, could stand in it.  Those rows are computed again
-// after the march by the naive kernel's row code, as tie rows are, which also
-// reports non-finite values.  Zero sums (cells without links) are plain.
-__device__ __forceinline__ bool odd_sum(float s) { return fabsf(s) < 0x1p-60f && s != 0.f; }
-constexpr uint32_t kOddHigh = 0x43b00000u;  // high word of 2^60
-// The smaller magnitude, NaN if either is NaN.
-__device__ __forceinline__ float min_abs(float a, float b) {
-    float r;
-    asm("min.NaN.f32 %0, %1, %2;" : "=f"(r) : "f"(fabsf(a)), "f"(fabsf(b)));
-    return r;
+// The marches (PLAIN) form a row's FP64 results, R = (A + s) - c and the
+// diagonal s - c, from its compensated FP32 sums (s, c), A = mn expm1(x) and mn
+// with the cheap conversions, which are exact for normal values and zero.  Rows
+// with another value among them, odd rows, are computed again after the march
+// by the naive kernel's row code, as tie rows are, which also reports
+// non-finite values.  The tests are on these values themselves, two integer
+// instructions each and no branch: sub_word of the sums and of A's factors, one
+// finiteness test of their sum, and odd_mass.  A sum that is merely small or zero
+// (cells of next to no permeability, no change of pressure) makes no row odd;
+// a compensation is subnormal where fluxes are below 1e-31 (k below 1e-43 m^2).
+// (Testing the results' size instead, with these tests behind a branch, took
+// 3 % of an ensemble's time.)
+__device__ __forceinline__ bool odd_mass(double mn) {  // outside FP32's normal range, not zero
+    const uint32_t w = 2u * (uint32_t)__double2hiint(mn);
+    return w - 2u * 0x38100000u >= 2u * 0x0fe00000u && w != 0u;
 }
-// A NaN sum's compensation is NaN too, and their cheap widenings cancel.
-__device__ __forceinline__ bool nan_sum(float s) { return s != s; }
 
 struct AccD {
     double A, dA;

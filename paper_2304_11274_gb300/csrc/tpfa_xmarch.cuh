@@ -96,12 +96,14 @@ __device__ __forceinline__ void kahan2_masked(Kahan2& k, float2 x, bool va, bool
 // FP64 terms A of both cells and the pair of dA/dp.
 template <bool CRK>
 __device__ __forceinline__ float2 accumulation2(const PhysF& q, float2 p, float2 pn, double2 mn, float2 rho,
-                                                float2 phi0, double& Aa, double& Ab) {
+                                                float2 phi0, double& Aa, double& Ab, uint32_t& low, float2& all) {
     if constexpr (CRK) {
         const AccF a = accumulation<true, true>(q, p.x, pn.x, mn.x, rho.x, phi0.x);
         const AccF b = accumulation<true, true>(q, p.y, pn.y, mn.y, rho.y, phi0.y);
         Aa = a.A;
         Ab = b.A;
+        low = min(a.low, b.low);
+        all = f2(a.all, b.all);
         return f2(a.dA, b.dA);
     } else {
         const float2 m1 = f2(-1.f);
@@ -120,6 +122,8 @@ __device__ __forceinline__ float2 accumulation2(const PhysF& q, float2 p, float2
         }
         Aa = __dmul_rn(mn.x, ea);
         Ab = __dmul_rn(mn.y, eb);
+        low = min(sub_word(e.x), sub_word(e.y));
+        all = e;
         return __fmul2_rn(__fmul2_rn(f2(q.c_f), f2(narrow_flush(mn.x), narrow_flush(mn.y))), __fadd2_rn(f2(1.f), e));
     }
 }
@@ -315,7 +319,6 @@ struct XState {
     const double* wv = nullptr;
     double* Jw = nullptr;
     XW wP, wC;
-    bool w_odd = false;  // a w of rows up to j + 1 lies outside the FP32 normal range
 
     __device__ __forceinline__ XState(const GridGeom& g_, const PhysF& q_, const AsmFields<float>& f_,
                                       const AsmOut<float>& o_, float* ring_, int lane_, int k_, int bx)
@@ -397,22 +400,31 @@ struct XState {
         }
         asm volatile("cp.async.commit_group;" ::: "memory");
     }
-    // w as FP32 (truncated), and whether the cheap narrowing is exact for it
-    __device__ __forceinline__ float narrow_w(double x) {
-        const uint32_t a = abs_hi(x);
-        w_odd = w_odd || (a - 0x38100000u >= 0x0fe00000u && a != 0u);
-        return narrow_flush(x);
+    // w as FP32 (truncated) of ring slots sn (the lane's cells of the row and
+    // the halo cell) and sd (planes k - 1 and k + 1): the cheap narrowing, or, if
+    // any of the warp's values lies outside FP32's normal range, the exact one.
+    // (A test of its own behind each value cost 14 % of J w at 512 x 512 x 256.)
+    __device__ __forceinline__ double2 w_ring(int sl, int plane) const {
+        return *reinterpret_cast<const double2*>(ring + sl * X::SLOT + X::OFF_W + 128 * plane + 4 * lane);
     }
-    __device__ __forceinline__ float2 w_pair(int sl, int plane) {
-        const double2 d = *reinterpret_cast<const double2*>(ring + sl * X::SLOT + X::OFF_W + 128 * plane + 4 * lane);
-        return f2(narrow_w(d.x), narrow_w(d.y));
-    }
-    __device__ __forceinline__ XW w_row(int sl) {
+    __device__ __forceinline__ XW w_rows(int sn, int sd, float2& zmw, float2& zpw) const {
+        const double2 d = w_ring(sn, 0), dm = w_ring(sd, 1), dp = w_ring(sd, 2);
+        const double h64 = hact ? reinterpret_cast<const double*>(ring + sn * X::SLOT + X::OFF_W)[192 + (hl ? 1 : 0)] : 0.0;
+        // twice the high words (no sign): outside the normal range, or zero
+        const auto word = [](double x) { return 2u * (uint32_t)__double2hiint(x) - 2u * 0x38100000u; };
+        const uint32_t rare = max(max(max(word(d.x), word(d.y)), max(word(dm.x), word(dm.y))),
+                                  max(max(word(dp.x), word(dp.y)), hact ? word(h64) : 0u));
         XW r;
-        r.c = w_pair(sl, 0);
-        const double* Wh = reinterpret_cast<const double*>(ring + sl * X::SLOT + X::OFF_W) + 192;
-        float h = 0.f;
-        if (hact) h = narrow_w(Wh[hl ? 1 : 0]);
+        r.c = f2(narrow_flush(d.x), narrow_flush(d.y));
+        zmw = f2(narrow_flush(dm.x), narrow_flush(dm.y));
+        zpw = f2(narrow_flush(dp.x), narrow_flush(dp.y));
+        float h = narrow_flush(h64);
+        if (__any_sync(0xffffffffu, act && rare >= 2u * 0x0fe00000u)) {
+            r.c = f2(narrow_any(d.x), narrow_any(d.y));
+            zmw = f2(narrow_any(dm.x), narrow_any(dm.y));
+            zpw = f2(narrow_any(dp.x), narrow_any(dp.y));
+            h = narrow_any(h64);
+        }
         r.m = __shfl_up_sync(0xffffffffu, r.c.y, 1);
         r.p = __shfl_down_sync(0xffffffffu, r.c.x, 1);
         if (lane == 0) r.m = h;
@@ -505,8 +517,9 @@ struct XState {
         // zero flux on a link reused next (only links that exist; none from row -1)
         tie_up = j0 > 0 && act && (ties(Uy) || (DIAG && (ties(Uxy, true, okb) || ties(Umxy, oka))));
         if constexpr (JV) {
-            wP = w_row(0);
-            wC = w_row(1);
+            float2 zm_, zp_;
+            wP = w_rows(0, 0, zm_, zp_);
+            wC = w_rows(1, 1, zm_, zp_);
         }
         issue(j0 + 1, 0);
     }
@@ -532,9 +545,7 @@ struct XState {
         XW wN{};
         float2 wzm = f2(0.f), wzp = f2(0.f);
         if constexpr (JV) {
-            wN = w_row(sN);
-            wzm = w_pair(sD, 1);
-            wzp = w_pair(sD, 2);
+            wN = w_rows(sN, sD, wzm, wzp);
         }
         issue(j + 2, sD);
 
@@ -640,7 +651,9 @@ struct XState {
         // ---- accumulation (Eq. vk) and the FP64 combinations
         R.gather();
         double Aa, Ab;
-        const float2 dA = accumulation2<CRK>(q, Cc.p, pn, mn, Cc.rho, phi, Aa, Ab);
+        uint32_t low;
+        float2 all;
+        const float2 dA = accumulation2<CRK>(q, Cc.p, pn, mn, Cc.rho, phi, Aa, Ab, low, all);
         const double Ra = __dadd_rn(__dadd_rn(Aa, widen_flush(R.kr.s.x)), -widen_flush(R.kr.c.x));
         const double Rb = __dadd_rn(__dadd_rn(Ab, widen_flush(R.kr.s.y)), -widen_flush(R.kr.c.y));
         Kahan2 dd = R.kd;  // dA (J w: times w) joins the second sums last
@@ -657,17 +670,16 @@ struct XState {
             Da64 = __dadd_rn(widen(dd.s.x), -widen(dd.c.x));
             Db64 = __dadd_rn(widen(dd.s.y), -widen(dd.c.y));
         }
-        // rows that need exact conversions (odd_sum; min_abs is NaN if a sum is)
-        uint32_t hi = max(abs_hi(mn.x), abs_hi(mn.y));
-        float rmin = 1.f, dmin = 1.f;
-        if (RES) hi = max(hi, max(abs_hi(Ra), abs_hi(Rb))), rmin = min_abs(R.kr.s.x, R.kr.s.y);
-        if (JAC || JV) hi = max(hi, max(abs_hi(Da64), abs_hi(Db64)));
-        if (JAC) dmin = min_abs(dd.s.x, dd.s.y);
-        bool odd = hi >= kOddHigh || (JV && w_odd);
-        if (!(rmin >= 0x1p-60f && dmin >= 0x1p-60f)) {  // small, zero or NaN: which
-            if (RES) odd = odd || odd_sum(R.kr.s.x) || odd_sum(R.kr.s.y) || nan_sum(rmin);
-            if (JAC) odd = odd || odd_sum(dd.s.x) || odd_sum(dd.s.y) || nan_sum(dmin);
-        }
+        // odd rows (odd_mass); J w: a non-finite result
+        bool odd = odd_mass(mn.x) || odd_mass(mn.y);
+        const auto pair_words = [&](const Kahan2& k) {
+            low = min(low, min(min(sub_word(k.s.x), sub_word(k.s.y)), min(sub_word(k.c.x), sub_word(k.c.y))));
+            all = __fadd2_rn(all, k.s);
+        };
+        if (RES) pair_words(R.kr);
+        if (JAC) pair_words(dd);
+        if (RES) odd = odd || low < kSubnormal || !finite_f32(__fadd_rn(all.x, all.y));
+        if (JV) odd = odd || max(abs_hi(Da64), abs_hi(Db64)) >= 0x7ff00000u;
         const bool tie = __any_sync(0xffffffffu, tie_here || (on && odd));
         if (on) {
             const int c = kb + nx * j + ia;

@@ -674,11 +674,11 @@ struct YMarch {
         }
         out.R = __dadd_rn(__dadd_rn(acc.A, widen_flush(ks.s.x)), -widen_flush(ks.c.x));
         out.diag64 = JAC ? __dadd_rn(widen_flush(ds.s), -widen_flush(ds.c)) : 0.0;
-        uint32_t hi = max(abs_hi(out.R), abs_hi(D.mn));
-        if (JAC) hi = max(hi, abs_hi(out.diag64));
-        // `bad` here: the row needs exact conversions
-        out.bad = act && (hi >= kOddHigh || odd_sum(ks.s.x) || nan_sum(ks.s.x) ||
-                          (JAC && (odd_sum(ds.s) || nan_sum(ds.s))));
+        // `bad` here: the row is odd (odd_mass)
+        uint32_t low = min(acc.low, min(sub_word(ks.s.x), sub_word(ks.c.x)));
+        float all = __fadd_rn(acc.all, ks.s.x);
+        if (JAC) low = min(low, min(sub_word(ds.s), sub_word(ds.c))), all = __fadd_rn(all, ds.s);
+        out.bad = act && (low < kSubnormal || !finite_f32(all) || odd_mass(D.mn));
         return out;
     }
 
