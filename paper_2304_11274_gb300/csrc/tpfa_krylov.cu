@@ -52,17 +52,20 @@ constexpr int kVecBlocks = 152 * 5;   // blocks of the vector kernels, at most
 constexpr int kMaxBlocks = 152 * 4;   // blocks of the products: one wave
 
 // v as an FP32 pair hi + lo without the FP64 pipe: hi the truncation of v, lo the
-// 29 fraction bits it leaves, rounded to 24.  Beyond the FP32 range hi is
-// infinite (the solve then breaks down, as it must), below it the pair is zero.
+// 29 fraction bits it leaves, rounded to 24 (below 2^-126 to a multiple of
+// 2^-149).  A v below 2^-126 is rounded to a subnormal hi alone, beyond the FP32
+// range hi is infinite (the solve then breaks down, as it must).
 __device__ __forceinline__ float2 split_pair(double v) {
     const uint32_t h = (uint32_t)__double2hiint(v), l = (uint32_t)__double2loint(v);
     const uint32_t a = h & 0x7fffffffu, sign = h & 0x80000000u;
-    uint32_t hi = a >= 0x38100000u ? ((a - 0x38000000u) << 3) | (l >> 29) : 0u;
-    // lo = (low bits / 2^29) ulp(hi)
-    const uint32_t e = hi & 0x7f800000u;
-    const float ulp = __uint_as_float((e > (23u << 23) ? e - (23u << 23) : 0u) | sign);
-    const float lo = __fmul_rn(__fmul_rn(__uint2float_rn(l & 0x1fffffffu), 0x1p-29f), ulp);
-    if (a >= 0x47f00000u) hi = 0x7f800000u;
+    uint32_t hi = ((a - 0x38000000u) << 3) | (l >> 29);
+    // lo = low bits 2^-52 times the power of two of hi
+    float lo = __fmul_rn(__fmul_rn(__uint2float_rn(l & 0x1fffffffu), 0x1p-52f),
+                         __uint_as_float((hi & 0x7f800000u) | sign));
+    if (a - 0x38100000u >= 0x0fe00000u) {
+        hi = a ? narrow_rare(a, l) : 0u;
+        lo = 0.f;
+    }
     return make_float2(__uint_as_float(hi | sign), lo);
 }
 
@@ -300,11 +303,13 @@ __global__ void __launch_bounds__(kThreads, sizeof(Real) == 4 ? 4 : 2)
             term(slot_array<DIAG>(10), pp);
             double yc;
             if constexpr (MIXED) {
-                // a non-finite sum would not survive the cheap widening
-                const bool plain = (__float_as_uint(ah) & 0x7fffffffu) < 0x7f800000u;
-                yc = __fma_rn(w.d, w.x,
-                              plain ? __dadd_rn(widen_flush(ah), widen_flush(al))
-                                    : __hiloint2double(0x7ff80000, 0));
+                // a subnormal or non-finite part would not survive the cheap widening
+                double off;
+                if (min(sub_word(ah), sub_word(al)) >= kSubnormal && finite_f32(ah))
+                    off = __dadd_rn(widen_flush(ah), widen_flush(al));
+                else
+                    off = __dadd_rn(widen(ah), widen(al));
+                yc = __fma_rn(w.d, w.x, off);
             } else {
                 yc = __fma_rn(w.d, pc, acc);
             }
