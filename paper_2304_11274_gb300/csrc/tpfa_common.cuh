@@ -129,6 +129,12 @@ __device__ __forceinline__ bool finite_f32(float x) { return fabsf(x) < __int_as
 constexpr uint32_t kSubnormal = 2u * 0x007fffffu;
 __device__ __forceinline__ uint32_t sub_word(float x) { return 2u * __float_as_uint(x) - 2u; }
 
+__device__ __forceinline__ float rcp_approx(float x) {  // 1/x within 2^-23
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+
 // A double as an unevaluated FP32 pair v = hi + lo (hi the truncation of v,
 // lo the exact remainder narrowed; |lo| < ulp(hi)), so differences of nearby
 // values can be formed in FP32: (hi_a - hi_b) + (lo_a - lo_b) is accurate to

@@ -31,10 +31,10 @@
 // adjoint): R + J of 256^3, 10 links 7.79 -> 3.13 ms (95 FP64 operations per cell
 // instead of 230, at 84 % of the pipe's rate), of 32^3, 6 links 223 -> 12.3 us (one
 // plane per block instead of a serial march of 32 rows), J w of 161 x 119 x 67,
-// 6 links 615 -> 234 us, the adjoint of 97 x 83 x 50 436 -> 135 us, R alone there
-// 283 -> 71 us.  Three blocks per multiprocessor (80 registers, a few spilled
-// values) instead of two: 3.39 -> 3.13 ms for R + J, the adjoint the other way
-// round (380 against 383 us for the whole gradient call).
+// 6 links 615 -> 234 us, the adjoint call of 97 x 83 x 50, 10 links 449 -> 160 us (142
+// with k_L / (k_K + k_L) from T alone: see Perm), R alone there 283 -> 71 us.  Three
+// blocks per multiprocessor (80 registers, a few spilled values) instead of two:
+// 3.39 -> 3.13 ms for R + J; the adjoint needs the registers of two.
 //
 // The rows are those of naive_row<double> bit for bit (same link, same sums in
 // slot order).
@@ -69,16 +69,71 @@ struct Args64 {
     LinkGeoD lg;          // adjoint
 };
 
+// The adjoint's k_L / (k_K + k_L) of a link without a division: T (d/A) / (2 k_K)
+// is that ratio but for T's four roundings, and for the ones of (d/A) / (2 k_K);
+// one correction by its remainder takes them out again,
+//   q0 = T (d/A) / (2 k_K),  q = q0 + q0 (k_L - (k_K + k_L) q0) / k_L,
+// the last quotient in FP32: it is below 2^-38, or the division is taken.  Four
+// FP64 operations per link.  Against 80-bit values, 10 links, log-normal k, the
+// sums' error in the 2-norm is 1.77e-16, with the rounded quotient 1.95e-16,
+// with q0 alone 2.35e-16.
+struct Perm {
+    double k = 0.0, cx = 0.0, cy = 0.0, cz = 0.0, cd = 0.0;  // k_K, (d/A) / (2 k_K)
+    // x 2^60 as FP32 (m^2 are small numbers); NaN from x = 2^65 on
+    static __device__ __forceinline__ float up60(double x) {
+        const float r = narrow_flush(__hiloint2double(__double2hiint(x) + (60 << 20), __double2loint(x)));
+        return abs_hi(x) < 0x44000000u ? r : __int_as_float(0x7fffffff);
+    }
+    __device__ __forceinline__ void set(const LinkGeoD& lg, double kK) {
+        k = kK;
+        // 1 / (2 k) to about 2^-44: any error is corrected per link
+        const double y = widen_flush(__fmul_rn(rcp_approx(up60(kK)), 0.5f));
+        const double y60 = __hiloint2double(y != 0.0 ? __double2hiint(y) + (60 << 20) : 0, __double2loint(y));
+        const double i2k = __fma_rn(y60, __fma_rn(-2.0 * k, y60, 1.0), y60);
+        cx = __dmul_rn(lg.cx, i2k), cy = __dmul_rn(lg.cy, i2k), cz = __dmul_rn(lg.cz, i2k), cd = __dmul_rn(lg.cd, i2k);
+    }
+    // ok: false for k = 0 (a link without flux, T = 0) and outside up60's range
+    template <int S>
+    __device__ __forceinline__ double ratio(double T, double kL, bool& ok) const {
+        const double q0 = __dmul_rn(T, (S == 0 || S == 10) ? cz : (S == 2 || S == 8) ? cy : (S == 4 || S == 6) ? cx : cd);
+        const double rem = __fma_rn(-kL, q0, __fma_rn(-k, q0, kL));
+        const float kf = up60(kL), d = __fmul_rn(up60(rem), rcp_approx(kf));
+        ok = fabsf(d) <= 0x1p-38f && kf >= 0x1p-60f;
+        return ok ? __fma_rn(q0, widen_flush(d), q0) : 0.0;
+    }
+};
+
+// The sum over cell (i, j, k)'s links with divisions, from global memory: for the
+// rows with a permeability outside ratio()'s range.
+__device__ __noinline__ double lnk_by_division(const Args64& a, int i, int j, int k) {
+    const int nx = a.g.nx, nxy = nx * a.g.ny, c = i + nx * j + nxy * k;
+    const unsigned mask = slot_mask(a.g, i, j, k);
+    const CellVal<double> me = make_cell(a.q, a.f.p[c], a.f.z[c]);
+    double sum = 0.0;
+#pragma unroll 1
+    for (int s = 0; s < NSLOT; ++s) {
+        if (s == SLOT_SELF || !((mask >> s) & 1u)) continue;
+        const int x = s == 0 || s == 10 ? 0 : (s - 1) % 3 - 1, y = s == 0 || s == 10 ? 0 : (s - 1) / 3 - 1;
+        const int d = s == 0 ? c - nxy : s == 10 ? c + nxy : c + x + nx * y;
+        const double* T = s == 0 || s == 10 ? a.f.Tz : x == 0 ? a.f.Ty : y == 0 ? a.f.Tx : x == y ? a.f.Tpp : a.f.Tmp;
+        const double F = link(a.q, T[s < SLOT_SELF ? d : c], me, make_cell(a.q, a.f.p[d], a.f.z[d])).F;
+        const double kk = __dadd_rn(a.kperm[c], a.kperm[d]);
+        sum = __fma_rn(__dmul_rn(F, __dsub_rn(a.dir[c], a.dir[d])), kk > 0.0 ? a.kperm[d] / kk : 0.0, sum);
+    }
+    return sum;
+}
+
 // One cell's sums over its links.
 template <Op64 OP>
 struct Sums {
     RowAccD row;
-    double acc = 0.0;                                // J w: sum dF/dp_L (w_L - w_K); adjoint: g_p
-    double gx = 0.0, gy = 0.0, gz = 0.0, gd = 0.0;  // adjoint: sum F (v_K - v_L) T per link direction
+    double acc = 0.0;  // J w: sum dF/dp_L (w_L - w_K); adjoint: g_p
+    double lnk = 0.0;  // adjoint: sum F (v_K - v_L) k_L / (k_K + k_L)
+    bool divide = false;  // ... a ratio of which has to be divided
 
-    // dv: w_L - w_K or v_K - v_L; vL: v_L; lt: the link from L's side at a tie
+    // dv: w_L - w_K or v_K - v_L; adjoint: T and k_L of the link (0 if g_lnk is not wanted)
     template <int S, bool FLAT>
-    __device__ __forceinline__ void add(const LinkOut<double>& l, double T, double dv) {
+    __device__ __forceinline__ void add(const LinkOut<double>& l, double T, double dv, const Perm& pm, double kL) {
         if constexpr (OP == Op64::Jacobian) row.add<true, FLAT>(l);
         if constexpr (OP == Op64::Residual) row.add<false, FLAT>(l);
         if constexpr (OP == Op64::Jvp) {
@@ -87,9 +142,9 @@ struct Sums {
         }
         if constexpr (OP == Op64::Vjp) {
             acc = __fma_rn(l.Da, dv, acc);
-            const double h = __dmul_rn(l.F, dv);
-            double& s = (S == 0 || S == 10) ? gz : (S == 2 || S == 8) ? gy : (S == 4 || S == 6) ? gx : gd;
-            s = __fma_rn(h, T, s);
+            bool ok;
+            lnk = __fma_rn(__dmul_rn(l.F, dv), pm.ratio<S>(T, kL, ok), lnk);
+            divide = divide || !(ok || zero_flux(l));
         }
     }
     // adjoint: v_L (dF_KL/dp_K + dF_LK/dp_K) of a tie (zero otherwise)
@@ -99,10 +154,10 @@ struct Sums {
 };
 
 template <Op64 OP, bool DIAG, bool CRK>
-__global__ void __launch_bounds__(kMaxThreads, OP == Op64::Vjp ? 2 : 3) k_cells_fp64(const Args64 a) {
+__global__ void __launch_bounds__(kMaxThreads, OP == Op64::Vjp ? 2 : 3) k_cells_fp64(const __grid_constant__ Args64 a) {
     constexpr bool JAC = OP == Op64::Jacobian, JVP = OP == Op64::Jvp, VJP = OP == Op64::Vjp;
     constexpr bool DIR = JVP || VJP;
-    constexpr int NF = DIR ? 4 : 3;         // tile fields: p, depth, mobility, direction
+    constexpr int NF = VJP ? 5 : DIR ? 4 : 3;  // tile fields: p, depth, mobility, direction, k
     constexpr int L = DIAG ? 11 : 7;        // values of an interior row
     extern __shared__ __align__(16) double sm64[];
     const GridGeom& g = a.g;
@@ -128,6 +183,7 @@ __global__ void __launch_bounds__(kMaxThreads, OP == Op64::Vjp ? 2 : 3) k_cells_
     const int sp = (ly + 1) * PX + lx + 1;
     const bool xm = i > 0, xp = i + 1 < nx, ym = j > 0, yp = j + 1 < ny;
 
+    const bool lnk = VJP && a.g_lnk;
     auto load_cell = [&](int c) { return make_cell(q, a.f.p[c], a.f.z[c]); };
     auto put_cell = [&](double* P, int s, const CellVal<double>& v) {
         P[s] = v.p;
@@ -149,11 +205,13 @@ __global__ void __launch_bounds__(kMaxThreads, OP == Op64::Vjp ? 2 : 3) k_cells_
             const int c = ci + nx * cj + nxy * k;
             put_cell(P, y * PX + x, load_cell(c));
             if (DIR) P[3 * NP + y * PX + x] = a.dir[c];
+            if (VJP && lnk) P[4 * NP + y * PX + x] = a.kperm[c];
         }
     };
 
     CellVal<double> me = load_cell(own + nxy * kA);
     double dme = DIR ? a.dir[own + nxy * kA] : 0.0;
+    double kme = VJP && lnk ? a.kperm[own + nxy * kA] : 0.0, kdn = 0.0;  // k of this cell and the one below
     // the vertical link below this plane, from this cell's side
     LinkOut<double> zl{};
     double Tzm = 0.0, ddn = 0.0;  // its T; the direction's difference (and v_L, tie partner) for it
@@ -168,11 +226,13 @@ __global__ void __launch_bounds__(kMaxThreads, OP == Op64::Vjp ? 2 : 3) k_cells_
             vdn = a.dir[c];
             ddn = JVP ? __dsub_rn(vdn, dme) : __dsub_rn(dme, vdn);
         }
+        if (VJP && lnk) kdn = a.kperm[c];
         zl_other = up.Db;
     }
     if (in) {
         put_cell(sm64 + (kA & 1) * NF * NP, sp, me);
         if (DIR) sm64[((kA & 1) * NF + 3) * NP + sp] = dme;
+        if (VJP && lnk) sm64[((kA & 1) * NF + 4) * NP + sp] = kme;
     }
     fill_rim(sm64 + (kA & 1) * NF * NP, kA);
 
@@ -213,10 +273,11 @@ __global__ void __launch_bounds__(kMaxThreads, OP == Op64::Vjp ? 2 : 3) k_cells_
         }
         // the cell above: the vertical link's other end now, this thread's cell next
         CellVal<double> up = me;
-        double dup = dme;
+        double dup = dme, kup = kme;
         if (zp) {
             up = load_cell(c + nxy);
             if (DIR) dup = a.dir[c + nxy];
+            if (VJP && lnk) kup = a.kperm[c + nxy];
         }
 
         // staging position of this row's values
@@ -226,6 +287,8 @@ __global__ void __launch_bounds__(kMaxThreads, OP == Op64::Vjp ? 2 : 3) k_cells_
                             (int)(axis_links_before(i, nx) - axis_links_before(i0, nx)) * perx;
 
         Sums<OP> sum;
+        Perm pm;
+        if (VJP && lnk) pm.set(a.lg, kme);
         auto neighbour = [&](int s) {
             return CellVal<double>{P[s], P[NP + s], P[2 * NP + s]};
         };
@@ -239,9 +302,10 @@ __global__ void __launch_bounds__(kMaxThreads, OP == Op64::Vjp ? 2 : 3) k_cells_
                 if (DIR) {
                     const double dn = P[3 * NP + sp + off];
                     dv = JVP ? __dsub_rn(dn, dme) : __dsub_rn(dme, dn);
-                    if (VJP && zero_flux(l)) sum.tie(l.Da, link(q, T[S], nb, me).Db, dn);
+                    // (a flat tie has equal pressures: its term is zero)
+                    if (VJP && !FLAT && zero_flux(l)) sum.tie(l.Da, link(q, T[S], nb, me).Db, dn);
                 }
-                sum.template add<S, FLAT>(l, T[S], dv);
+                sum.template add<S, FLAT>(l, T[S], dv, pm, VJP && lnk ? P[4 * NP + sp + off] : 0.0);
                 if (JAC && act) row[slot_pos(mask, S)] = l.Db;
             }
         };
@@ -258,7 +322,7 @@ __global__ void __launch_bounds__(kMaxThreads, OP == Op64::Vjp ? 2 : 3) k_cells_
         };
 
         if (zm) {  // slot 0
-            sum.template add<0, false>(zl, Tzm, ddn);
+            sum.template add<0, false>(zl, Tzm, ddn, pm, kdn);
             if (VJP && zero_flux(zl)) sum.tie(zl.Da, zl_other, vdn);
             if (JAC && act) row[0] = zl.Db;
         }
@@ -277,7 +341,7 @@ __global__ void __launch_bounds__(kMaxThreads, OP == Op64::Vjp ? 2 : 3) k_cells_
             zl = tie ? link(q, Tz, up, me) : flip(l);
             double dv = 0.0;
             if (DIR) dv = JVP ? __dsub_rn(dup, dme) : __dsub_rn(dme, dup);
-            sum.template add<10, false>(l, Tz, dv);
+            sum.template add<10, false>(l, Tz, dv, pm, kup);
             if (VJP && tie) sum.tie(l.Da, zl.Db, dup);
             if (JAC && act) row[slot_pos(mask, 10)] = l.Db;
             Tzm = Tz;
@@ -313,13 +377,7 @@ __global__ void __launch_bounds__(kMaxThreads, OP == Op64::Vjp ? 2 : 3) k_cells_
             bad = nonfinite(gp);
             if (act) a.out[c] = gp;
             if (a.g_lnk) {
-                // k_L / (k_K + k_L) = T (d/A) / (2 k_K); an impermeable cell's links have T = 0
-                const double kk = a.kperm[c];
-                double gk = __dmul_rn(sum.gx, a.lg.cx);
-                gk = __fma_rn(sum.gy, a.lg.cy, gk);
-                gk = __fma_rn(sum.gz, a.lg.cz, gk);
-                gk = __fma_rn(sum.gd, a.lg.cd, gk);
-                gk = gk != 0.0 ? gk / (2.0 * kk) : 0.0;
+                const double gk = act && sum.divide ? lnk_by_division(a, i, j, k) : sum.lnk;
                 bad = bad || nonfinite(gk);
                 if (act) a.g_lnk[c] = gk;
             }
@@ -331,11 +389,14 @@ __global__ void __launch_bounds__(kMaxThreads, OP == Op64::Vjp ? 2 : 3) k_cells_
             if (in) {
                 put_cell(N, sp, up);
                 if (DIR) N[3 * NP + sp] = dup;
+                if (VJP && lnk) N[4 * NP + sp] = kup;
             }
             fill_rim(N, k + 1);
         }
         me = up;
         dme = dup;
+        kdn = kme;
+        kme = kup;
     }
     if (JAC) {
         __syncthreads();
@@ -360,7 +421,7 @@ int run_length(long long tiles, int planes, int sms) {
 
 template <Op64 OP, bool DIAG, bool CRK>
 cudaError_t launch64(Args64& a, cudaStream_t st) {
-    constexpr int NF = OP == Op64::Jvp || OP == Op64::Vjp ? 4 : 3, L = DIAG ? 11 : 7;
+    constexpr int NF = OP == Op64::Vjp ? 5 : OP == Op64::Jvp ? 4 : 3, L = DIAG ? 11 : 7;
     int dev = 0, sms = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);

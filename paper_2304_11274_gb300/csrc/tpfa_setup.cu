@@ -85,11 +85,6 @@ __device__ __forceinline__ Pair32 pair_step(float c, Pair32 t, Pair32 s) {
     const float h = __fadd_rn(c, p);
     return {h, __fadd_rn(__fsub_rn(p, __fsub_rn(h, c)), e)};
 }
-__device__ __forceinline__ float rcp_approx(float x) {  // 1/x within 2^-23
-    float r;
-    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
-    return r;
-}
 // num / d: the quotient h of the leading parts and the remainder over d
 __device__ __forceinline__ Pair32 pair_div(Pair32 num, Pair32 d) {
     const float q = rcp_approx(d.h);
