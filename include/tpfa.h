@@ -200,6 +200,20 @@ int tpfa_set_permeability(tpfa_handle h, const double* perm_dev, void* stream);
 int tpfa_set_log_permeability(tpfa_handle h, const double* log_perm_dev, void* stream);
 
 /*
+ * For a forward pass and its adjoint with other calls between them.
+ * tpfa_tag_log_permeability is tpfa_set_log_permeability and writes a tag of this
+ * permeability to tag_dev (8 bytes on the device).
+ * tpfa_restore_log_permeability, with the same ln k and that tag, binds it again:
+ * one launch that computes nothing if the grid still holds the tagged
+ * permeability.  The tag is compared on the device when the launch runs, so
+ * whatever replaced the permeability in between (another call, another thread, a
+ * replayed CUDA graph) is seen.
+ */
+int tpfa_tag_log_permeability(tpfa_handle h, const double* log_perm_dev, unsigned long long* tag_dev, void* stream);
+int tpfa_restore_log_permeability(tpfa_handle h, const double* log_perm_dev, const unsigned long long* tag_dev,
+                                  void* stream);
+
+/*
  * Adjoint of the residual (vector-Jacobian products) at the bound state:
  *   g_p[i]   = sum_K v_K dR_K/dp_i              (= J^T v)
  *   g_lnk[i] = sum_K v_K dR_K/d(ln k_i)         (natural log)

@@ -79,6 +79,8 @@ SIGNATURES = [
     ("tpfa_assemble_jacobian_host", _I, [_VP, _VP, _VP, _VP, _VP, _VP]),
     ("tpfa_set_permeability", _I, [_VP, _VP, _VP]),
     ("tpfa_set_log_permeability", _I, [_VP, _VP, _VP]),
+    ("tpfa_tag_log_permeability", _I, [_VP, _VP, _VP, _VP]),
+    ("tpfa_restore_log_permeability", _I, [_VP, _VP, _VP, _VP]),
     ("tpfa_vjp", _I, [_VP, _VP, _VP, _VP, _VP]),
     ("tpfa_vjp_kernel", _I, [_VP, ctypes.c_int, _VP, _VP, _VP, _VP]),
     ("tpfa_jvp", _I, [_VP, _VP, _VP, _VP, _VP]),

@@ -84,7 +84,6 @@ class Grid:
         self.nnz = int(nnz.value)
         self._p = None
         self._pn = None
-        self._perm_set = 0  # how often the permeability was replaced
 
     def _create(self, h, prm, k, ph, z):
         check(self.lib.tpfa_create_grid(ctypes.byref(h), self.nx, self.ny, self.nz, ctypes.byref(prm),
@@ -167,7 +166,6 @@ class Grid:
         k = _dev_f64(perm, self.device)
         if k.numel() != self.n:
             raise ValueError(f"expected {self.n} values, got {k.numel()}")
-        self._perm_set += 1
         check(self.lib.tpfa_set_permeability(self.handle, _ptr(k), _stream(stream)))
         self._perm = k  # read asynchronously: keep it alive
 
@@ -177,9 +175,22 @@ class Grid:
         lk = _dev_f64(log_k, self.device)
         if lk.numel() != self.n:
             raise ValueError(f"expected {self.n} values, got {lk.numel()}")
-        self._perm_set += 1
         check(self.lib.tpfa_set_log_permeability(self.handle, _ptr(lk), _stream(stream)))
         self._perm = lk  # read asynchronously: keep it alive
+
+    def _tagged_log_permeability(self, log_k, tag=None):
+        """Binds log_k and returns its tag (an int64 tensor), or, given the tag,
+        binds it again unless the grid still holds it (decided on the device)."""
+        lk = _dev_f64(log_k, self.device)
+        if lk.numel() != self.n:
+            raise ValueError(f"expected {self.n} values, got {lk.numel()}")
+        call = self.lib.tpfa_restore_log_permeability
+        if tag is None:
+            tag = torch.empty(1, dtype=torch.int64, device=self.device)
+            call = self.lib.tpfa_tag_log_permeability
+        check(call(self.handle, _ptr(lk), _ptr(tag), _stream()))
+        self._perm = lk  # read asynchronously: keep it alive
+        return tag
 
     def vjp(self, v, want_lnk=True, kernel="auto", stream=None):
         """(g_p, g_lnk) = (v^T dR/dp, v^T dR/d ln k) at the bound state, FP64."""
@@ -518,14 +529,13 @@ class TPFAResidual(torch.autograd.Function):
     forward(grid, p, log_k) -> R (FP64, N).  log_k is the natural log of the
     permeability; the grid's transmissibilities are recomputed from it in the
     forward pass, and again in the backward pass if the grid's permeability
-    was replaced in between (by another forward, or by the caller).  backward
-    runs the library's adjoint kernel (checkpoint-free: nothing is saved but p
-    and log_k)."""
+    was replaced in between (by another forward, the caller or a CUDA graph).
+    backward runs the library's adjoint kernel (checkpoint-free: nothing is
+    saved but p, log_k and the permeability's tag)."""
 
     @staticmethod
     def forward(ctx, grid, p, log_k):
-        grid.set_log_permeability(log_k.detach())
-        ctx.perm_set = grid._perm_set
+        ctx.tag = grid._tagged_log_permeability(log_k.detach())
         grid.set_pressure(p.detach())
         R = grid.assemble_residual()
         ctx.grid = grid
@@ -536,8 +546,7 @@ class TPFAResidual(torch.autograd.Function):
     def backward(ctx, gR):
         p, log_k = ctx.saved_tensors  # raises if one was modified in place
         grid = ctx.grid
-        if grid._perm_set != ctx.perm_set:
-            grid.set_log_permeability(log_k.detach())
+        grid._tagged_log_permeability(log_k.detach(), ctx.tag)
         grid.set_pressure(p.detach())
         g_p, g_lnk = grid.vjp(gR.detach(), want_lnk=ctx.needs_input_grad[2])
         gp = g_p.to(p.dtype) if ctx.needs_input_grad[1] else None

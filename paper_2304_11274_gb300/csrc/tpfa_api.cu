@@ -107,6 +107,7 @@ struct tpfa_grid {
     void* z = nullptr;
     void* kperm = nullptr;  // permeability in the field type (adjoint)
     float2* vsplit = nullptr;  // the mixed adjoint's cotangent as FP32 pairs (allocated on first use)
+    unsigned long long* perm_set = nullptr;  // device: how often the permeability was replaced (PermTag)
     LinkGeo lg{};           // distance / area per link direction (adjoint)
     LinkGeoD lgd{};         // the same for the FP64 path
     double* phi0_d = nullptr;
@@ -198,6 +199,8 @@ struct tpfa_grid {
         for (auto& t : T) dev_free(t), t = nullptr;
         dev_free(z);
         dev_free(kperm);
+        dev_free(perm_set);
+        perm_set = nullptr;
         dev_free(vsplit);
         vsplit = nullptr;
         dev_free(phi0_d);
@@ -703,6 +706,7 @@ int tpfa_create_grid(tpfa_handle* out, int nx, int ny, int nz, const tpfa_params
     for (int t = 0; t < nT && ok; ++t) ok = dev_alloc(&h->T[t], rb) == cudaSuccess;
     ok = ok && dev_alloc(&h->z, rb) == cudaSuccess;
     ok = ok && dev_alloc(&h->kperm, rb) == cudaSuccess;
+    ok = ok && dev_alloc((void**)&h->perm_set, sizeof(unsigned long long)) == cudaSuccess;
     ok = ok && dev_alloc((void**)&h->phi0_d, sizeof(double) * (size_t)N) == cudaSuccess;
     if (ok && h->crk) ok = dev_alloc(&h->phi0_r, rb) == cudaSuccess;
     ok = ok && dev_alloc((void**)&h->mn, sizeof(double) * (size_t)N) == cudaSuccess;
@@ -714,6 +718,7 @@ int tpfa_create_grid(tpfa_handle* out, int nx, int ny, int nz, const tpfa_params
         return fail(TPFA_ERR_OOM, "device allocation failed for a %d x %d x %d grid", nx, ny, nz);
     }
     e = cudaMemsetAsync(h->status, 0, sizeof(unsigned int), st);
+    if (e == cudaSuccess) e = cudaMemsetAsync(h->perm_set, 0, sizeof(unsigned long long), st);
     if (e == cudaSuccess) {
         if (prec == TPFA_MIXED)
             e = launch_transmissibility_f32(h->geom, h->sp, perm_dev, (float*)h->T[0], (float*)h->T[1], (float*)h->T[2],
@@ -917,20 +922,22 @@ int tpfa_assemble_jacobian_host(tpfa_handle h, const void* p_host, double* R_hos
 }
 
 namespace {
-int set_perm(tpfa_handle h, const double* perm_dev, void* stream, bool log_k) {
+int set_perm(tpfa_handle h, const double* perm_dev, void* stream, bool log_k, unsigned long long* take = nullptr,
+             const unsigned long long* held = nullptr) {
     int rc = check_handle(h);
     if (rc) return rc;
     if (!perm_dev) return fail(TPFA_ERR_INVALID_ARG, "perm must be non-NULL");
     DeviceGuard dg(h->device);
     cudaStream_t st = static_cast<cudaStream_t>(stream);
+    const PermTag tag{h->perm_set, take, held};
     cudaError_t e;
     if (h->prec == TPFA_MIXED)
         e = launch_transmissibility_f32(h->geom, h->sp, perm_dev, (float*)h->T[0], (float*)h->T[1], (float*)h->T[2],
-                                        (float*)h->T[3], (float*)h->T[4], (float*)h->kperm, st, log_k);
+                                        (float*)h->T[3], (float*)h->T[4], (float*)h->kperm, st, log_k, tag);
     else
         e = launch_transmissibility_f64(h->geom, h->sp, perm_dev, (double*)h->T[0], (double*)h->T[1],
                                         (double*)h->T[2], (double*)h->T[3], (double*)h->T[4], (double*)h->kperm, st,
-                                        log_k);
+                                        log_k, tag);
     if (e != cudaSuccess) return cuda_fail(e, "set_permeability launch");
     return TPFA_OK;
 }
@@ -942,6 +949,17 @@ int tpfa_set_permeability(tpfa_handle h, const double* perm_dev, void* stream) {
 
 int tpfa_set_log_permeability(tpfa_handle h, const double* log_perm_dev, void* stream) {
     return set_perm(h, log_perm_dev, stream, true);
+}
+
+int tpfa_tag_log_permeability(tpfa_handle h, const double* log_perm_dev, unsigned long long* tag_dev, void* stream) {
+    if (!tag_dev) return fail(TPFA_ERR_INVALID_ARG, "tag must be non-NULL");
+    return set_perm(h, log_perm_dev, stream, true, tag_dev, nullptr);
+}
+
+int tpfa_restore_log_permeability(tpfa_handle h, const double* log_perm_dev, const unsigned long long* tag_dev,
+                                  void* stream) {
+    if (!tag_dev) return fail(TPFA_ERR_INVALID_ARG, "tag must be non-NULL");
+    return set_perm(h, log_perm_dev, stream, true, nullptr, tag_dev);
 }
 
 int tpfa_vjp_kernel(tpfa_handle h, tpfa_kernel kern, const double* v_dev, double* g_p_dev, double* g_lnk_dev,

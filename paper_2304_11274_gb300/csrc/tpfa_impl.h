@@ -50,16 +50,25 @@ struct SetupPhys {
     double dx, dy, dz;
     double rho_ref, p_ref, c_f, c_r, V_dt;
 };
+// Which permeability a grid's transmissibilities come from, on the device: every
+// launch that computes them counts `set` up.  A tag takes the count (`take`), and
+// a launch with `held` computes nothing if the count is still that tag's.
+struct PermTag {
+    unsigned long long* set = nullptr;
+    unsigned long long* take = nullptr;
+    const unsigned long long* held = nullptr;
+};
 // Owned transmissibilities from permeability, computed in FP64 and stored as
 // `Real` (float or double).  Tpp/Tmp may be null with 6-point connectivity.
 // With log_k the array holds ln k and k = exp(ln k) is formed here.  kperm
 // (may be null) receives k in the path's precision, the adjoint's copy.
 cudaError_t launch_transmissibility_f32(const GridGeom& g, const SetupPhys& s, const double* perm,
                                         float* Tx, float* Ty, float* Tz, float* Tpp, float* Tmp, float* kperm,
-                                        cudaStream_t st, bool log_k = false);
+                                        cudaStream_t st, bool log_k = false, const PermTag& tag = PermTag());
 cudaError_t launch_transmissibility_f64(const GridGeom& g, const SetupPhys& s, const double* perm,
                                         double* Tx, double* Ty, double* Tz, double* Tpp, double* Tmp,
-                                        double* kperm, cudaStream_t st, bool log_k = false);
+                                        double* kperm, cudaStream_t st, bool log_k = false,
+                                        const PermTag& tag = PermTag());
 cudaError_t launch_convert_f32(const double* in, float* out, long long n, cudaStream_t st);
 cudaError_t launch_copy_f64(const double* in, double* out, long long n, cudaStream_t st);
 // m^n = (V/dt) phi(p^n) rho(p^n) in FP64 from p^n of either field type.

@@ -217,7 +217,15 @@ constexpr int kTransRun = 4;      // planes a block walks (its next plane's own 
 template <typename Real, bool LOG>
 __global__ void __launch_bounds__(kTileThreads)
     k_trans(GridGeom g, Geo geo, int TX, int TY, const double* __restrict__ perm, Real* Tx, Real* Ty, Real* Tz,
-            Real* Tpp, Real* Tmp, Real* kperm) {
+            Real* Tpp, Real* Tmp, Real* kperm, PermTag tag) {
+    // (the count only grows, so a block that reads it after block 0 has counted
+    // this launch decides as the others)
+    if (tag.held && *tag.held == *static_cast<const volatile unsigned long long*>(tag.set)) return;
+    if (tag.set && blockIdx.x == 0 && threadIdx.x == 0) {
+        const unsigned long long n = *tag.set + 1;
+        *tag.set = n;
+        if (tag.take) *tag.take = n;
+    }
     using R = Tile<Real>;
     using RT = typename R::type;
     // (TX + 2)(TY + 1) with TX TY <= 256 and TX <= 128 is at most 3 * 257
@@ -382,7 +390,8 @@ __global__ void k_pattern(GridGeom g, long long* row_ptr, int* col_idx) {
 
 template <typename Real>
 static cudaError_t launch_trans_t(const GridGeom& g, const SetupPhys& s, const double* perm, Real* Tx, Real* Ty,
-                                  Real* Tz, Real* Tpp, Real* Tmp, Real* kperm, cudaStream_t st, bool log_k) {
+                                  Real* Tz, Real* Tpp, Real* Tmp, Real* kperm, cudaStream_t st, bool log_k,
+                                  const PermTag& tag) {
     // one block index for tiles and z-runs: any grid shape of fewer than 2^31 cells fits
     int TX = 1, TY = 1;
     tile_shape(g.nx, g.ny, kTileThreads, TX, TY);
@@ -390,21 +399,21 @@ static cudaError_t launch_trans_t(const GridGeom& g, const SetupPhys& s, const d
                          ((g.nz + kTransRun - 1) / kTransRun);
     const int block = (TX * TY + 31) / 32 * 32;
     const Geo q = make_geo(s);
-    if (log_k) k_trans<Real, true><<<(unsigned)nb, block, 0, st>>>(g, q, TX, TY, perm, Tx, Ty, Tz, Tpp, Tmp, kperm);
-    else k_trans<Real, false><<<(unsigned)nb, block, 0, st>>>(g, q, TX, TY, perm, Tx, Ty, Tz, Tpp, Tmp, kperm);
+    if (log_k) k_trans<Real, true><<<(unsigned)nb, block, 0, st>>>(g, q, TX, TY, perm, Tx, Ty, Tz, Tpp, Tmp, kperm, tag);
+    else k_trans<Real, false><<<(unsigned)nb, block, 0, st>>>(g, q, TX, TY, perm, Tx, Ty, Tz, Tpp, Tmp, kperm, tag);
     return cudaGetLastError();
 }
 
 cudaError_t launch_transmissibility_f32(const GridGeom& g, const SetupPhys& s, const double* perm, float* Tx,
                                         float* Ty, float* Tz, float* Tpp, float* Tmp, float* kperm, cudaStream_t st,
-                                        bool log_k) {
-    return launch_trans_t<float>(g, s, perm, Tx, Ty, Tz, Tpp, Tmp, kperm, st, log_k);
+                                        bool log_k, const PermTag& tag) {
+    return launch_trans_t<float>(g, s, perm, Tx, Ty, Tz, Tpp, Tmp, kperm, st, log_k, tag);
 }
 
 cudaError_t launch_transmissibility_f64(const GridGeom& g, const SetupPhys& s, const double* perm, double* Tx,
                                         double* Ty, double* Tz, double* Tpp, double* Tmp, double* kperm,
-                                        cudaStream_t st, bool log_k) {
-    return launch_trans_t<double>(g, s, perm, Tx, Ty, Tz, Tpp, Tmp, kperm, st, log_k);
+                                        cudaStream_t st, bool log_k, const PermTag& tag) {
+    return launch_trans_t<double>(g, s, perm, Tx, Ty, Tz, Tpp, Tmp, kperm, st, log_k, tag);
 }
 
 cudaError_t launch_convert_f32(const double* in, float* out, long long n, cudaStream_t st) {
