@@ -359,23 +359,27 @@ int tpfa_slab_exchange(tpfa_handle lower, void* p_lower_dev, tpfa_handle upper, 
  * Tiling of the assembly kernel: a warp marches along y over
  * `rows_per_march` (1 to 64) rows of a 32-cell x-segment, and a block stacks
  * `warps_per_block` (4 or 8) consecutive z-planes.  Results do not depend on
- * the tiling (every row is summed in the same order); only speed does.  The
- * J w and adjoint marches use the same tiling, with the rows per march
- * halved (down to 8) while the launch has fewer than three or four blocks per
- * multiprocessor.  Until a tiling is set or autotuned, the marches choose
- * fewer than the default 32 rows on grids whose blocks would not fill the
- * GPU.  The FP64 path's tiles follow from the grid alone.
+ * the tiling (every row is summed in the same order); only speed does.  Until
+ * a tiling is set, every mixed launch chooses its own rows per march, at most 32,
+ * with four warps per block; after tpfa_set_tiling the J w and adjoint marches
+ * halve the given rows (down to 8) while the launch has fewer than three or
+ * four blocks per multiprocessor.  tpfa_get_tiling returns what was set or what
+ * tpfa_autotune preferred, else 32 and 4.  The FP64 path's tiles follow from
+ * the grid alone.
  */
 int tpfa_set_tiling(tpfa_handle h, int rows_per_march, int warps_per_block);
 int tpfa_get_tiling(tpfa_handle h, int* rows_per_march, int* warps_per_block);
 
 /*
- * Choose the tiling by timing candidates (rows_per_march 8, 16, 24, 32, 40,
- * 48, 64 x warps_per_block 4, 8) on this grid at its bound state, or take it from
- * `cache_path` (a text file of "key rows warps" lines, key = device, path,
- * connectivity, porosity law and log2 of the cell count); a new choice is
- * written back.  cache_path may be NULL (no cache).  Allocates and frees
- * temporary outputs on `stream` and synchronises it.
+ * Choose the tiling of the residual + Jacobian assembly by timing it on this grid
+ * at its bound state: the launch's own choice, and rows_per_march 8, 16, 24, 32,
+ * 40, 48, 64 x warps_per_block 4, 8, one of which must be 2 % faster.  Or take it
+ * from `cache_path` (a text file of "key rows warps" lines, key = device, path,
+ * connectivity, porosity law and extents; rows 0: the launch's own choice); a
+ * new choice is written back.  cache_path may be NULL (no cache).  A tiling set
+ * before is given up; the other operations choose their own.  Allocates and
+ * frees temporary outputs on `stream` and synchronises it (mixed path; the FP64
+ * path has nothing to time).
  */
 int tpfa_autotune(tpfa_handle h, const char* cache_path, void* stream);
 

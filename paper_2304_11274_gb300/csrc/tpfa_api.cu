@@ -91,6 +91,8 @@ cudaError_t ensure_smem_limit(const void* func, int bytes) {
 }
 }  // namespace tpfa
 
+constexpr int kDefaultRows = 32, kDefaultWarps = 4;
+
 struct tpfa_grid {
     int device = 0;
     int nx = 0, ny = 0, nz = 0;
@@ -120,10 +122,11 @@ struct tpfa_grid {
     const void* p = nullptr;
     const void* pn = nullptr;
     bool has_state = false;
-    int JY = 32;  // rows per warp march (tpfa_set_tiling, tpfa_autotune)
-    bool tiling_set = false;  // JY was set by one of them; else the launches choose (rows_for)
+    int JY = kDefaultRows;  // rows per warp march
+    bool tiling_set = false;  // JY and W were set (tpfa_set_tiling); else the launches choose (rows_for)
     int sms = 0;  // multiprocessors of the grid's device
-    int W = 4;    // warps (z-planes) per block
+    int W = kDefaultWarps;  // warps (z-planes) per block
+    int tuned_JY = 0, tuned_W = 0;  // R + J's, if timing preferred them (tpfa_autotune)
     // a z-slab of a larger grid (tpfa_create_slab): the handle's planes are
     // the slab and its one-plane halos; assemblies write the rows of the
     // owned planes [own0, own1) only
@@ -346,12 +349,14 @@ int launch(tpfa_grid* h, AsmKernel kern, double* R, void* vals, double* diag64, 
     if (h->prec == TPFA_MIXED) {
         AsmOut<float> o{R, static_cast<float*>(vals), diag64, h->status};
         const bool two = kern == AsmKernel::XMarch && xmarch_ok(h->geom, fields_of<float>(h));
-        const int rows = rows_for(h, two ? 64 : 32, (k1 < 0 ? h->nz : k1) - k0, two && vals ? 3 : 4);
+        const bool tuned = vals && h->tuned_JY;
+        const int W = tuned ? h->tuned_W : h->W;
+        const int rows = tuned ? h->tuned_JY : rows_for(h, two ? 64 : 32, (k1 < 0 ? h->nz : k1) - k0, two && vals ? 3 : 4);
         if (kern == AsmKernel::YMarchTma)
-            e = launch_assemble_mixed_tma(h->geom, h->qf, h->crk, fields_of<float>(h), o, h->tm, rows, h->W, st, k0,
+            e = launch_assemble_mixed_tma(h->geom, h->qf, h->crk, fields_of<float>(h), o, h->tm, rows, W, st, k0,
                                           k1);
         else
-            e = launch_assemble_mixed(kern, h->geom, h->qf, h->crk, fields_of<float>(h), o, rows, h->W, st, k0, k1);
+            e = launch_assemble_mixed(kern, h->geom, h->qf, h->crk, fields_of<float>(h), o, rows, W, st, k0, k1);
     } else {
         AsmOut<double> o{R, static_cast<double*>(vals), nullptr, h->status};
         e = launch_assemble_fp64(kern, h->geom, h->qd, h->crk, fields_of<double>(h), o, st, k0, k1);
@@ -1452,7 +1457,8 @@ int tpfa_destroy_mesh(tpfa_mesh m) {
 
 namespace {
 
-// Autotune cache: a text file of "key JY W" lines (a header line starts with '#').
+// Autotune cache: a text file of "key JY W" lines (a header line starts with
+// '#'); JY = 0: the launches' own choice.
 std::map<std::string, std::pair<int, int>> cache_read(const char* path) {
     std::map<std::string, std::pair<int, int>> m;
     if (!path) return m;
@@ -1463,7 +1469,7 @@ std::map<std::string, std::pair<int, int>> cache_read(const char* path) {
     char line[512];
     while (fgets(line, sizeof line, fp)) {
         if (line[0] == '#') continue;
-        if (sscanf(line, "%255s %d %d", key, &jy, &w) == 3 && jy >= 1 && jy <= 64 && (w == 4 || w == 8))
+        if (sscanf(line, "%255s %d %d", key, &jy, &w) == 3 && jy >= 0 && jy <= 64 && (w == 4 || w == 8))
             m[key] = {jy, w};
     }
     fclose(fp);
@@ -1651,52 +1657,59 @@ int tpfa_set_tiling(tpfa_handle h, int rows_per_march, int warps_per_block) {
     h->JY = rows_per_march;
     h->W = warps_per_block;
     h->tiling_set = true;
+    h->tuned_JY = h->tuned_W = 0;
     return TPFA_OK;
 }
 
 int tpfa_get_tiling(tpfa_handle h, int* rows_per_march, int* warps_per_block) {
     int rc = check_handle(h);
     if (rc) return rc;
-    if (rows_per_march) *rows_per_march = h->JY;
-    if (warps_per_block) *warps_per_block = h->W;
+    if (rows_per_march) *rows_per_march = h->tuned_JY ? h->tuned_JY : h->JY;
+    if (warps_per_block) *warps_per_block = h->tuned_JY ? h->tuned_W : h->W;
     return TPFA_OK;
 }
 
+// The timed candidates are R + J's, so the winner is R + J's alone.  The launches'
+// own choice (rows_for) is the first of them and kept unless another is 2 % faster:
+// timing rows of 8 and more over it made small grids slower (24 x 20 x 16: R + J
+// 10.9 -> 19.1 us, and R alone, J w and the adjoint, which took the winner too,
+// 8.8 -> 12.9, 8.8 -> 15.0 and 13.0 -> 21.1 us).  The key holds the extents, as the
+// choice of march and the segments depend on them.
 int tpfa_autotune(tpfa_handle h, const char* cache_path, void* stream) {
     int rc = check_handle(h);
     if (rc) return rc;
     if (!h->has_state) return fail(TPFA_ERR_NO_STATE, "tpfa_set_state has not been called");
     DeviceGuard dg(h->device);
     char key[256];
-    snprintf(key, sizeof key, "grid/%s/%s/c%d/r%d/n%d", device_tag(h->device).c_str(),
-             h->prec == TPFA_MIXED ? "mixed" : "fp64", h->prm.connectivity, h->crk ? 1 : 0, log2_bucket(h->N));
+    snprintf(key, sizeof key, "grid/%s/%s/c%d/r%d/%dx%dx%d", device_tag(h->device).c_str(),
+             h->prec == TPFA_MIXED ? "mixed" : "fp64", h->prm.connectivity, h->crk ? 1 : 0, h->nx, h->ny, h->nz);
     auto cache = cache_read(cache_path);
     auto it = cache.find(key);
+    const int old_JY = h->JY, old_W = h->W, old_tuned_JY = h->tuned_JY, old_tuned_W = h->tuned_W;
+    const bool old_set = h->tiling_set;
+    h->JY = kDefaultRows, h->W = kDefaultWarps, h->tiling_set = false;
+    h->tuned_JY = h->tuned_W = 0;
     if (it != cache.end()) {
-        h->JY = it->second.first;
-        h->W = it->second.second;
-        h->tiling_set = true;
+        if (it->second.first) h->tuned_JY = it->second.first, h->tuned_W = it->second.second;
         return TPFA_OK;
     }
-    cudaStream_t st = static_cast<cudaStream_t>(stream);
-    void *R = nullptr, *vals = nullptr, *diag = nullptr;
-    cudaError_t e = cudaMallocAsync(&R, sizeof(double) * (size_t)h->N, st);
-    if (e == cudaSuccess) e = cudaMallocAsync(&vals, h->real_size * (size_t)h->nnz, st);
-    if (e == cudaSuccess && h->prec == TPFA_MIXED) e = cudaMallocAsync(&diag, sizeof(double) * (size_t)h->N, st);
-    cudaEvent_t a = nullptr, b = nullptr;
-    if (e == cudaSuccess) e = cudaEventCreate(&a);
-    if (e == cudaSuccess) e = cudaEventCreate(&b);
-    float best = 1e30f;
-    int bj = h->JY, bw = h->W;
-    const bool was_set = h->tiling_set;
-    h->tiling_set = true;  // the candidates are launched as they are
-    for (int jy : kTuneJY) {
-        for (int w : kTuneW) {
-            if (e != cudaSuccess) break;
-            h->JY = jy;
-            h->W = w;
+    int bj = 0, bw = kDefaultWarps;
+    cudaError_t e = cudaSuccess;
+    if (h->prec == TPFA_MIXED) {  // the FP64 path's tiles follow from the grid
+        cudaStream_t st = static_cast<cudaStream_t>(stream);
+        void *R = nullptr, *vals = nullptr, *diag = nullptr;
+        e = cudaMallocAsync(&R, sizeof(double) * (size_t)h->N, st);
+        if (e == cudaSuccess) e = cudaMallocAsync(&vals, h->real_size * (size_t)h->nnz, st);
+        if (e == cudaSuccess) e = cudaMallocAsync(&diag, sizeof(double) * (size_t)h->N, st);
+        cudaEvent_t a = nullptr, b = nullptr;
+        if (e == cudaSuccess) e = cudaEventCreate(&a);
+        if (e == cudaSuccess) e = cudaEventCreate(&b);
+        float best = 1e30f;
+        const auto time = [&](int jy, int w) {
+            if (e != cudaSuccess || rc) return;
+            h->tuned_JY = jy, h->tuned_W = w;
             for (int r = 0; r < 2 && !rc; ++r) rc = launch(h, auto_kernel(h), (double*)R, vals, (double*)diag, st);
-            if (rc) break;
+            if (rc) return;
             cudaEventRecord(a, st);
             for (int r = 0; r < 5 && !rc; ++r) rc = launch(h, auto_kernel(h), (double*)R, vals, (double*)diag, st);
             cudaEventRecord(b, st);
@@ -1704,20 +1717,23 @@ int tpfa_autotune(tpfa_handle h, const char* cache_path, void* stream) {
             float ms = 0.f;
             if (e == cudaSuccess) e = cudaEventElapsedTime(&ms, a, b);
             if (e == cudaSuccess && ms < best) best = ms, bj = jy, bw = w;
-        }
-        if (rc) break;
+        };
+        time(0, kDefaultWarps);
+        best *= 0.98f;
+        for (int jy : kTuneJY)
+            for (int w : kTuneW) time(jy, w);
+        if (a) cudaEventDestroy(a);
+        if (b) cudaEventDestroy(b);
+        if (R) cudaFreeAsync(R, st);
+        if (vals) cudaFreeAsync(vals, st);
+        if (diag) cudaFreeAsync(diag, st);
+        cudaStreamSynchronize(st);
     }
-    if (a) cudaEventDestroy(a);
-    if (b) cudaEventDestroy(b);
-    if (R) cudaFreeAsync(R, st);
-    if (vals) cudaFreeAsync(vals, st);
-    if (diag) cudaFreeAsync(diag, st);
-    cudaStreamSynchronize(st);
-    h->JY = bj;
-    h->W = bw;
-    if (rc || e != cudaSuccess) h->tiling_set = was_set;
-    if (rc) return rc;
-    if (e != cudaSuccess) return cuda_fail(e, "autotune");
+    if (rc || e != cudaSuccess) {
+        h->JY = old_JY, h->W = old_W, h->tiling_set = old_set, h->tuned_JY = old_tuned_JY, h->tuned_W = old_tuned_W;
+        return rc ? rc : cuda_fail(e, "autotune");
+    }
+    h->tuned_JY = bj, h->tuned_W = bj ? bw : 0;
     cache[key] = {bj, bw};
     if (!cache_write(cache_path, cache)) return fail(TPFA_ERR_INVALID_ARG, "cannot write autotune cache %s", cache_path);
     return TPFA_OK;
@@ -1817,7 +1833,7 @@ int tpfa_ensemble_autotune(tpfa_ensemble e, const char* cache_path, void* stream
              e->diag ? 10 : 6, e->crk ? 1 : 0, log2_bucket(cells));
     auto cache = cache_read(cache_path);
     auto it = cache.find(key);
-    if (it != cache.end()) {
+    if (it != cache.end() && it->second.first) {
         e->JY = it->second.first;
         e->W = it->second.second;
         return TPFA_OK;
