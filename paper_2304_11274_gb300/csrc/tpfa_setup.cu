@@ -29,7 +29,7 @@ __device__ __forceinline__ double two_point(double kK, double kL, double area_ov
 
 struct Geo {
     double ax, ay, az, ad;  // area / distance of x, y, z faces and of an in-plane diagonal
-    float2 px, py, pz, pd;  // twice that as FP32 pairs
+    float2 px, py, pz, pd;  // twice that as FP32 pairs, zero outside their range
 };
 
 // Permeability of cell c: the stored value, or exp of the stored natural
@@ -325,7 +325,9 @@ Geo make_geo(const SetupPhys& s) {
     q.az = s.dx * s.dy / s.dz;
     // diagonal: distance sqrt(dx^2 + dy^2), area dz dx dy / distance
     q.ad = s.dz * s.dx * s.dy / (s.dx * s.dx + s.dy * s.dy);
+    // outside the pairs' range (pair_range): zero, whose links the FP64 formula decides
     auto pair = [](double v) {
+        if (!(v >= 0x1p-90 && v <= 0x1p90)) return make_float2(0.f, 0.f);
         const float h = (float)v;
         return make_float2(h, (float)(v - (double)h));
     };
