@@ -23,7 +23,12 @@ PRECISIONS = {"fp64": TPFA_FP64, "mixed": TPFA_MIXED}
 # The library's functions declare their argument types, so addresses and
 # stream handles are passed as plain integers.  The current stream is asked
 # for as a raw handle: torch.cuda.current_stream() builds a Stream object,
-# 3 us of the 10 to 15 us that a call on a small grid costs the host.
+# 3 us of the 10 to 15 us that a call on a small grid costs the host.  The raw
+# calls are torch's internal ones: without them the public one is used.
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+_current_device = getattr(torch._C, "_cuda_getDevice", None)
+
+
 def _ptr(t: torch.Tensor | None):
     return t.data_ptr() if t is not None else None
 
@@ -31,7 +36,9 @@ def _ptr(t: torch.Tensor | None):
 def _stream(stream=None):
     if stream is not None:
         return stream.cuda_stream
-    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+    if _raw_stream is None or _current_device is None:
+        return torch.cuda.current_stream().cuda_stream
+    return _raw_stream(_current_device())
 
 
 def _unused_mesh_params() -> dict:
