@@ -98,6 +98,13 @@ __device__ __forceinline__ float narrow_flush(double x) {
     const uint32_t f = ((a - 0x38000000u) << 3) | (lo >> 29);
     return __uint_as_float((hi & 0x80000000u) | (a >= 0x38100000u ? f : 0u));
 }
+// The same for any x: from 2^128 on an infinity or NaN.
+__device__ __forceinline__ float narrow_sat(double x) {
+    const uint32_t hi = (uint32_t)__double2hiint(x);
+    const uint32_t a = min(hi & 0x7fffffffu, 0x47f00000u);
+    const uint32_t f = ((a - 0x38000000u) << 3) | ((uint32_t)__double2loint(x) >> 29);
+    return __uint_as_float((hi & 0x80000000u) | (a >= 0x38100000u ? f : 0u));
+}
 // Magnitude bits of (float)x for |x| outside [2^-126, 2^128), from its words.
 __device__ __forceinline__ uint32_t narrow_rare(uint32_t a, uint32_t lo) {
     if (a >= 0x47f00000u) return a > 0x7ff00000u || (a == 0x7ff00000u && lo) ? 0x7fc00000u : 0x7f800000u;

@@ -402,7 +402,8 @@ struct XState {
     }
     // w as FP32 (truncated) of ring slots sn (the lane's cells of the row and
     // the halo cell) and sd (planes k - 1 and k + 1): the cheap narrowing, or, if
-    // any of the warp's values lies outside FP32's normal range, the exact one.
+    // any of the warp's values would be an FP32 subnormal, the exact one.  From
+    // 2^128 on either gives an infinity or NaN, and so a row that is computed again.
     // (A test of its own behind each value cost 14 % of J w at 512 x 512 x 256.)
     __device__ __forceinline__ double2 w_ring(int sl, int plane) const {
         return *reinterpret_cast<const double2*>(ring + sl * X::SLOT + X::OFF_W + 128 * plane + 4 * lane);
@@ -410,16 +411,16 @@ struct XState {
     __device__ __forceinline__ XW w_rows(int sn, int sd, float2& zmw, float2& zpw) const {
         const double2 d = w_ring(sn, 0), dm = w_ring(sd, 1), dp = w_ring(sd, 2);
         const double h64 = hact ? reinterpret_cast<const double*>(ring + sn * X::SLOT + X::OFF_W)[192 + (hl ? 1 : 0)] : 0.0;
-        // twice the high words (no sign): outside the normal range, or zero
-        const auto word = [](double x) { return 2u * (uint32_t)__double2hiint(x) - 2u * 0x38100000u; };
-        const uint32_t rare = max(max(max(word(d.x), word(d.y)), max(word(dm.x), word(dm.y))),
-                                  max(max(word(dp.x), word(dp.y)), hact ? word(h64) : 0u));
+        // twice the high words (no sign), from 2^-150 on: (float)x is zero below it
+        const auto word = [](double x) { return 2u * (uint32_t)__double2hiint(x) - 2u * 0x36900000u; };
+        const uint32_t least = min(min(min(word(d.x), word(d.y)), min(word(dm.x), word(dm.y))),
+                                   min(min(word(dp.x), word(dp.y)), word(h64)));
         XW r;
-        r.c = f2(narrow_flush(d.x), narrow_flush(d.y));
-        zmw = f2(narrow_flush(dm.x), narrow_flush(dm.y));
-        zpw = f2(narrow_flush(dp.x), narrow_flush(dp.y));
-        float h = narrow_flush(h64);
-        if (__any_sync(0xffffffffu, act && rare >= 2u * 0x0fe00000u)) {
+        r.c = f2(narrow_sat(d.x), narrow_sat(d.y));
+        zmw = f2(narrow_sat(dm.x), narrow_sat(dm.y));
+        zpw = f2(narrow_sat(dp.x), narrow_sat(dp.y));
+        float h = narrow_sat(h64);
+        if (__any_sync(0xffffffffu, least < 2u * (0x38100000u - 0x36900000u))) {
             r.c = f2(narrow_any(d.x), narrow_any(d.y));
             zmw = f2(narrow_any(dm.x), narrow_any(dm.y));
             zpw = f2(narrow_any(dp.x), narrow_any(dp.y));
