@@ -325,14 +325,22 @@ int rows_for(const tpfa_grid* h, int seg, int planes, int resident) {
 // 224 x 96 x 48, 59.3 vs 91.0 at 512 x 512 x 128.
 AsmKernel residual_kernel(const tpfa_grid* h) { return h->nx >= 64 ? AsmKernel::XMarch : AsmKernel::YMarch; }
 
-// J w: two cells per lane where a row's last segment is not mostly idle (an
-// even number of 32-cell segments) or the row is long.  Measured (10 links, one-
-// cell vs two-cell): 33.2 vs 37.4 at 128^3, 33.0 vs 29.9 at 160 x 160 x 80, 34.1
-// vs 36.8 at 192 x 160 x 80, 27.6 vs 22.2 at 224 x 96 x 48, 40.0 vs 48.3 at
-// 256 x 256 x 128, 44.8 vs 58.0 at 512 x 512 x 128.
+// J w: two cells per lane on grids of 2^21 cells and more where a row's last
+// segment is not mostly idle (an even number of 32-cell segments) or the row is
+// long; with 10 links and whole 64-cell segments from 2^20 cells on.  Smaller
+// launches leave its blocks, fewer and longer than the one-cell march's, too few.
+// Measured (us, 10 links, one-cell vs two-cell): 10 vs 18 at 512 x 2 x 128, 19 vs
+// 23 at 128 x 16 x 128, 26.7 vs 30.8 at 190 x 60 x 50, 39.0 vs 35.0 at 128 x 128 x
+// 64, 53.3 vs 49.6 at 448 x 64 x 50, 49.1 vs 51.4 at 192 x 100 x 70, 63.7 vs 59.3 at
+// 256 x 128 x 64, 78.2 vs 73.7 at 190 x 120 x 110, 101.5 vs 90.2 at 448 x 100 x 80, 213
+// vs 178 at 512 x 128 x 128; 6 links: 27 vs 30 at 128 x 128 x 64 and 256 x 64 x 64, 49.1 vs
+// 47.2 at 256 x 128 x 64, 76.8 vs 69.5 at 448 x 100 x 80.  (Where the planes are few it
+// may lose above that too: 87 vs 113 at 300 x 300 x 30, 10 links.)
 AsmKernel jvp_kernel(const tpfa_grid* h) {
     const int nx = h->nx;
-    return nx >= 256 || (nx >= 128 && (nx + 31) / 32 % 2 == 0) ? AsmKernel::XMarch : AsmKernel::YMarch;
+    const bool wide = nx >= 256 || (nx >= 128 && (nx + 31) / 32 % 2 == 0);
+    const long long least = h->geom.diag && nx % 64 == 0 ? 1LL << 20 : 1LL << 21;
+    return wide && h->N >= least ? AsmKernel::XMarch : AsmKernel::YMarch;
 }
 
 int launch(tpfa_grid* h, AsmKernel kern, double* R, void* vals, double* diag64, cudaStream_t st, int k0 = 0,
