@@ -202,8 +202,52 @@ struct Tile<double> {
     }
 };
 
+// Whether the grid still holds the tagged permeability; else counts this launch.
+// (The count only grows, so a block that reads it after block 0 has counted
+// decides as the others.)
+__device__ __forceinline__ bool still_held(const PermTag& tag) {
+    if (tag.held && *tag.held == *static_cast<const volatile unsigned long long*>(tag.set)) return true;
+    if (tag.set && blockIdx.x == 0 && threadIdx.x == 0) {
+        const unsigned long long n = *tag.set + 1;
+        *tag.set = n;
+        if (tag.take) *tag.take = n;
+    }
+    return false;
+}
+
+// The FP64 formula, a thread per cell: for planes of so few cells that a tile
+// of theirs leaves most of its warp idle.  Measured against the tile kernel below
+// (us, from k and from ln k): FP64 100000 cells of 1 x 1 planes 64 -> 6 and 269 ->
+// 12, 50000 2 x 2 planes, 10 links 152 -> 33 and 254 -> 72, 20000 4 x 4 planes 64 ->
+// 49 and 105 -> 106 (8 x 4: 31 and 49, 47 and 107 this way); mixed 1 x 1 planes 41 ->
+// 8 and 59 -> 14 (2 x 2: 28 and 37, 27 and 57 this way).
+template <typename Real, bool LOG>
+__global__ void k_trans_cells(GridGeom g, Geo geo, const double* __restrict__ perm, Real* Tx, Real* Ty, Real* Tz,
+                              Real* Tpp, Real* Tmp, Real* kperm, PermTag tag) {
+    if (still_held(tag)) return;
+    const long long nx = g.nx, nxy = nx * g.ny, N = nxy * g.nz;
+    for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < N;
+         c += (long long)gridDim.x * blockDim.x) {
+        const int k = (int)(c / nxy), j = (int)((c - k * nxy) / nx), i = (int)(c - k * nxy - j * nx);
+        const bool xp = i + 1 < g.nx, yp = j + 1 < g.ny;
+        const double kc = perm_at<LOG>(perm, c);
+        // an absent link's neighbour is the cell itself, so every address is in range
+        auto T = [&](bool there, long long d, double a) {
+            return there ? (Real)two_point(kc, perm_at<LOG>(perm, there ? d : c), a) : Real(0);
+        };
+        Tx[c] = T(xp, c + 1, geo.ax);
+        Ty[c] = T(yp, c + nx, geo.ay);
+        Tz[c] = T(k + 1 < g.nz, c + nxy, geo.az);
+        if (g.diag) {
+            Tpp[c] = T(xp && yp, c + nx + 1, geo.ad);
+            Tmp[c] = T(i > 0 && yp, c + nx - 1, geo.ad);
+        }
+        if (kperm) kperm[c] = (Real)kc;
+    }
+}
+
 constexpr int kTileThreads = 256;  // cells of a tile at most (one thread each)
-constexpr int kTransRun = 4;      // planes a block walks (its next plane's own cells are already there)
+constexpr int kTransRun = 4;      // planes a block walks at most (its next plane's own cells are already there)
 
 // Owned transmissibilities of a tile of TX x TY cells over kTransRun planes,
 // and (kperm != null) the adjoint's copy of k.  Per plane the tile's
@@ -211,21 +255,15 @@ constexpr int kTransRun = 4;      // planes a block walks (its next plane's own 
 // column on each side) sit
 // in shared memory: 1.2 per cell instead of six.  Measured from ln k with the
 // copy of k (a kernel of its own before): mixed 128^3 704 -> 42 us, FP64
-// 97 x 83 x 50 144 -> 87 us (bound by the FP64 pipe: 1.5 exponentials and five
+// 97 x 83 x 50 144 -> 68 us (bound by the FP64 pipe: 1.5 exponentials and five
 // quotients per cell).  Runs of 8 planes instead of 4 measured the same on the
-// mixed path and 7 % slower in FP64 (fewer blocks).
+// mixed path and 7 % slower in FP64 (fewer blocks); shorter ones where the tiles are
+// too few for the multiprocessors (20^3, FP64, 10 links, from ln k 24.7 -> 10.4 us).
 template <typename Real, bool LOG>
 __global__ void __launch_bounds__(kTileThreads)
-    k_trans(GridGeom g, Geo geo, int TX, int TY, const double* __restrict__ perm, Real* Tx, Real* Ty, Real* Tz,
+    k_trans(GridGeom g, Geo geo, int TX, int TY, int run, const double* __restrict__ perm, Real* Tx, Real* Ty, Real* Tz,
             Real* Tpp, Real* Tmp, Real* kperm, PermTag tag) {
-    // (the count only grows, so a block that reads it after block 0 has counted
-    // this launch decides as the others)
-    if (tag.held && *tag.held == *static_cast<const volatile unsigned long long*>(tag.set)) return;
-    if (tag.set && blockIdx.x == 0 && threadIdx.x == 0) {
-        const unsigned long long n = *tag.set + 1;
-        *tag.set = n;
-        if (tag.take) *tag.take = n;
-    }
+    if (still_held(tag)) return;
     using R = Tile<Real>;
     using RT = typename R::type;
     // (TX + 2)(TY + 1) with TX TY <= 256 and TX <= 128 is at most 3 * 257
@@ -255,7 +293,7 @@ __global__ void __launch_bounds__(kTileThreads)
     };
     const long long own = cell(tx + 1, ty);
     const int sp = ty * PX + tx + 1;
-    const int k0 = (int)(bt / by) * kTransRun, k1 = min(k0 + kTransRun, g.nz);
+    const int k0 = (int)(bt / by) * run, k1 = min(k0 + run, g.nz);
     double vc = R::template pre<LOG>(perm[own + nxy * k0]);  // own k (FP64 path) or the stored value
     RT rc = R::template of<LOG>(vc, eighth);
     for (int k = k0; k < k1; ++k) {
@@ -397,12 +435,25 @@ static cudaError_t launch_trans_t(const GridGeom& g, const SetupPhys& s, const d
     // one block index for tiles and z-runs: any grid shape of fewer than 2^31 cells fits
     int TX = 1, TY = 1;
     tile_shape(g.nx, g.ny, kTileThreads, TX, TY);
-    const long long nb = (long long)((g.nx + TX - 1) / TX) * ((g.ny + TY - 1) / TY) *
-                         ((g.nz + kTransRun - 1) / kTransRun);
+    const long long tiles = (long long)((g.nx + TX - 1) / TX) * ((g.ny + TY - 1) / TY);
+    // shorter runs where the long ones would leave multiprocessors idle
+    int dev = 0, sms = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e != cudaSuccess) return e;
+    int run = kTransRun;
+    while (run > 1 && tiles * ((g.nz + run - 1) / run) < 2LL * sms) run /= 2;
+    const long long nb = tiles * ((g.nz + run - 1) / run);
     const int block = (TX * TY + 31) / 32 * 32;
     const Geo q = make_geo(s);
-    if (log_k) k_trans<Real, true><<<(unsigned)nb, block, 0, st>>>(g, q, TX, TY, perm, Tx, Ty, Tz, Tpp, Tmp, kperm, tag);
-    else k_trans<Real, false><<<(unsigned)nb, block, 0, st>>>(g, q, TX, TY, perm, Tx, Ty, Tz, Tpp, Tmp, kperm, tag);
+    if (TX * TY <= (sizeof(Real) == 8 ? 16 : 2)) {
+        const unsigned cells = blocks_for((long long)g.nx * g.ny * g.nz);
+        if (log_k) k_trans_cells<Real, true><<<cells, kThreads, 0, st>>>(g, q, perm, Tx, Ty, Tz, Tpp, Tmp, kperm, tag);
+        else k_trans_cells<Real, false><<<cells, kThreads, 0, st>>>(g, q, perm, Tx, Ty, Tz, Tpp, Tmp, kperm, tag);
+        return cudaGetLastError();
+    }
+    if (log_k) k_trans<Real, true><<<(unsigned)nb, block, 0, st>>>(g, q, TX, TY, run, perm, Tx, Ty, Tz, Tpp, Tmp, kperm, tag);
+    else k_trans<Real, false><<<(unsigned)nb, block, 0, st>>>(g, q, TX, TY, run, perm, Tx, Ty, Tz, Tpp, Tmp, kperm, tag);
     return cudaGetLastError();
 }
 
