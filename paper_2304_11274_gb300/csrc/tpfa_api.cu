@@ -1531,6 +1531,8 @@ struct tpfa_ensemble_s {
     long long total = 0;
     int JY = 64, W = 4;  // rows per march of the early models (build_table)
     int blocks = 0, slots = 0;
+    std::vector<int> order, runs;  // models by size, their runs of rows (plan_runs), for plan_JY, plan_W and plan_slots
+    int plan_JY = 0, plan_W = 0, plan_slots = 0;
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t exec = nullptr;
     // parameters the graph's kernel node was built with
@@ -1550,6 +1552,26 @@ struct tpfa_ensemble_s {
 
 namespace {
 
+// Estimated time of tiles, in groups of equal ones, claimed in order by `slots`
+// blocks: in row steps, 0.3 of the last block's end and 0.7 of the mean (a
+// multiprocessor with fewer blocks left runs them faster).  Fitted to 19
+// ensembles of 1 to 20 models under two choices of rows each, within 4 % rms.
+double tiles_time(const std::vector<std::pair<long long, double>>& groups, int slots) {
+    std::map<double, long long> free{{0.0, slots}};  // blocks by the time they are free
+    double work = 0.0;
+    for (const auto& g : groups) {
+        work += (double)g.first * g.second;
+        for (long long n = g.first; n > 0;) {
+            const auto first = free.begin();
+            const long long take = std::min(n, first->second);
+            free[first->first + g.second] += take;
+            n -= take;
+            if ((first->second -= take) == 0) free.erase(first);
+        }
+    }
+    return 0.3 * free.rbegin()->first + 0.7 * work / slots;
+}
+
 // Rows per march, model by model.  A march's start costs about 2.5 rows, so the
 // early models' marches are long (the tiling's rows, 64 until it is tuned); the
 // last models, once fewer tiles are left than blocks, get short ones, so that the
@@ -1559,7 +1581,61 @@ namespace {
 // 1632 -> 1563, 64 models 4337 -> 4136, 8 models 750 -> 722, 3 models with 6 links
 // 165 -> 146; 64 rows without the short tail 1590, 4156, 761, 177; the tail from
 // 1.5 or 2 tiles per block, or with 16 or 32 rows, up to 3 % slower.
+// A single model, or an ensemble of up to two short tiles per block, ends too soon
+// for that to even out (up to 13 % slower than 32 rows everywhere), so its two
+// lengths are those of the least estimated time: one model of 223 x 129 x 126, 10
+// links 186 -> 154 us, of 300 x 300 x 60 265 -> 220, two of 189 x 82 x 70 and 97 x 187 x 33
+// 116 -> 89.  Larger ensembles do worse by the estimate (up to 8 %).
 constexpr int kTailRows = 24, kFewestRows = 6;
+const int kEnsembleRows[] = {64, 48, 40, 32, 28, 24, 20, 16, 12, 8, 6};
+
+void plan_runs(tpfa_ensemble e) {
+    if (e->plan_JY == e->JY && e->plan_W == e->W && e->plan_slots == e->slots) return;
+    e->plan_JY = e->JY, e->plan_W = e->W, e->plan_slots = e->slots;
+    // tiles are numbered (and claimed) largest model first, so the launch
+    // ends on the small models' tiles
+    e->order.resize(e->M);
+    for (int m = 0; m < e->M; ++m) e->order[m] = m;
+    std::stable_sort(e->order.begin(), e->order.end(), [&](int a, int b) { return e->grids[a]->N > e->grids[b]->N; });
+    const auto columns = [&](const tpfa_grid* h) { return (long long)((h->nx + 31) / 32) * ((h->nz + e->W - 1) / e->W); };
+    long long longs = 0, shorts = 0;  // tiles of e->JY rows, and of short ones
+    for (const tpfa_grid* h : e->grids) {
+        longs += columns(h) * ((h->ny + e->JY - 1) / e->JY);
+        shorts += columns(h) * ((h->ny + kTailRows - 1) / kTailRows);
+    }
+    // runs of each model, in order, with at most `early` and later `tail` rows each
+    const auto runs_of = [&](int early, int tail, std::vector<int>& runs) {
+        long long left = longs;
+        runs.clear();
+        for (int m : e->order) {
+            const tpfa_grid* h = e->grids[m];
+            const int most = left < e->slots ? tail : early;
+            left -= columns(h) * ((h->ny + e->JY - 1) / e->JY);
+            runs.push_back((h->ny + most - 1) / most);
+        }
+    };
+    int tail = std::min(e->JY, kTailRows);
+    if (shorts < e->slots) tail = std::min(tail, std::max(kFewestRows, (int)(kTailRows * shorts / e->slots)));
+    runs_of(e->JY, tail, e->runs);
+    if (e->M > 1 && shorts > 2LL * e->slots) return;
+    const auto time_of = [&](const std::vector<int>& runs) {
+        std::vector<std::pair<long long, double>> groups;
+        for (int t = 0; t < e->M; ++t) {
+            const tpfa_grid* h = e->grids[e->order[t]];
+            groups.push_back({columns(h) * runs[t], (h->ny + runs[t] - 1) / runs[t] + 2.5});
+        }
+        return tiles_time(groups, e->slots);
+    };
+    double best = 0.97 * time_of(e->runs);
+    std::vector<int> runs;
+    for (int early : kEnsembleRows)
+        for (int late : kEnsembleRows) {
+            if (early > e->JY || late > early) continue;
+            runs_of(early, late, runs);
+            const double t = time_of(runs);
+            if (t < best) best = t, e->runs = runs;
+        }
+}
 
 int build_table(tpfa_ensemble e, std::vector<BatchModel>& tab) {
     int bps = 0, sms = 0;
@@ -1567,23 +1643,11 @@ int build_table(tpfa_ensemble e, std::vector<BatchModel>& tab) {
     if (ce != cudaSuccess) return cuda_fail(ce, "ensemble kernel occupancy");
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, e->device);
     e->slots = sms * (bps > 0 ? bps : 1);
-    const auto columns = [&](const tpfa_grid* h) { return (long long)((h->nx + 31) / 32) * ((h->nz + e->W - 1) / e->W); };
-    long long left = 0, shorts = 0;  // tiles of e->JY rows in this model and those after it; of short ones in all
-    for (const tpfa_grid* h : e->grids) {
-        left += columns(h) * ((h->ny + e->JY - 1) / e->JY);
-        shorts += columns(h) * ((h->ny + kTailRows - 1) / kTailRows);
-    }
-    int tail = std::min(e->JY, kTailRows);
-    if (shorts < e->slots) tail = std::min(tail, std::max(kFewestRows, (int)(kTailRows * shorts / e->slots)));
+    plan_runs(e);
     tab.resize(e->M);
     long long first = 0;
-    // tiles are numbered (and claimed) largest model first, so the launch
-    // ends on the small models' tiles
-    std::vector<int> order(e->M);
-    for (int m = 0; m < e->M; ++m) order[m] = m;
-    std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return e->grids[a]->N > e->grids[b]->N; });
     for (int t = 0; t < e->M; ++t) {
-        const int m = order[t];
+        const int m = e->order[t];
         tpfa_grid* h = e->grids[m];
         if (!h->has_state) return fail(TPFA_ERR_NO_STATE, "ensemble model %d has no state (tpfa_set_state)", m);
         if (!e->vals[m]) return fail(TPFA_ERR_INVALID_ARG, "ensemble model %d has no outputs (tpfa_ensemble_set_outputs)", m);
@@ -1593,10 +1657,8 @@ int build_table(tpfa_ensemble e, std::vector<BatchModel>& tab) {
         bm.q = h->qf;
         bm.f = fields_of<float>(h);
         bm.o = AsmOut<float>{e->R[m], e->vals[m], e->diag64[m], h->status};
-        const int most = left < e->slots ? tail : e->JY;
-        left -= columns(h) * ((h->ny + e->JY - 1) / e->JY);
         bm.tx = (h->nx + 31) / 32;
-        bm.ty = (h->ny + most - 1) / most;
+        bm.ty = e->runs[t];
         bm.rows = (h->ny + bm.ty - 1) / bm.ty;
         bm.tz = (h->nz + e->W - 1) / e->W;
         bm.crk = h->crk ? 1 : 0;
