@@ -112,13 +112,16 @@ __device__ __noinline__ double lnk_by_division(const Args64& a, int i, int j, in
     double sum = 0.0;
 #pragma unroll 1
     for (int s = 0; s < NSLOT; ++s) {
-        if (s == SLOT_SELF || !((mask >> s) & 1u)) continue;
-        const int x = s == 0 || s == 10 ? 0 : (s - 1) % 3 - 1, y = s == 0 || s == 10 ? 0 : (s - 1) / 3 - 1;
-        const int d = s == 0 ? c - nxy : s == 10 ? c + nxy : c + x + nx * y;
-        const double* T = s == 0 || s == 10 ? a.f.Tz : x == 0 ? a.f.Ty : y == 0 ? a.f.Tx : x == y ? a.f.Tpp : a.f.Tmp;
+        // a link that does not exist is formed from the cell itself: every address is in range
+        const bool there = s != SLOT_SELF && ((mask >> s) & 1u);
+        const bool z = s == 0 || s == 10;
+        const int x = z ? 0 : (s - 1) % 3 - 1, y = z ? 0 : (s - 1) / 3 - 1;
+        const int d = !there ? c : s == 0 ? c - nxy : s == 10 ? c + nxy : c + x + nx * y;
+        const double* T = z ? a.f.Tz : x == 0 ? a.f.Ty : y == 0 ? a.f.Tx : x == y ? a.f.Tpp : a.f.Tmp;
         const double F = link(a.q, T[s < SLOT_SELF ? d : c], me, make_cell(a.q, a.f.p[d], a.f.z[d])).F;
         const double kk = __dadd_rn(a.kperm[c], a.kperm[d]);
-        sum = __fma_rn(__dmul_rn(F, __dsub_rn(a.dir[c], a.dir[d])), kk > 0.0 ? a.kperm[d] / kk : 0.0, sum);
+        const double ratio = kk > 0.0 ? a.kperm[d] / kk : 0.0;
+        if (there) sum = __fma_rn(__dmul_rn(F, __dsub_rn(a.dir[c], a.dir[d])), ratio, sum);
     }
     return sum;
 }
