@@ -247,15 +247,19 @@ int tpfa_vjp_kernel(tpfa_handle h, tpfa_kernel kern, const double* v_dev, double
  * matrix with w up to FP64 rounding.  w_dev, Jw_dev: N doubles (device,
  * caller-owned, w read and Jw written asynchronously on `stream`).
  * R_dev: N doubles or NULL; when given it receives R of Eq. vk with exactly
- * the bits tpfa_assemble_residual writes.  Links in the path's precision,
- * the w-weighted sums in FP64.  Device-side errors (non-finite output, an
- * out-of-range checked access) are reported by tpfa_sync_status.
+ * the bits tpfa_assemble_residual writes.  TPFA_FP64: links and sums in FP64.
+ * TPFA_MIXED: FP32 links and w narrowed to FP32, the w-weighted terms summed
+ * with compensation in FP32, the sums combined in FP64.  Device-side errors (a
+ * non-finite output; an out-of-range access, in the mixed path's naive kernel and
+ * in rows computed again after a march, whose loads are checked) are reported by
+ * tpfa_sync_status.
  */
 int tpfa_jvp(tpfa_handle h, const double* w_dev, double* Jw_dev, double* R_dev, void* stream);
 
-/* As tpfa_jvp with an explicit kernel variant (TPFA_MIXED: the tiled march
- * and the naive gather give identical bits; TPFA_FP64 has one kernel and
- * ignores the choice). */
+/* As tpfa_jvp with an explicit kernel variant (TPFA_MIXED: AUTO is a march with
+ * two cells per lane on large grids, else the one-cell march TILED; they and the
+ * naive gather give identical bits; TILED2 and TILED_TMA are refused; TPFA_FP64
+ * has one kernel and ignores the choice). */
 int tpfa_jvp_kernel(tpfa_handle h, tpfa_kernel kern, const double* w_dev, double* Jw_dev, double* R_dev,
                     void* stream);
 

@@ -282,12 +282,13 @@ bool tma_ready(tpfa_grid* h) {
 // pair-aligned).  A ragged last segment leaves lanes idle
 // and the x-boundary segments cost their lanes masked sums, so narrow grids
 // whose width is not a multiple of 64 do better one cell per lane: measured
-// (G cells/s, one-cell vs two-cell, best rows per march each) 26.4 vs 28.3 at
-// 128^3, 26.9 vs 24.7 at 160 x 160 x 80, 28.5 vs 29.2 at 192 x 160 x 80, 22.3
-// vs 18.1 at 224 x 96 x 48, 11.5 vs 10.4 at 64^3, 33.4 vs 36.3 at
-// 256 x 256 x 128, 38.0 vs 46.4 at 512 x 512 x 256.  (The TMA march gives the
-// same bits but measured 8 % slower than the one-cell march at
-// 512 x 512 x 256: its row waits stall where the per-lane prefetch does not.)
+// (G cells/s, 10 links, one-cell vs two-cell, the launches' own rows) 26.3 vs 34.1
+// at 128^3, 27.2 vs 24.1 at 160 x 160 x 80, 29.7 vs 30.8 at 192 x 160 x 80, 22.8 vs
+// 20.8 at 224 x 96 x 48, 27.4 vs 26.1 at 200 x 200 x 100, 12.5 vs 12.8 at 64^3, 33.0
+// vs 39.3 at 256 x 256 x 128, 37.9 vs 48.4 at 512 x 512 x 256; 6 links 34.4 vs 32.7 at
+// 160 x 160 x 80, 30.0 vs 31.3 at 224 x 96 x 48, 50.7 vs 62.2 at 512 x 512 x 256.  (The
+// TMA march gives the same bits but measured 8 % slower than the one-cell march
+// at 512 x 512 x 256: its row waits stall where the per-lane prefetch does not.)
 AsmKernel auto_kernel(tpfa_grid* h) {
     const int nx = h->nx;
     return nx >= 256 || nx == 128 || nx == 192 ? AsmKernel::XMarch : AsmKernel::YMarch;

@@ -231,7 +231,10 @@ inline PhysD make_phys_d(double rho_ref, double p_ref, double c_f, double mu, do
 // the value, so their sum over x^5 is taken in FP32 (its error stays below
 // 2^-59 of the value) and five FP64 operations remain of eight; below 2^-10 the
 // terms of expm1 from x^4 / 4! on are less than 2^-34 of it, and four of ten
-// remain.  The range tests read the high word (integer pipe).
+// remain.  Against 80-bit values over 4 million arguments of each binade the errors
+// are those of the all-FP64 series to four digits in the mean (exp 5.05e-17, expm1
+// 6.80e-17 rms) and below 2^-8 in the largest (1.11e-16, 2.20e-16); at 2^-6 exp's
+// largest is 1.116e-16.  The range tests read the high word (integer pipe).
 __device__ __forceinline__ uint32_t abs_hi(double x) { return (uint32_t)__double2hiint(x) & 0x7fffffffu; }
 __device__ __forceinline__ double exp_fp64(double x) {
     const uint32_t a = abs_hi(x);
@@ -547,7 +550,10 @@ __device__ __forceinline__ AccD accumulation(const PhysD& q, double p, double pn
 // Sums of an FP64 row over its links, in slot order.  The diagonal needs no
 // term of its own per link: dF/dp_a + dF/dp_b = c_f F - u (lam_a + lam_b), so
 //   sum dF/dp_a = -sum dF/dp_b + (c_f sum F - sum u rs),
-// the bracket and dA small beside the first sum, which they join last.
+// the bracket and dA small beside the first sum, which they join last.  (Against
+// 80-bit values the diagonals are 2 % closer than with a term per link while
+// c_f |dPhi| <= 0.1; the bracket cancels by 1 + c_f |dPhi|, so they are 7 % further
+// off at c_f |dPhi| = 1, a density that changes e-fold from cell to cell.)
 struct RowAccD {
     double F = 0.0, d = 0.0, grav = 0.0;  // sum F, -sum dF/dp_b, -sum u rs
     template <bool JAC, bool FLAT = false>

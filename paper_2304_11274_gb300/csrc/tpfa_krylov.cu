@@ -19,8 +19,8 @@
 // host only polls the record.  Once `done` is set every kernel returns at
 // entry, so the host may enqueue several iterations between polls.
 //
-// What bounds it: HBM (about 0.55 GB per iteration at 128^3 of which the L2
-// keeps some) and the FP64 pipe (two operations per clock and multiprocessor;
+// What bounds it: HBM (0.83 GB per iteration at 128^3 of which the L2 keeps
+// some) and the FP64 pipe (two operations per clock and multiprocessor;
 // 24 per cell and iteration).  So the matrix is copied once per solve from its
 // CSR order to slot-major groups of 32 cells (the CSR rows of 11 values would
 // cost eleven times the L1 wavefronts in each of the two products of every

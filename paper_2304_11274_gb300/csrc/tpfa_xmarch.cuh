@@ -19,9 +19,10 @@
 //     a neighbour lane's).  Negating every input that changes sign between
 //     the two ends of a link negates every output, so these reused values
 //     are exact, except at an exact tie dPhi == 0 (each end then takes the
-//     other cell as upstream): a warp that meets a zero flux on a reused
-//     link records the row and recomputes it after the march with the naive
-//     kernel's row code, so every row is bit-identical to that kernel's;
+//     other cell as upstream): a warp that meets one on a reused link records
+//     the row and recomputes it after the march with the naive kernel's row
+//     code, so every row is bit-identical to that kernel's (the zero derivatives
+//     of a link with T = 0 may have the other sign);
 //   * densities: the two cells of row j+1 and the halo cell (lanes 0 and
 //     31) as they enter the window, the four vertical neighbours per row;
 //   * every pair-valued input of row j+2 (p, depth, the five owned T, p^n,
